@@ -609,9 +609,9 @@ __device__ __forceinline__ void neighbour(int nbi, int px, int py, int& qx, int&
 // PEEL: A is a layer of a depth-peeled composite (A.peel set); a separate
 // instantiation keeps the opaque path's registers to its own needs
 template <bool PEEL = false>
-__device__ __forceinline__ void aa_loss_block(const ShadeArgs& A, int b, int px, int py, double* red) {
+__device__ __forceinline__ void aa_loss_block(const ShadeArgs& A, int b, int px, int py, float* red) {
     bool inside = px < A.W && py < A.H;
-    double lsum = 0.0;
+    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
     if (inside) {
         size_t pix = ((size_t)b * A.H + py) * A.W + px;
         unsigned long long kp = __ldg(A.keys + (pix));
@@ -636,9 +636,15 @@ __device__ __forceinline__ void aa_loss_block(const ShadeArgs& A, int b, int px,
         }
         if (A.ref) {
             const float* y = A.ref + pix * 3;
-            float g0, g1, g2;
-            lsum = (double)loss_term(A.loss_kind, out.x, y[0], &g0) + (double)loss_term(A.loss_kind, out.y, y[1], &g1) +
-                   (double)loss_term(A.loss_kind, out.z, y[2], &g2);
+            float y0 = y[0], y1 = y[1], y2 = y[2];
+            float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+            // black on black (the background, half of most views) has no loss and no gradient in
+            // any of the losses: the warps that see nothing else skip their tone maps
+            if (out.x != 0.f || out.y != 0.f || out.z != 0.f || y0 != 0.f || y1 != 0.f || y2 != 0.f) {
+                l0 = loss_term(A.loss_kind, out.x, y0, &g0);
+                l1 = loss_term(A.loss_kind, out.y, y1, &g1);
+                l2 = loss_term(A.loss_kind, out.z, y2, &g2);
+            }
             A.gprime[pix] = make_float4(g0 * A.loss_scale, g1 * A.loss_scale, g2 * A.loss_scale, __uint_as_float(amask));
         }
         if (A.out_img) {
@@ -648,15 +654,10 @@ __device__ __forceinline__ void aa_loss_block(const ShadeArgs& A, int b, int px,
         }
         if (A.acol) A.acol[pix] = make_float4(out.x, out.y, out.z, __uint_as_float(amask));
     }
-    lsum = warp_sum_d(lsum);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
-    __syncthreads();
-    if (threadIdx.x == 0 && A.loss_acc) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(A.loss_acc, s * (double)A.loss_scale);
-    }
+    if (!A.loss_acc) return;
+    __syncthreads();  // red is free: a persistent block's last item has been summed
+    double s = block_sum3(l0, l1, l2, red);
+    if (threadIdx.x == 0 && s != 0.0) atomicAdd(A.loss_acc, s * (double)A.loss_scale);
 }
 
 // ------------------------------------------------------------------ backward

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(ADMS_FWD_THREADS, ADMS_FWD_BLOCKS) k_shade_fwd
 
 template <bool PEEL>
 __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(ShadeArgs A) {
-    __shared__ double red[ADMS_AA_THREADS / 32];
+    __shared__ alignas(8) float red[ADMS_AA_THREADS / 16];
     int px, py;
     band_pixel<ADMS_AA_THREADS>(A.W, px, py);
     aa_loss_block<PEEL>(A, blockIdx.y, px, py, red);
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) k_refine_batch(const ShadeBatch P) {
 template <int KIND>
 __global__ void __launch_bounds__(256, KIND == 2 ? 3 : (KIND == 1 ? 8 : 5))
     k_pixels_batch(const ShadeBatch P, const WorkItem* __restrict__ items, int n, int tw, int job0) {
-    __shared__ double red[8];
+    __shared__ alignas(8) float red[16];
     __shared__ float rows[KIND == 2 ? 8 * 32 * ADMS_VROW : 1];
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         WorkItem w = items[it];
@@ -244,10 +244,10 @@ __global__ void __launch_bounds__(256, KIND == 2 ? 3 : (KIND == 1 ? 8 : 5))
 
 // ------------------------------------------------------------------ supersample resolve
 __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
-    __shared__ double red[8];
+    __shared__ alignas(8) float red[16];
     long long n = (long long)r.B * r.H * r.W;
     long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double lsum = 0.0;
+    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
     if (pix < n) {
         int b = (int)(pix / ((long long)r.H * r.W));
         int rem = (int)(pix - (long long)b * r.H * r.W);
@@ -267,8 +267,9 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
         if (r.ref) {
             const float* y = r.ref + pix * 3;
             float g0, g1, g2;
-            lsum = (double)loss_term(r.loss_kind, c.x, y[0], &g0) + (double)loss_term(r.loss_kind, c.y, y[1], &g1) +
-                   (double)loss_term(r.loss_kind, c.z, y[2], &g2);
+            l0 = loss_term(r.loss_kind, c.x, y[0], &g0);
+            l1 = loss_term(r.loss_kind, c.y, y[1], &g1);
+            l2 = loss_term(r.loss_kind, c.z, y[2], &g2);
             float k = r.loss_scale * inv;  // each sample carries 1 / s^2 of its pixel
             for (int sy = 0; sy < r.S; ++sy)
                 for (int sx = 0; sx < r.S; ++sx) {
@@ -277,14 +278,9 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
                 }
         }
     }
-    lsum = warp_sum_d(lsum);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
-    __syncthreads();
-    if (threadIdx.x == 0 && r.loss_acc) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += red[w];
-        atomicAdd(r.loss_acc, s * (double)r.loss_scale);
-    }
+    if (!r.loss_acc) return;
+    double s = block_sum3(l0, l1, l2, red);
+    if (threadIdx.x == 0 && s != 0.0) atomicAdd(r.loss_acc, s * (double)r.loss_scale);
 }
 
 cudaError_t resolve_loss(const ResolveArgs& r, cudaStream_t st) {
