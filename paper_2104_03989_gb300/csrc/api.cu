@@ -1877,8 +1877,11 @@ adms_status adms_job_invalidate(adms_ctx* ctx, adms_job job) {
     if (!j) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
     if (adms_status fs = flush_job(ctx, *j)) return fs;  // its deferred texture step first
     TexState* maps[3] = {&j->kd, &j->orm, &j->nrm};
+    TexDev chains[3];
+    int n_chains = 0;
     for (int m = 0; m < 3; ++m)
-        if (!maps[m]->per_level) CK(TIMED(ST_MIP, mip_build(maps[m]->dev(), ctx->stream)));
+        if (!maps[m]->per_level) chains[n_chains++] = maps[m]->dev();
+    CK(TIMED(ST_MIP, mip_build(chains, n_chains, ctx->stream)));
     j->frame_valid = false;
     j->lap_valid = false;
     return ADMS_OK;

@@ -301,7 +301,9 @@ cudaError_t adam_texture(const TexDev& t, float4* m, float4* v, int clamp_kind, 
 // hold the whole chain); no mip adjoint, no rebuild
 cudaError_t adam_texture_levels(const TexDev& t, float4* m, float4* v, int clamp_kind, const JobState* js,
                                 cudaStream_t st);
-// rebuild levels 1.. of a mip chain from level 0 (2x2 box average)
+// rebuild levels 1.. of mip chains from level 0 (2x2 box average); n <= 3 textures that tile
+// take two launches together, others one per level
+cudaError_t mip_build(const TexDev* ts, int n, cudaStream_t st);
 cudaError_t mip_build(const TexDev& t, cudaStream_t st);
 // Adam on a texture, then the rebuild of its mip chain (textures that do not tile)
 cudaError_t adam_texture_and_mips(const TexDev& t, float4* m, float4* v, int clamp_kind, const JobState* js,

@@ -208,17 +208,6 @@ __global__ void k_adam_tex(TexDev t, float4* __restrict__ m, float4* __restrict_
     t.grad[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// weight of a level-k texel's gradient in each of its level-0 texels (product of
-// the 2x2 / 2x1 box-filter factors down the chain)
-__device__ __forceinline__ float level_weight(const TexDev& t, int k) {
-    float w = 1.f;
-    for (int j = 1; j <= k; ++j) {
-        int wp = max(t.w0 >> (j - 1), 1), hp = max(t.h0 >> (j - 1), 1);
-        w *= 1.f / (float)((wp > 1 ? 2 : 1) * (hp > 1 ? 2 : 1));
-    }
-    return w;
-}
-
 // Adam on the 32x32 texel tiles of level 0 of every texture of a launch (up to
 // ADMS_ADAM_TEX textures of any jobs, tile ranges from tile0), each followed by
 // levels 1..5 of its tile from the updated texels (2x2 box average, same order of
@@ -527,29 +516,48 @@ __global__ void __launch_bounds__(ADMS_ADAM_THREADS, ADMS_ADAM_MIN_BLOCKS)
     if (tid == 0) bulk_wait0();
 }
 
-// Levels 6.. of every texture of a streamed-Adam launch, one block per texture,
-// from the level 5 that the tiles wrote (2x2 box average, same order as
-// k_mip_level); their gradients, read by every tile above, are cleared here.
-__global__ void k_adam_mip_top(const __grid_constant__ TexAdamBatch P) {
-    const TexAdam& A = P.a[blockIdx.x];
-    if (A.js->status) return;
-    const TexDev& t = A.t;
+// Levels 6.. of a texture that tiles, by one block, from the level 5 that its tiles wrote
+// (2x2 box average, same order as k_mip_level). Once a level fits the block (one texel per
+// thread) the next is formed from shared memory: a level costs two block barriers instead of
+// a round trip to L2.
+// CLEAR: the levels' gradients, read by every tile of the optimizer step, are cleared.
+#define ADMS_MIP_TOP_THREADS 1024
+template <bool CLEAR>
+__device__ __forceinline__ void mip_top(const TexDev& t, float4* s) {
     float4* tex = const_cast<float4*>(t.tex);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool held = false;  // s holds level lv - 1
     for (int lv = 6; lv < t.levels; ++lv) {
         int ws = max(t.w0 >> (lv - 1), 1), hs = max(t.h0 >> (lv - 1), 1);
         int wd = max(t.w0 >> lv, 1), hd = max(t.h0 >> lv, 1);
         int sx = ws > 1 ? 2 : 1, sy = hs > 1 ? 2 : 1;
+        float inv = 1.f / (float)(sx * sy);
+        const float4* src = held ? s : tex + t.off[lv - 1];
+        bool fits = wd * hd <= ADMS_MIP_TOP_THREADS;
+        float4 v = zero;
         for (int i = threadIdx.x; i < wd * hd; i += blockDim.x) {
             int x = i % wd, y = i / wd;
             float4 acc = zero;
             for (int dy = 0; dy < sy; ++dy)
-                for (int dx = 0; dx < sx; ++dx) acc = f4madd(acc, 1.f, tex[t.off[lv - 1] + (y * sy + dy) * ws + (x * sx + dx)]);
-            tex[t.off[lv] + i] = f4scale(acc, 1.f / (float)(sx * sy));
-            t.grad[t.off[lv] + i] = zero;
+                for (int dx = 0; dx < sx; ++dx) acc = f4madd(acc, 1.f, src[(y * sy + dy) * ws + (x * sx + dx)]);
+            v = f4scale(acc, inv);
+            tex[t.off[lv] + i] = v;
+            if (CLEAR) t.grad[t.off[lv] + i] = zero;
         }
-        __syncthreads();
+        __syncthreads();  // level lv - 1 has been read
+        if (fits) {
+            if ((int)threadIdx.x < wd * hd) s[threadIdx.x] = v;
+            __syncthreads();
+        }
+        held = fits;
     }
+}
+
+__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_adam_mip_top(const __grid_constant__ TexAdamBatch P) {
+    __shared__ float4 s[ADMS_MIP_TOP_THREADS];
+    const TexAdam& A = P.a[blockIdx.x];
+    if (A.js->status) return;
+    mip_top<true>(A.t, s);
 }
 
 bool adam_tiled(const TexDev& t) { return t.levels > 5 && (t.w0 % 32) == 0 && (t.h0 % 32) == 0; }
@@ -608,7 +616,7 @@ cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uin
         P.extra_tx = extra_tx;
         int blocks = std::min(tiles, std::max(1, sms * ADMS_ADAM_GRID_PCT / 100));
         k_adam_tex_stream<<<blocks, ADMS_ADAM_THREADS, sizeof(AdamSmem), st>>>(P, tiles);
-        k_adam_mip_top<<<P.n, 256, 0, st>>>(P);
+        k_adam_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P);
         count_launches(2);
         cudaError_t e = cudaGetLastError();
         if (e) return e;
@@ -623,23 +631,54 @@ cudaError_t adam_texture_and_mips(const TexDev& t, float4* m, float4* v, int cla
     return mip_build(t, st);
 }
 
-// level-0 gradient including the adjoint of the mip chain, written to out (no update)
-__global__ void k_fold_mips(TexDev t, float4* __restrict__ out) {
-    int n = t.w0 * t.h0;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int x = i % t.w0, y = i / t.w0;
-    float4 g = t.grad[i];
-    for (int k = 1; k < t.levels; ++k) {
-        int wk = max(t.w0 >> k, 1);
-        g = f4madd(g, level_weight(t, k), t.grad[t.off[k] + (y >> k) * wk + (x >> k)]);
+// level-0 gradient including the adjoint of the mip chain, written to out (no update):
+// g0 + w1 g1 + w2 g2 + ... per texel, finest level first. Bound by HBM (16 B in and out per
+// texel and the coarser third of it again); a thread takes a 2x2 quad of level-0 texels, which
+// share every coarser texel: the levels' loads are issued together and reused four times, and
+// the levels' weights come as parameters. One texel per thread with its index divisions and
+// the weights rebuilt per level took 58.7 us for a 1024^2 map and 257 us for a 2048^2 one.
+struct FoldWeights {
+    float w[ADMS_MAX_LEVELS];
+};
+__global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ TexDev t, const FoldWeights fw,
+                                                   float4* __restrict__ out) {
+    int x = 2 * (blockIdx.x * 32 + (threadIdx.x & 31)), y = 2 * (blockIdx.y * 8 + (threadIdx.x >> 5));
+    if (x >= t.w0 || y >= t.h0) return;
+    bool bx = x + 1 < t.w0, by = y + 1 < t.h0;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    size_t i = (size_t)y * t.w0 + x;
+    float4 g[4] = {t.grad[i], bx ? t.grad[i + 1] : zero, by ? t.grad[i + t.w0] : zero,
+                   bx && by ? t.grad[i + t.w0 + 1] : zero};
+#pragma unroll
+    for (int k0 = 1; k0 < ADMS_MAX_LEVELS; k0 += 5) {  // five levels' loads in flight at a time
+        if (k0 >= t.levels) break;
+        float4 c[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            int k = k0 + j;
+            c[j] = k < t.levels ? t.grad[t.off[k] + (y >> k) * max(t.w0 >> k, 1) + (x >> k)] : zero;
+        }
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+            if (k0 + j < t.levels) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) g[q] = f4madd(g[q], fw.w[k0 + j], c[j]);
+            }
     }
-    out[i] = g;
+    out[i] = g[0];
+    if (bx) out[i + 1] = g[1];
+    if (by) out[i + t.w0] = g[2];
+    if (bx && by) out[i + t.w0 + 1] = g[3];
 }
 
 cudaError_t fold_mip_gradient(const TexDev& t, float4* out, cudaStream_t st) {
-    int n = t.w0 * t.h0;
-    k_fold_mips<<<(n + 255) / 256, 256, 0, st>>>(t, out);
+    FoldWeights fw;
+    fw.w[0] = 1.f;
+    // the share of a level-k texel in each of its level-0 texels: the 2x2 / 2x1 box factors down the chain
+    for (int k = 1; k < ADMS_MAX_LEVELS; ++k)
+        fw.w[k] = fw.w[k - 1] / (float)(((t.w0 >> (k - 1)) > 1 ? 2 : 1) * ((t.h0 >> (k - 1)) > 1 ? 2 : 1));
+    dim3 grid((t.w0 + 63) / 64, (t.h0 + 15) / 16);
+    k_fold_mips<<<grid, 256, 0, st>>>(t, fw, out);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -669,15 +708,83 @@ __global__ void k_mip_level(float4* __restrict__ tex, int src_off, int ws, int h
     tex[dst_off + i] = f4scale(acc, 1.f / (float)(sx * sy));
 }
 
-cudaError_t mip_build(const TexDev& t, cudaStream_t st) {
-    for (int k = 1; k < t.levels; ++k) {
-        int ws = max(t.w0 >> (k - 1), 1), hs = max(t.h0 >> (k - 1), 1);
-        int wd = max(t.w0 >> k, 1), hd = max(t.h0 >> k, 1);
-        k_mip_level<<<(wd * hd + 255) / 256, 256, 0, st>>>(const_cast<float4*>(t.tex), t.off[k - 1], ws, hs, t.off[k],
-                                                          wd, hd);
+// Levels 1..5 of up to three textures that tile, a 32x32 tile of level 0 per block, the
+// thread's quad and the shuffles as in k_adam_tex_stream: level 0 is read once and nothing of
+// the chain is read back (HBM bound: 16 B per level-0 texel in, 5.3 out). A launch per level
+// took 36 us for a 1024^2 map (ten launches), three maps 110 us.
+#define ADMS_MIP_TEX 3
+struct MipBatch {
+    TexDev t[ADMS_MIP_TEX];
+    int tile0[ADMS_MIP_TEX];
+    int n;
+};
+__global__ void __launch_bounds__(256) k_mip_tiles(const __grid_constant__ MipBatch P) {
+    __shared__ float4 s3[16];
+    int e = 0, tile = blockIdx.x;
+    while (e + 1 < P.n && P.tile0[e + 1] <= tile) ++e;
+    const TexDev& t = P.t[e];
+    float4* tex = const_cast<float4*>(t.tex);
+    tile -= P.tile0[e];
+    int bx = tile % (t.w0 >> 5), by = tile / (t.w0 >> 5);
+    int tid = threadIdx.x, lane = tid & 31;
+    int cx = even_bits(tid), cy = even_bits(tid >> 1), x = 2 * cx, y = 2 * cy;
+    const float4* src = t.tex + (size_t)(32 * by + y) * t.w0 + 32 * bx + x;
+    float4 l = quad_mean(src[0], src[1], src[t.w0], src[t.w0 + 1]);
+    tex[t.off[1] + ((by << 4) + cy) * (t.w0 >> 1) + (bx << 4) + cx] = l;
+#pragma unroll
+    for (int lv = 2; lv <= 3; ++lv) {
+        int d = lv == 2 ? 1 : 4;  // lane distance of the x neighbour
+        float4 a1 = shfl_down4(l, d), a2 = shfl_down4(l, 2 * d), a3 = shfl_down4(l, 3 * d);
+        l = quad_mean(l, a1, a2, a3);
+        int n = 32 >> lv;
+        if ((lane & (4 * d - 1)) == 0) tex[t.off[lv] + (by * n + (y >> lv)) * (t.w0 >> lv) + bx * n + (x >> lv)] = l;
+    }
+    if ((lane & 15) == 0) s3[tid >> 4] = l;
+    __syncthreads();
+    if (tid >= 4) return;
+    float4 l4 = quad_mean(s3[4 * tid], s3[4 * tid + 1], s3[4 * tid + 2], s3[4 * tid + 3]);
+    tex[t.off[4] + (by * 2 + (tid >> 1)) * (t.w0 >> 4) + bx * 2 + (tid & 1)] = l4;
+    float4 a1 = shfl_down4(l4, 1, 0xfu), a2 = shfl_down4(l4, 2, 0xfu), a3 = shfl_down4(l4, 3, 0xfu);
+    if (tid == 0) tex[t.off[5] + by * (t.w0 >> 5) + bx] = quad_mean(l4, a1, a2, a3);
+}
+
+__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_mip_top(const __grid_constant__ MipBatch P) {
+    __shared__ float4 s[ADMS_MIP_TOP_THREADS];
+    mip_top<false>(P.t[blockIdx.x], s);
+}
+
+cudaError_t mip_build(const TexDev* ts, int n, cudaStream_t st) {
+    MipBatch P;
+    P.n = 0;
+    int tiles = 0, top = 0;
+    for (int j = 0; j < n; ++j) {
+        const TexDev& t = ts[j];
+        if (adam_tiled(t) && P.n < ADMS_MIP_TEX) {
+            P.t[P.n] = t;
+            P.tile0[P.n++] = tiles;
+            tiles += (t.w0 >> 5) * (t.h0 >> 5);
+            top = max(top, t.levels - 6);
+            continue;
+        }
+        for (int k = 1; k < t.levels; ++k) {
+            int ws = max(t.w0 >> (k - 1), 1), hs = max(t.h0 >> (k - 1), 1);
+            int wd = max(t.w0 >> k, 1), hd = max(t.h0 >> k, 1);
+            k_mip_level<<<(wd * hd + 255) / 256, 256, 0, st>>>(const_cast<float4*>(t.tex), t.off[k - 1], ws, hs,
+                                                              t.off[k], wd, hd);
+            count_launches(1);
+        }
+    }
+    if (tiles) {
+        k_mip_tiles<<<tiles, 256, 0, st>>>(P);
         count_launches(1);
+        if (top > 0) {
+            k_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P);
+            count_launches(1);
+        }
     }
     return cudaGetLastError();
 }
+
+cudaError_t mip_build(const TexDev& t, cudaStream_t st) { return mip_build(&t, 1, st); }
 
 }  // namespace adms
