@@ -375,7 +375,7 @@ adms_status ensure_scratch(adms_ctx* ctx, Job& j, int B, int H, int W) {
         AL(j.rs.clip, (size_t)B * j.V);
         AL(j.rs.scr, (size_t)B * j.V);
         AL(j.rs.vs, (size_t)B * j.V);
-        AL(j.rs.rec, (size_t)B * j.F);
+        AL(j.rs.rec, (size_t)B * j.F * ADMS_REC_PAD);
         AL(j.rs.bin, (size_t)B * j.F);
         AL(j.rs.asign, (size_t)B * j.F);
         AL(j.rs.silmask, (size_t)B * j.F);
@@ -1040,6 +1040,7 @@ adms_status batch_upload(adms_ctx* ctx, const std::vector<Job*>& js, float* cons
         memset(&r, 0, sizeof(r));
         r.rec = j.rs.rec;
         r.bin = j.rs.bin;
+        r.records = (long long)j.B * j.F;
         r.F = j.F;
         r.W = j.W;
         r.H = j.H;

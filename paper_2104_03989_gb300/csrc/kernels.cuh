@@ -23,22 +23,23 @@ struct VtxS {
     int ok;
 };
 
-// triangle setup record of one view: oriented edge functions s E_k = ea Sx + eb Sy + ec
-// (s = sign of the snapped area), fill-rule thresholds, depth plane, pixel bbox
-struct TriRec {
-    long long ec[3];
-    int ea[3], eb[3];
-    int thr[3];
-    float fA, z0, dz1, dz2;
-    int sg, id, valid;
-    short bx0, bx1, by0, by1;
-};
-
 // pixel bounding box of a binned triangle of one view; empty (bx0 > bx1) for
 // triangles rasterized by the small-triangle pass or not drawn at all
 struct TriBin {
     short bx0, bx1, by0, by1;
 };
+
+// record of a binned triangle of one view: snapped corners, depth plane, pixel box (the edge
+// functions follow from the corners, in int32 where `near` is set). 48 bytes; a record buffer
+// holds ADMS_REC_PAD records per triangle and view, the second half taking tile-list entries.
+struct alignas(16) TriRec {
+    int X[3], Y[3];
+    float z0, dz1, dz2;
+    int near;
+    TriBin box;
+};
+static_assert(sizeof(TriRec) == 48, "two records per triangle and view fill the 96-byte allocation");
+#define ADMS_REC_PAD 2
 
 // triangles with at most this many samples in their pixel bbox skip binning (default)
 #define ADMS_SMALL_PX 16
@@ -60,7 +61,7 @@ struct RasterScratch {
     float4* clip;       // [B][V]
     float4* scr;        // [B][V] screen position as (x_hi, x_lo, y_hi, y_lo) float pairs
     VtxS* vs;           // [B][V]
-    TriRec* rec;        // [B][F] (written for binned triangles only)
+    TriRec* rec;        // [ADMS_REC_PAD][B][F] (the first written for binned triangles only)
     TriBin* bin;        // [B][F]
     int8_t* asign;      // [B][F]
     uint8_t* silmask;   // [B][F] bit e: edge e is a silhouette edge in that view
@@ -172,6 +173,7 @@ int batched_occupancy(int kind);
 struct RasterJob {
     const TriRec* rec;
     const TriBin* bin;
+    long long records;  // views x triangles
     int F, W, H, tiles_x, tiles_y;
     const int* tile_off;
     const int* tile_count;
@@ -179,9 +181,6 @@ struct RasterJob {
     long long capacity;
     unsigned long long* keys;
     unsigned long long* overflow_ctr;
-};
-struct RasterBatch {
-    RasterJob a[ADMS_BATCH_JOBS];
 };
 // persistent launch of the 16x16-tile raster over (job, view, tile) items; arguments
 // and item ranges as for pixels_batched

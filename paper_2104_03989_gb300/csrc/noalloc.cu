@@ -40,7 +40,7 @@ bool plan_layout(size_t B, size_t V, size_t F, size_t ntiles, Layout& L) {
     if (__builtin_mul_overflow(B, V, &BV) || __builtin_mul_overflow(B, F, &BF) || __builtin_mul_overflow(F, (size_t)3, &F3))
         return false;
     bool ok = add_part(off, BV, sizeof(float4), L.clip) && add_part(off, BV, sizeof(float4), L.scr) &&
-              add_part(off, BV, sizeof(VtxS), L.vs) && add_part(off, BF, sizeof(TriRec), L.rec) &&
+              add_part(off, BV, sizeof(VtxS), L.vs) && add_part(off, BF, ADMS_REC_PAD * sizeof(TriRec), L.rec) &&
               add_part(off, BF, sizeof(TriBin), L.bin) && add_part(off, BF, 1, L.asign) &&
               add_part(off, BF, 1, L.silmask) && add_part(off, F3, sizeof(int), L.adj) &&
               add_part(off, ntiles, sizeof(int), L.tile_count) && add_part(off, ntiles, sizeof(int), L.tile_off) &&

@@ -12,13 +12,6 @@
 
 namespace adms {
 
-__device__ __forceinline__ long long floor_div_ll(long long a, long long b) {  // b > 0
-    long long q = a / b;
-    if ((a % b != 0) && (a < 0)) q -= 1;
-    return q;
-}
-__device__ __forceinline__ long long ceil_div_ll(long long a, long long b) { return -floor_div_ll(-a, b); }
-
 // m0 x + m1 y + m2 z + m3 (float inputs, double-float result)
 __device__ __forceinline__ DF df_row(const float* m, float x, float y, float z) {
     DF p0 = df_two_prod(m[0], x), p1 = df_two_prod(m[1], y), p2 = df_two_prod(m[2], z);
@@ -119,205 +112,210 @@ __global__ void __launch_bounds__(256) k_list_alloc(const int* __restrict__ coun
     if (i < n) off[i] = (int)min((long long)base + x - c, (long long)0x7fffffff);
 }
 
-// ---------------------------------------------------------------- coverage test
-// coverage + depth key of one triangle at a sample with oriented edge values
-// e0, e1, e2 there, or ADMS_EMPTY_KEY
-__device__ __forceinline__ unsigned long long key_of(const TriRec& r, long long e0, long long e1, long long e2) {
-    if (e0 < r.thr[0] || e1 < r.thr[1] || e2 < r.thr[2]) return ADMS_EMPTY_KEY;
-    // back to the triangle's own vertex order: E_20 = s e1, E_01 = s e2
-    long long E20 = r.sg > 0 ? e1 : -e1;
-    long long E01 = r.sg > 0 ? e2 : -e2;
-    float b1 = __fdiv_rn(__ll2float_rn(E20), r.fA);
-    float b2 = __fdiv_rn(__ll2float_rn(E01), r.fA);
-    float d = __fadd_rn(__fadd_rn(r.z0, __fmul_rn(b1, r.dz1)), __fmul_rn(b2, r.dz2));
-    if (!(d >= 0.f && d <= 1.f)) return ADMS_EMPTY_KEY;
-    if (d == 0.f) d = 0.f;
-    return ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)r.id;
-}
+// ---------------------------------------------------------------- edge functions
+// Oriented edge functions of a triangle (s E_k, s the sign of its snapped area; edge 0 =
+// 1->2, 1 = 2->0, 2 = 0->1): a_k = -s dy, b_k = s dx, value a_k (Sx - Xa) + b_k (Sy - Ya),
+// covered where value >= thr_k for every k.
+//
+// "Near" triangles (snapped extents of at most ADMS_NEAR = 96 pixels a side) are evaluated
+// in int32: at any sample within 16 pixels of the box |Sx - Xa|, |Sy - Ya| <= 112 * 256 =
+// 28672 and |a|, |b| <= 24576, so |value| <= 2 * 28672 * 24576 < 2^31, and the area fits
+// too; the values, and with them the keys, are those of the int64 form. It saves the wide
+// multiplies, and above all the int64 -> float conversions of the depth: those run on the
+// FP64 pipe at 1/64 rate (the tile raster held it 50% busy). Larger triangles keep int64.
+#define ADMS_NEAR (96 * 256)
 
-// coverage + depth key of one triangle at one sample, or ADMS_EMPTY_KEY
-__device__ __forceinline__ unsigned long long tri_key(const TriRec& r, int Sx, int Sy) {
-    return key_of(r, (long long)r.ea[0] * Sx + (long long)r.eb[0] * Sy + r.ec[0],
-                  (long long)r.ea[1] * Sx + (long long)r.eb[1] * Sy + r.ec[1],
-                  (long long)r.ea[2] * Sx + (long long)r.eb[2] * Sy + r.ec[2]);
-}
-
-// keeps the minimum in best
-__device__ __forceinline__ void test_tri(const TriRec& r, int Sx, int Sy, unsigned long long& best) {
-    unsigned long long key = tri_key(r, Sx, Sy);
-    if (key < best) best = key;
-}
-
-// keeps the KB smallest keys in kb[0] < kb[1] < ... (a per-sample k-buffer; the
-// keys of one sample are distinct, each triangle giving at most one): the
-// fragment sinks into place and the largest falls out
-template <int KB>
-__device__ __forceinline__ void test_tri_kbuf(const TriRec& r, int Sx, int Sy, unsigned long long (&kb)[KB]) {
-    unsigned long long key = tri_key(r, Sx, Sy);
-    if (key >= kb[KB - 1]) return;
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-        unsigned long long lo = key < kb[i] ? key : kb[i];
-        key = key < kb[i] ? kb[i] : key;
-        kb[i] = lo;
+template <typename T>
+struct Edges {
+    T a[3], b[3], area;  // area: absolute
+    int x[3], y[3];      // a point of each edge
+    int thr[3];
+    int sg;
+    __device__ __forceinline__ T at(int k, int Sx, int Sy) const {
+        return a[k] * (T)(Sx - x[k]) + b[k] * (T)(Sy - y[k]);
     }
-}
+};
 
-// z-buffer update of the direct raster, for dense clouds of small triangles (a
-// foliage canopy puts ~160 fragments on each sample). The stored key is read
-// first: zlo is a lower bound on every key the triangle can produce, so when it
-// is above the stored key the sample is skipped without its coverage test; else
-// the key goes in only if it is below the stored one. The stored key only ever
-// decreases, so a read that lags behind other threads' updates is never below the
-// current minimum and can only let an unneeded test or atomicMin through.
-// Without the filter (zfilter = 0: closed surfaces, about two fragments per sample)
-// the read would only add a dependent round trip: the key goes straight to atomicMin.
-__device__ __forceinline__ void zmin_test(unsigned long long* a, const TriRec& r, int Sx, int Sy,
-                                          unsigned long long zlo, int zfilter) {
-    if (!zfilter) {
-        unsigned long long key = tri_key(r, Sx, Sy);
-        if (key != ADMS_EMPTY_KEY) atomicMin(a, key);
-        return;
-    }
-    unsigned long long cur = __ldcg(a);
-    if (zlo > cur) return;
-    unsigned long long key = tri_key(r, Sx, Sy);
-    if (key != ADMS_EMPTY_KEY && key < cur) atomicMin(a, key);
-}
-
-// A lower bound on the keys of a triangle with vertex depths z0, z1, z2: its
-// interpolated depth d = z0 + b1 (z1 - z0) + b2 (z2 - z0) (b1, b2 >= 0, b1 + b2 <= 1,
-// each operation rounded once) is at least min z less a few units of rounding of
-// the largest |z| (1e-6 x max(1, |z|) covers them with room), and a key needs d >= 0.
-__device__ __forceinline__ unsigned long long key_floor(float z0, float z1, float z2) {
-    float zmn = fminf(z0, fminf(z1, z2));
-    float zmx = fmaxf(fabsf(z0), fmaxf(fabsf(z1), fabsf(z2)));
-    float lo = fmaxf(zmn - 1e-6f * fmaxf(1.f, zmx), 0.f);
-    return (unsigned long long)__float_as_uint(lo) << 32;
-}
-
-// the setup record of lane src, for every lane of the warp
-__device__ __forceinline__ TriRec shfl_rec(const TriRec& r, int src) {
-    const unsigned full = 0xffffffffu;
-    TriRec o;
+template <typename T>
+__device__ __forceinline__ Edges<T> make_edges(const int X[3], const int Y[3]) {
+    Edges<T> e;
+    T A = (T)(X[1] - X[0]) * (T)(Y[2] - Y[0]) - (T)(Y[1] - Y[0]) * (T)(X[2] - X[0]);
+    e.sg = A > 0 ? 1 : -1;
+    e.area = A > 0 ? A : -A;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        o.ec[k] = __shfl_sync(full, r.ec[k], src);
-        o.ea[k] = __shfl_sync(full, r.ea[k], src);
-        o.eb[k] = __shfl_sync(full, r.eb[k], src);
-        o.thr[k] = __shfl_sync(full, r.thr[k], src);
+        int i = (k + 1) % 3, j = (k + 2) % 3;
+        int odx = e.sg * (X[j] - X[i]), ody = e.sg * (Y[j] - Y[i]);
+        e.a[k] = (T)-ody;
+        e.b[k] = (T)odx;
+        e.x[k] = X[i];
+        e.y[k] = Y[i];
+        e.thr[k] = ((ody < 0) || (ody == 0 && odx > 0)) ? 0 : 1;
     }
-    o.fA = __shfl_sync(full, r.fA, src);
-    o.z0 = __shfl_sync(full, r.z0, src);
-    o.dz1 = __shfl_sync(full, r.dz1, src);
-    o.dz2 = __shfl_sync(full, r.dz2, src);
-    o.sg = __shfl_sync(full, r.sg, src);
-    o.id = __shfl_sync(full, r.id, src);
-    o.valid = 1;
-    int bx = __shfl_sync(full, ((int)(unsigned short)r.bx0) | ((int)r.bx1 << 16), src);
-    int by = __shfl_sync(full, ((int)(unsigned short)r.by0) | ((int)r.by1 << 16), src);
-    o.bx0 = (short)(bx & 0xffff);
-    o.bx1 = (short)(bx >> 16);
-    o.by0 = (short)(by & 0xffff);
-    o.by1 = (short)(by >> 16);
-    return o;
+    return e;
+}
+
+// Calls f(tile index) for the 16x16 tiles of the box in which the triangle may cover a
+// sample: a tile goes when some edge function is below its threshold at the tile's sample
+// where it is largest. The setup's counts and the fill's entries come from the same loop.
+// (A box of one tile is taken as it is.) On billboards of ~60 pixels a third of the boxes'
+// tiles go; their entries, records and tests with them.
+template <typename T, typename F>
+__device__ __forceinline__ void for_tiles(const Edges<T>& e, const TriBin& tb, int tiles_x, F&& f) {
+    int tx0 = tb.bx0 / ADMS_TILE, tx1 = tb.bx1 / ADMS_TILE, ty0 = tb.by0 / ADMS_TILE, ty1 = tb.by1 / ADMS_TILE;
+    if (tx0 == tx1 && ty0 == ty1) {
+        f(ty0 * tiles_x + tx0);
+        return;
+    }
+    constexpr int step = 256 * ADMS_TILE, last = 256 * (ADMS_TILE - 1);
+    T row[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        row[k] = e.at(k, step * tx0 + 128 + (e.a[k] > 0 ? last : 0), step * ty0 + 128 + (e.b[k] > 0 ? last : 0)) -
+                 e.thr[k];
+    for (int ty = ty0; ty <= ty1; ++ty) {
+        T v[3] = {row[0], row[1], row[2]};
+        for (int tx = tx0; tx <= tx1; ++tx) {
+            if ((v[0] | v[1] | v[2]) >= 0) f(ty * tiles_x + tx);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] += e.a[k] * (T)step;
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) row[k] += e.b[k] * (T)step;
+    }
+}
+
+// depth key from the oriented edge values e1, e2 (b1 = s E_20 / A = e1 / |A|: the sign
+// cancels exactly), or ADMS_EMPTY_KEY outside the depth range
+__device__ __forceinline__ unsigned long long depth_key(float e1, float e2, float area, float z0, float dz1, float dz2,
+                                                        int id) {
+    float b1 = __fdiv_rn(e1, area), b2 = __fdiv_rn(e2, area);
+    float d = __fadd_rn(__fadd_rn(z0, __fmul_rn(b1, dz1)), __fmul_rn(b2, dz2));
+    if (!(d >= 0.f && d <= 1.f)) return ADMS_EMPTY_KEY;
+    if (d == 0.f) d = 0.f;
+    return ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)id;
+}
+
+// A lower bound on the keys of a triangle with vertex depths z0, z1, z2 (its high word):
+// the interpolated depth d = z0 + b1 (z1 - z0) + b2 (z2 - z0) (b1, b2 >= 0, b1 + b2 <= 1,
+// each operation rounded once) is at least min z less a few units of rounding of
+// the largest |z| (1e-6 x max(1, |z|) covers them with room), and a key needs d >= 0.
+__device__ __forceinline__ unsigned key_floor(float z0, float z1, float z2) {
+    float zmn = fminf(z0, fminf(z1, z2));
+    float zmx = fmaxf(fabsf(z0), fmaxf(fabsf(z1), fabsf(z2)));
+    return __float_as_uint(fmaxf(zmn - 1e-6f * fmaxf(1.f, zmx), 0.f));
+}
+
+// A near triangle as the per-sample loops read it, at sample offsets (x, y) from an origin:
+//   p = (E0', A0, B0, C), q = (E1', A1, B1, -), r = (|area|, z0, dz1, dz2)
+// E_k' = value - thr_k at the origin, A, B the steps per pixel, C the sum of the three E'
+// (the edge functions add up to |area| everywhere): covered where e0, e1 and C - e0 - e1
+// are all non-negative.
+__device__ __forceinline__ int near_third(int c, int e0, int e1) {  // c - e0 - e1 (fits; the partial sum may wrap)
+    return (int)((unsigned)c - (unsigned)e0 - (unsigned)e1);
+}
+__device__ __forceinline__ void near_pack(const Edges<int>& e, int Sx, int Sy, int4& p, int4& q) {
+    int E0 = e.at(0, Sx, Sy) - e.thr[0], E1 = e.at(1, Sx, Sy) - e.thr[1];
+    p = make_int4(E0, 256 * e.a[0], 256 * e.b[0], e.area - e.thr[0] - e.thr[1] - e.thr[2]);
+    q = make_int4(E1, 256 * e.a[1], 256 * e.b[1], 0);
 }
 
 // ---------------------------------------------------------------- setup, small triangles, tile counts
-// One thread per (view, triangle). Triangles whose pixel bounding box holds at
-// most small_px samples are rasterized here directly, one 64-bit atomicMin per
-// covered sample (the minimum does not depend on the order); larger ones get a
-// setup record and are counted into the tiles they overlap. Direct triangles of
-// up to ADMS_SMALL_PX samples loop over their box in their own thread; larger
-// direct ones are rasterized by the whole warp, one triangle after another with
-// the lanes striding over its box (a thread per triangle left three quarters of
-// the lanes idle on a canopy of leaves of 20-300 samples each).
-// COOP: the instantiation with the warp-wide path and the filtered z-buffer
-// updates, launched when small_px exceeds ADMS_SMALL_PX; the other keeps the
-// common case (small_px = ADMS_SMALL_PX) to its own registers.
-template <bool COOP>
-__global__ void __launch_bounds__(256, COOP ? 3 : 1) k_setup(const int* __restrict__ tri, int F, const VtxS* __restrict__ vs, int V, int B, int W, int H,
-                        int tiles_x, int tiles_y, TriRec* __restrict__ rec, TriBin* __restrict__ bin,
-                        int8_t* __restrict__ asign, int* __restrict__ tile_count, unsigned long long* __restrict__ keys,
-                        int small_px, int zfilter) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    bool coop = false;  // this lane's triangle goes to the warp-wide direct raster
-    TriRec r;
-    int b = 0;
-    unsigned long long zlo = 0ull;  // lower bound on the triangle's keys (COOP)
+// One thread per (view, triangle). Near triangles whose pixel box holds at most small_px
+// samples are rasterized here directly, one 64-bit atomicMin per covered sample (the
+// minimum does not depend on the order); the others get a record and are counted into the
+// tiles they may touch.
+//
+// The direct raster flattens the warp's triangles: their packed edge functions go to shared
+// memory, their sample counts are scanned, and the lanes take the boxes' samples 32 at a
+// time whatever triangle they belong to. The triangle of a lane is the number of boxes that
+// begin at or before its sample, from one mask of the beginnings in the batch (__reduce_or
+// and a population count), so that every lane of every batch but the last has a sample. (A
+// thread per triangle of up to 16 samples and the whole warp per larger one left half of
+// the lanes idle and moved 30 words a triangle by shuffles: 3.41 -> 1.63 ms for 600k leaf
+// quads under 8 views of 512x512, 0.40 -> 0.20 ms for 62k displaced triangles under 16 of
+// 1024x1024, 12.4 -> 6.6 us for 5000 triangles under 8 of 512x512.)
+//
+// ZF (in.zfilter): the stored key is read before the depth is computed, for dense clouds (a
+// foliage canopy puts ~160 fragments on each sample). zlo is a lower bound on every key of
+// the triangle, so above the stored key the sample is done; else the key goes in only if it
+// is below the stored one. The stored key only ever decreases, so a read that lags behind
+// other threads' updates can only let an unneeded atomicMin through. Without it (closed
+// surfaces, about two fragments per sample) the read would only add a round trip.
+#ifndef ADMS_SETUP_BLOCKS
+#define ADMS_SETUP_BLOCKS 4
+#endif
+struct DirectTri {  // 80 bytes: 16-byte reads of consecutive slots touch distinct banks
+    int4 p, q, r;
+    int id;
+    unsigned inv_w;      // 2^32 / box width, rounded up (0: width 1)
+    long long origin;    // key index of the box's first sample
+    int start, width;    // first of its samples among the warp's
+    unsigned zlo;
+    int thr;             // thr_1 | thr_2 << 1
+};
+template <bool ZF>
+__global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
+    k_setup(const int* __restrict__ tri, int F, const VtxS* __restrict__ vs, int V, int B, int W, int H, int tiles_x,
+            int tiles_y, TriRec* __restrict__ rec, TriBin* __restrict__ bin, int8_t* __restrict__ asign,
+            int* __restrict__ tile_count, unsigned long long* __restrict__ keys, int small_px) {
+    __shared__ DirectTri slots[8][32];
+    const unsigned full = 0xffffffffu;
+    int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    int npx = 0;  // samples of this lane's direct triangle
+    DirectTri t;
     if (i < B * F) {
-        b = i / F;
-        int f = i - b * F;
-        int i0 = tri[3 * f], i1 = tri[3 * f + 1], i2 = tri[3 * f + 2];
+        int b = i / F, f = i - b * F;
         const VtxS* vb = vs + (size_t)b * V;
-        VtxS a0 = vb[i0], a1 = vb[i1], a2 = vb[i2];
+        VtxS v0 = vb[tri[3 * f]], v1 = vb[tri[3 * f + 1]], v2 = vb[tri[3 * f + 2]];
         TriBin tb;
-        tb.bx0 = 1;
-        tb.bx1 = 0;
-        tb.by0 = 1;
-        tb.by1 = 0;
+        tb.bx0 = tb.by0 = 1;
+        tb.bx1 = tb.by1 = 0;
         int8_t sgn = 0;
-        if (a0.ok && a1.ok && a2.ok) {
-            long long X0 = a0.X, Y0 = a0.Y, X1 = a1.X, Y1 = a1.Y, X2 = a2.X, Y2 = a2.Y;
-            long long A = (X1 - X0) * (Y2 - Y0) - (Y1 - Y0) * (X2 - X0);
+        if (v0.ok && v1.ok && v2.ok) {
+            int X[3] = {v0.X, v1.X, v2.X}, Y[3] = {v0.Y, v1.Y, v2.Y};
+            long long A = (long long)(X[1] - X[0]) * (Y[2] - Y[0]) - (long long)(Y[1] - Y[0]) * (X[2] - X[0]);
             if (A != 0) {
-                int sg = A > 0 ? 1 : -1;
-                sgn = (int8_t)sg;
-                long long minX = min(X0, min(X1, X2)), maxX = max(X0, max(X1, X2));
-                long long minY = min(Y0, min(Y1, Y2)), maxY = max(Y0, max(Y1, Y2));
-                long long ilo = max(ceil_div_ll(minX - 128, 256), 0ll), ihi = min(floor_div_ll(maxX - 128, 256), (long long)W - 1);
-                long long jlo = max(ceil_div_ll(minY - 128, 256), 0ll), jhi = min(floor_div_ll(maxY - 128, 256), (long long)H - 1);
+                sgn = A > 0 ? 1 : -1;
+                int minX = min(X[0], min(X[1], X[2])), maxX = max(X[0], max(X[1], X[2]));
+                int minY = min(Y[0], min(Y[1], Y[2])), maxY = max(Y[0], max(Y[1], Y[2]));
+                // samples at 256 i + 128; |X| <= 2^27, so the shifts round down without overflow
+                int ilo = max((minX + 127) >> 8, 0), ihi = min((maxX - 128) >> 8, W - 1);
+                int jlo = max((minY + 127) >> 8, 0), jhi = min((maxY - 128) >> 8, H - 1);
                 if (ilo <= ihi && jlo <= jhi) {
-                    // original-order edges: e0 = 1->2, e1 = 2->0, e2 = 0->1
-                    long long px[3] = {X0, X1, X2}, py[3] = {Y0, Y1, Y2};
-    #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        int a = (k + 1) % 3, c = (k + 2) % 3;
-                        long long dx = px[c] - px[a], dy = py[c] - py[a];
-                        // oriented value s E = a Sx + b Sy + cst with s = sign(A)
-                        r.ea[k] = (int)(-sg * dy);
-                        r.eb[k] = (int)(sg * dx);
-                        r.ec[k] = sg * (dy * px[a] - dx * py[a]);
-                        long long odx = sg * dx, ody = sg * dy;
-                        r.thr[k] = ((ody < 0) || (ody == 0 && odx > 0)) ? 0 : 1;
-                    }
-                    r.fA = __ll2float_rn(A);
-                    r.sg = sg;
-                    r.z0 = a0.z;
-                    r.dz1 = __fsub_rn(a1.z, a0.z);
-                    r.dz2 = __fsub_rn(a2.z, a0.z);
-                    r.id = f;
-                    r.valid = 1;
-                    r.bx0 = (short)ilo;
-                    r.bx1 = (short)ihi;
-                    r.by0 = (short)jlo;
-                    r.by1 = (short)jhi;
-                    long long npx = (ihi - ilo + 1) * (jhi - jlo + 1);
-                    if (COOP) zlo = key_floor(a0.z, a1.z, a2.z);
-                    if (COOP && npx <= small_px && npx > ADMS_SMALL_PX) {
-                        coop = true;
-                    } else if (npx <= small_px) {
-                        unsigned long long* kb = keys + (size_t)b * H * W;
-                        for (int y = (int)jlo; y <= (int)jhi; ++y)
-                            for (int x = (int)ilo; x <= (int)ihi; ++x) {
-                                if (COOP) {
-                                    zmin_test(kb + (size_t)y * W + x, r, 256 * x + 128, 256 * y + 128, zlo, zfilter);
-                                } else {
-                                    unsigned long long key = tri_key(r, 256 * x + 128, 256 * y + 128);
-                                    if (key != ADMS_EMPTY_KEY) atomicMin(kb + (size_t)y * W + x, key);
-                                }
-                            }
+                    bool near = maxX - minX <= ADMS_NEAR && maxY - minY <= ADMS_NEAR;
+                    float dz1 = __fsub_rn(v1.z, v0.z), dz2 = __fsub_rn(v2.z, v0.z);
+                    int w = ihi - ilo + 1, n = w * (jhi - jlo + 1);  // at most 2^28
+                    if (near && n <= small_px) {
+                        npx = n;
+                        Edges<int> e = make_edges<int>(X, Y);
+                        near_pack(e, 256 * ilo + 128, 256 * jlo + 128, t.p, t.q);
+                        t.r = make_int4(__float_as_int(__int2float_rn(e.area)), __float_as_int(v0.z),
+                                        __float_as_int(dz1), __float_as_int(dz2));
+                        t.id = f;
+                        t.inv_w = w > 1 ? 0xffffffffu / (unsigned)w + 1u : 0u;
+                        t.origin = ((long long)b * H + jlo) * W + ilo;
+                        t.width = w;
+                        t.zlo = ZF ? key_floor(v0.z, v1.z, v2.z) : 0u;
+                        t.thr = e.thr[1] | (e.thr[2] << 1);
                     } else {
+                        tb.bx0 = (short)ilo;
+                        tb.bx1 = (short)ihi;
+                        tb.by0 = (short)jlo;
+                        tb.by1 = (short)jhi;
+                        TriRec r;
+                        r.X[0] = X[0], r.X[1] = X[1], r.X[2] = X[2];
+                        r.Y[0] = Y[0], r.Y[1] = Y[1], r.Y[2] = Y[2];
+                        r.z0 = v0.z;
+                        r.dz1 = dz1;
+                        r.dz2 = dz2;
+                        r.near = near;
+                        r.box = tb;
                         rec[i] = r;
-                        tb.bx0 = r.bx0;
-                        tb.bx1 = r.bx1;
-                        tb.by0 = r.by0;
-                        tb.by1 = r.by1;
-                        int tx0 = (int)ilo / ADMS_TILE, tx1 = (int)ihi / ADMS_TILE;
-                        int ty0 = (int)jlo / ADMS_TILE, ty1 = (int)jhi / ADMS_TILE;
                         int* tc = tile_count + (size_t)b * tiles_x * tiles_y;
-                        for (int ty = ty0; ty <= ty1; ++ty)
-                            for (int tx = tx0; tx <= tx1; ++tx) atomicAdd(tc + ty * tiles_x + tx, 1);
+                        auto count = [&](int k) { atomicAdd(tc + k, 1); };
+                        if (near) for_tiles(make_edges<int>(X, Y), tb, tiles_x, count);
+                        else for_tiles(make_edges<long long>(X, Y), tb, tiles_x, count);
                     }
                 }
             }
@@ -325,34 +323,66 @@ __global__ void __launch_bounds__(256, COOP ? 3 : 1) k_setup(const int* __restri
         asign[i] = sgn;
         bin[i] = tb;
     }
-    if (!COOP) return;
-    // warp-wide direct raster of the lanes' mid-sized triangles (every lane of the
-    // warp reaches this point: none returned early)
-    unsigned todo = __ballot_sync(0xffffffffu, coop);
-    int lane = threadIdx.x & 31;
-    while (todo) {
-        int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        TriRec t = shfl_rec(r, src);
-        int tb_ = __shfl_sync(0xffffffffu, b, src);
-        unsigned long long tlo = __shfl_sync(0xffffffffu, zlo, src);
-        int bw = t.bx1 - t.bx0 + 1, n = bw * (t.by1 - t.by0 + 1);
-        unsigned long long* kb = keys + (size_t)tb_ * H * W;
-        for (int q = lane; q < n; q += 32) {
-            int y = t.by0 + q / bw, x = t.bx0 + q - (q / bw) * bw;
-            zmin_test(kb + (size_t)y * W + x, t, 256 * x + 128, 256 * y + 128, tlo, zfilter);
+    unsigned direct = __ballot_sync(full, npx > 0);
+    if (!direct) return;
+    int upto = npx;  // inclusive scan of the sample counts
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        int y = __shfl_up_sync(full, upto, o);
+        if (lane >= o) upto += y;
+    }
+    int total = __shfl_sync(full, upto, 31);
+    t.start = upto - npx;
+    DirectTri* ws = slots[threadIdx.x >> 5];
+    if (npx > 0) ws[__popc(direct & ((1u << lane) - 1u))] = t;
+    __syncwarp();
+    int before = 0;  // boxes that begin before the batch
+    for (int base = 0; base < total; base += 32) {
+        int at = t.start - base;
+        unsigned begins = __reduce_or_sync(full, npx > 0 && at >= 0 && at < 32 ? 1u << at : 0u);
+        const DirectTri& d = ws[before + __popc(begins & (full >> (31 - lane))) - 1];
+        before += __popc(begins);
+        if (base + lane >= total) break;
+        int k = base + lane - d.start, w = d.width;
+        int y = w > 1 ? (int)__umulhi((unsigned)k, d.inv_w) : k, x = k - y * w;
+        int4 p = d.p, q = d.q;
+        int e0 = p.x + p.y * x + p.z * y, e1 = q.x + q.y * x + q.z * y, e2 = near_third(p.w, e0, e1);
+        if ((e0 | e1 | e2) < 0) continue;
+        unsigned long long* a = keys + d.origin + (long long)y * W + x;
+        unsigned long long cur = ADMS_EMPTY_KEY;
+        if (ZF) {
+            cur = __ldcg(a);
+            if (d.zlo > (unsigned)(cur >> 32)) continue;
         }
+        int4 r = d.r;
+        unsigned long long key =
+            depth_key(__int2float_rn(e1 + (d.thr & 1)), __int2float_rn(e2 + (d.thr >> 1)), __int_as_float(r.x),
+                      __int_as_float(r.y), __int_as_float(r.z), __int_as_float(r.w), d.id);
+        if (ZF ? key < cur : key != ADMS_EMPTY_KEY) atomicMin(a, key);
     }
 }
 
 // ---------------------------------------------------------------- tile lists
+// The entries of the tile lists: list[0 .. capacity), then the second half of the records'
+// allocation (a record takes 48 of the 96 bytes per triangle and view that its buffer
+// holds), so that a list of 20 entries per triangle fits where 8 did.
+struct TileLists {
+    const int* list;
+    const int* ext;
+    long long capacity, total;
+    __device__ __forceinline__ int get(long long p) const { return p < capacity ? list[p] : ext[p - capacity]; }
+    __device__ __forceinline__ void set(long long p, int v) const {
+        if (p < total) const_cast<int*>(p < capacity ? list + p : ext + (p - capacity))[0] = v;
+    }
+};
+
 // Per (view, triangle), after the scan of the tile counts: the triangle's
 // silhouette-edge mask, then its entries in the tile lists. Bit e of
 // silmask[b][f] is set when edge e of triangle f is a silhouette edge in view b:
 // no neighbour across it, or a neighbour whose snapped area has another sign.
-__global__ void k_bin_fill(const TriBin* __restrict__ bin, int F, int B, int tiles_x, int tiles_y,
-                           const int* __restrict__ tile_off, int* __restrict__ tile_cursor, int* __restrict__ list,
-                           long long capacity, const int* __restrict__ adj, const int8_t* __restrict__ asign,
+__global__ void k_bin_fill(const TriRec* __restrict__ rec, const TriBin* __restrict__ bin, int F, int B, int tiles_x,
+                           int tiles_y, const int* __restrict__ tile_off, int* __restrict__ tile_cursor,
+                           const TileLists lists, const int* __restrict__ adj, const int8_t* __restrict__ asign,
                            uint8_t* __restrict__ silmask) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B * F) return;
@@ -373,167 +403,232 @@ __global__ void k_bin_fill(const TriBin* __restrict__ bin, int F, int B, int til
     TriBin tb = bin[i];
     if (tb.bx0 > tb.bx1) return;
     size_t tbase = (size_t)b * tiles_x * tiles_y;
-    int tx0 = tb.bx0 / ADMS_TILE, tx1 = tb.bx1 / ADMS_TILE, ty0 = tb.by0 / ADMS_TILE, ty1 = tb.by1 / ADMS_TILE;
-    for (int ty = ty0; ty <= ty1; ++ty)
-        for (int tx = tx0; tx <= tx1; ++tx) {
-            size_t t = tbase + ty * tiles_x + tx;
-            long long p = (long long)tile_off[t] + atomicAdd(tile_cursor + t, 1);
-            if (p < capacity) list[p] = f;
-        }
+    TriRec r = rec[i];
+    auto fill = [&](int k) { lists.set((long long)tile_off[tbase + k] + atomicAdd(tile_cursor + tbase + k, 1), f); };
+    if (r.near) for_tiles(make_edges<int>(r.X, r.Y), tb, tiles_x, fill);
+    else for_tiles(make_edges<long long>(r.X, r.Y), tb, tiles_x, fill);
 }
 
 // ---------------------------------------------------------------- tiled raster
-// One block per (view, 16x16 tile), one pixel per thread; the tile's triangle
-// records are staged through shared memory in chunks of 256. Each pixel starts
-// from the key left by the small-triangle pass. A tile whose list did not fit
-// the list buffer scans every binned triangle of its view instead.
-__device__ __forceinline__ void raster_tile_body(const TriRec* __restrict__ rec, const TriBin* __restrict__ bin, int F,
-                                                 int W, int H, int tiles_x, int tiles_y,
-                                                 const int* __restrict__ tile_off, const int* __restrict__ tile_count,
-                                                 const int* __restrict__ list, long long capacity,
-                                                 unsigned long long* __restrict__ keys,
-                                                 unsigned long long* __restrict__ overflow_ctr, int b, int tile,
-                                                 TriRec* sm) {
-    int tx = tile % tiles_x, ty = tile / tiles_x;
-    int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
-    int px = tx * ADMS_TILE + lx, py = ty * ADMS_TILE + ly;
-    int Sx = 256 * px + 128, Sy = 256 * py + 128;
-    bool inside = px < W && py < H;
-    size_t pix = ((size_t)b * H + py) * W + px;
-    size_t t = (size_t)b * tiles_x * tiles_y + tile;
-    long long off = tile_off[t];
-    int cnt = tile_count[t];
-    const TriRec* rb = rec + (size_t)b * F;
-    const TriBin* bb = bin + (size_t)b * F;
-    bool overflow = off + cnt > capacity;
-    int n = overflow ? F : cnt;
-    if (n == 0) return;  // no binned triangle: the small-triangle pass left the final keys
-    unsigned long long best = inside ? keys[pix] : ADMS_EMPTY_KEY;
-    if (overflow && threadIdx.x == 0) atomicAdd(overflow_ctr, 1ull);
-    // Each warp shades a 16 x 2 strip of the tile (rows 2w, 2w + 1): the staged records
-    // whose pixel box meets a warp's rows go to that warp's list, and each warp walks
-    // only its own. The key is a minimum over the same triangles in any order.
-    __shared__ unsigned char wlist[8][256];
-    __shared__ int wcount[8];
-    int warp = threadIdx.x >> 5;
-    int row0 = ty * ADMS_TILE;
+// One block per (view, 16x16 tile), one pixel per thread, a warp per 8x4 pixels. The tile's
+// triangles are staged through shared memory in chunks of 256: a thread takes one record,
+// forms its edge functions at the tile and the mask of the 8x4 blocks that it may cover
+// (box, and for near triangles the edges); the masks become one word per block and staging
+// warp by ballots, and each warp walks the set bits of its block. The minimum does not
+// depend on the order. Issue-bound (66%), with the FP64 pipe half busy on int64 -> float
+// conversions and 17 of 32 lanes active in 16x2 strips, at 69.9 us for 8 views of 512x512 of
+// 5000 triangles before; 47.5 us now (58% issue, 22 lanes, 28.6 M against 50.4 M warp
+// instructions). The k-buffer form on 11k billboards with 8 layers: 6.06 ms (its tile lists
+// had overflowed) -> 0.45 ms.
+//
+// Each pixel starts from the key left by the small-triangle pass. A tile whose list did
+// not fit scans every binned triangle of its view instead.
+struct TileSmem {
+    int4 p[256], q[256], r[256];  // near_pack at the tile's first sample; q.w: flags
+    int4 s[256];                  // large triangles only
+    int id[256];
+    unsigned mask[8][8];  // [8x4 block][staging warp]
+};
+#define ADMS_LARGE 8  // q.w: bits 0-2 thresholds, bit 3 large
+
+// minimum key / the KB smallest keys in kb[0] < kb[1] < ... (the keys of one sample are
+// distinct, each triangle giving at most one): a fragment sinks into place and the largest
+// falls out
+template <int KB>
+struct KeySink {
+    unsigned long long kb[KB];
+    __device__ __forceinline__ void take(unsigned long long key) {
+        if (key >= kb[KB - 1]) return;
+#pragma unroll
+        for (int i = 0; i < KB; ++i) {
+            unsigned long long lo = key < kb[i] ? key : kb[i];
+            key = key < kb[i] ? kb[i] : key;
+            kb[i] = lo;
+        }
+    }
+};
+
+// per-view arrays of one raster launch
+struct TileArgs {
+    const TriRec* rec;
+    const TriBin* bin;
+    int F, W, H, tiles_x, tiles_y;
+    const int* tile_off;
+    const int* tile_count;
+    TileLists lists;
+    unsigned long long* overflow_ctr;
+};
+
+// the pixel of a thread in its tile
+__device__ __forceinline__ int tile_x(int tid) { return ((tid >> 5) & 1) * 8 + (tid & 7); }
+__device__ __forceinline__ int tile_y(int tid) { return (tid >> 6) * 4 + ((tid >> 3) & 3); }
+
+template <int KB>
+__device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int tile, long long off, int cnt,
+                                                 TileSmem& sm, KeySink<KB>& sink) {
+    int tx = tile % A.tiles_x, ty = tile / A.tiles_x;
+    int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int lx = tile_x(tid), ly = tile_y(tid);
+    const TriRec* rb = A.rec + (size_t)b * A.F;
+    const TriBin* bb = A.bin + (size_t)b * A.F;
+    bool overflow = cnt > 0 && off + cnt > A.lists.total;
+    int n = overflow ? A.F : cnt;
+    if (overflow && tid == 0) atomicAdd(A.overflow_ctr, 1ull);
+    int ox = tx * ADMS_TILE, oy = ty * ADMS_TILE;
+    int S0x = 256 * ox + 128, S0y = 256 * oy + 128;
     for (int c0 = 0; c0 < n; c0 += 256) {
         int m = min(256, n - c0);
         __syncthreads();
-        if (threadIdx.x < 8) wcount[threadIdx.x] = 0;
-        if ((int)threadIdx.x < m) {
-            if (overflow) {
-                int id = c0 + threadIdx.x;
-                TriBin tb = bb[id];
-                if (tb.bx0 <= tb.bx1) sm[threadIdx.x] = rb[id];
-                else sm[threadIdx.x].valid = 0;
-            } else {
-                sm[threadIdx.x] = rb[list[off + c0 + threadIdx.x]];
+        unsigned mask = 0;
+        if (tid < m) {
+            int f = overflow ? c0 + tid : A.lists.get(off + c0 + tid);
+            TriBin tb = overflow ? bb[f] : rb[f].box;
+            // the box in the tile's pixels; empty boxes (not binned) and other tiles' fall out
+            int x0 = max(tb.bx0 - ox, 0), x1 = min(tb.bx1 - ox, ADMS_TILE - 1);
+            int y0 = max(tb.by0 - oy, 0), y1 = min(tb.by1 - oy, ADMS_TILE - 1);
+            if (x0 <= x1 && y0 <= y1) {
+                TriRec t = rb[f];
+                unsigned cols = (x0 < 8 ? 1u : 0u) | (x1 >= 8 ? 2u : 0u);
+                for (int w = y0 >> 2; w <= (y1 >> 2); ++w) mask |= cols << (2 * w);
+                float area;
+                if (t.near) {
+                    Edges<int> e = make_edges<int>(t.X, t.Y);
+                    int4 p, q;
+                    near_pack(e, S0x, S0y, p, q);
+                    q.w = e.thr[0] | (e.thr[1] << 1) | (e.thr[2] << 2);
+                    area = __int2float_rn(e.area);
+                    sm.p[tid] = p;
+                    sm.q[tid] = q;
+                    // the blocks where every edge function reaches its threshold at its largest sample
+                    int ax[3] = {p.y, q.y, -(p.y + q.y)}, by[3] = {p.z, q.z, -(p.z + q.z)};
+                    int v[3] = {p.x, q.x, near_third(p.w, p.x, q.x)};
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) v[k] += max(7 * ax[k], 0) + max(3 * by[k], 0);
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) {
+                        int x = 8 * (w & 1), y = 4 * (w >> 1);
+                        int e0 = v[0] + ax[0] * x + by[0] * y, e1 = v[1] + ax[1] * x + by[1] * y,
+                            e2 = v[2] + ax[2] * x + by[2] * y;
+                        if ((e0 | e1 | e2) < 0) mask &= ~(1u << w);
+                    }
+                } else {
+                    Edges<long long> e = make_edges<long long>(t.X, t.Y);
+                    long long E[3];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) E[k] = e.at(k, S0x, S0y);
+                    area = __ll2float_rn(e.area);
+                    sm.p[tid] = make_int4((int)E[0], (int)(E[0] >> 32), (int)E[1], (int)(E[1] >> 32));
+                    sm.q[tid] = make_int4((int)E[2], (int)(E[2] >> 32), (int)e.a[0],
+                                          ADMS_LARGE | e.thr[0] | (e.thr[1] << 1) | (e.thr[2] << 2));
+                    sm.s[tid] = make_int4((int)e.b[0], (int)e.a[1], (int)e.b[1], 0);
+                }
+                sm.r[tid] = make_int4(__float_as_int(area), __float_as_int(t.z0), __float_as_int(t.dz1),
+                                      __float_as_int(t.dz2));
+                sm.id[tid] = f;
             }
         }
-        __syncthreads();
-        unsigned wmask = 0;
-        if ((int)threadIdx.x < m && sm[threadIdx.x].valid) {
-            int r0 = max((int)sm[threadIdx.x].by0 - row0, 0), r1 = min((int)sm[threadIdx.x].by1 - row0, ADMS_TILE - 1);
-            for (int w = r0 >> 1; w <= (r1 >> 1); ++w) wmask |= 1u << w;  // empty when r1 < r0
-        }
-        for (unsigned mm = wmask; mm; mm &= mm - 1) {
-            int w = __ffs(mm) - 1;
-            wlist[w][atomicAdd(&wcount[w], 1)] = (unsigned char)threadIdx.x;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            unsigned mw = __ballot_sync(0xffffffffu, (mask >> w) & 1u);
+            if (lane == w) sm.mask[w][warp] = mw;
         }
         __syncthreads();
-        int cntw = wcount[warp];
-        for (int j = 0; j < cntw; ++j) {
-            const TriRec& r = sm[wlist[warp][j]];
-            if (px < r.bx0 || px > r.bx1 || py < r.by0 || py > r.by1) continue;
-            test_tri(r, Sx, Sy, best);
+        for (int g = 0; g < m; g += 32) {
+            for (unsigned mm = sm.mask[warp][g >> 5]; mm; mm &= mm - 1) {
+                int j = g + __ffs(mm) - 1;
+                int4 p = sm.p[j], q = sm.q[j];
+                float f1, f2;
+                if (!(q.w & ADMS_LARGE)) {
+                    int e0 = p.x + p.y * lx + p.z * ly, e1 = q.x + q.y * lx + q.z * ly, e2 = near_third(p.w, e0, e1);
+                    if ((e0 | e1 | e2) < 0) continue;
+                    f1 = __int2float_rn(e1 + ((q.w >> 1) & 1));
+                    f2 = __int2float_rn(e2 + (q.w >> 2));
+                } else {
+                    int4 s = sm.s[j];
+                    long long E0 = ((long long)p.y << 32) | (unsigned)p.x, E1 = ((long long)p.w << 32) | (unsigned)p.z;
+                    long long E2 = ((long long)q.y << 32) | (unsigned)q.x;
+                    int dx = 256 * lx, dy = 256 * ly;
+                    long long e0 = E0 + (long long)q.z * dx + (long long)s.x * dy;
+                    long long e1 = E1 + (long long)s.y * dx + (long long)s.z * dy;
+                    // a_2 = -(a_0 + a_1): the edges of a closed triangle
+                    long long e2 = E2 - ((long long)q.z + s.y) * dx - ((long long)s.x + s.z) * dy;
+                    if (e0 < (q.w & 1) || e1 < ((q.w >> 1) & 1) || e2 < ((q.w >> 2) & 1)) continue;
+                    f1 = __ll2float_rn(e1);
+                    f2 = __ll2float_rn(e2);
+                }
+                int4 r = sm.r[j];
+                sink.take(depth_key(f1, f2, __int_as_float(r.x), __int_as_float(r.y), __int_as_float(r.z),
+                                    __int_as_float(r.w), sm.id[j]));
+            }
         }
     }
-    if (inside) keys[pix] = best;
 }
 
-__global__ void __launch_bounds__(256) k_raster(const TriRec* __restrict__ rec, const TriBin* __restrict__ bin, int F,
-                                                int W, int H, int tiles_x, int tiles_y,
-                                                const int* __restrict__ tile_off, const int* __restrict__ tile_count,
-                                                const int* __restrict__ list, long long capacity,
-                                                unsigned long long* __restrict__ keys,
-                                                unsigned long long* __restrict__ overflow_ctr) {
-    __shared__ TriRec sm[256];
-    raster_tile_body(rec, bin, F, W, H, tiles_x, tiles_y, tile_off, tile_count, list, capacity, keys, overflow_ctr,
-                     blockIdx.y, blockIdx.x, sm);
+// one 16x16 tile of one view: the minimum key per pixel
+__device__ __forceinline__ void raster_tile_body(const TileArgs& A, unsigned long long* __restrict__ keys, int b,
+                                                 int tile, TileSmem& sm) {
+    size_t t = (size_t)b * A.tiles_x * A.tiles_y + tile;
+    long long off = A.tile_off[t];
+    int cnt = A.tile_count[t];
+    if (cnt == 0) return;  // no binned triangle: the small-triangle pass left the final keys
+    int px = (tile % A.tiles_x) * ADMS_TILE + tile_x(threadIdx.x), py = (tile / A.tiles_x) * ADMS_TILE + tile_y(threadIdx.x);
+    bool inside = px < A.W && py < A.H;
+    size_t pix = ((size_t)b * A.H + py) * A.W + px;
+    KeySink<1> sink;
+    sink.kb[0] = inside ? keys[pix] : ADMS_EMPTY_KEY;
+    raster_tile_walk<1>(A, b, tile, off, cnt, sm, sink);
+    if (inside) keys[pix] = sink.kb[0];
+}
+
+__global__ void __launch_bounds__(256) k_raster(const TileArgs A, unsigned long long* __restrict__ keys) {
+    __shared__ TileSmem sm;
+    raster_tile_body(A, keys, blockIdx.y, blockIdx.x, sm);
 }
 
 // Depth peeling in one pass (Sec. 5.2): per sample the L nearest fragments,
 // front to back, which are exactly the layers that L peeling passes with a
 // two-sided test on the packed depth|id key would find (the keys of a sample are
-// distinct). One block per (view, 16x16 tile) as in k_raster, the tile's records
-// staged through shared memory, a KB-entry k-buffer per thread in registers
+// distinct). The walk of k_raster with a KB-entry k-buffer per thread in registers
 // (KB >= L); every triangle must be binned (no small-triangle pass). keys holds
 // L slices of [B][H][W].
 template <int KB>
-__global__ void __launch_bounds__(256) k_raster_kbuf(const TriRec* __restrict__ rec, const TriBin* __restrict__ bin,
-                                                     int F, int W, int H, int tiles_x, int tiles_y,
-                                                     const int* __restrict__ tile_off,
-                                                     const int* __restrict__ tile_count, const int* __restrict__ list,
-                                                     long long capacity, unsigned long long* __restrict__ keys, int L,
-                                                     int B, unsigned long long* __restrict__ overflow_ctr) {
-    __shared__ TriRec sm[256];
+__global__ void __launch_bounds__(256) k_raster_kbuf(const TileArgs A, unsigned long long* __restrict__ keys, int L,
+                                                     int B) {
+    __shared__ TileSmem sm;
     int b = blockIdx.y, tile = blockIdx.x;
-    int tx = tile % tiles_x, ty = tile / tiles_x;
-    int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
-    int px = tx * ADMS_TILE + lx, py = ty * ADMS_TILE + ly;
-    int Sx = 256 * px + 128, Sy = 256 * py + 128;
-    bool inside = px < W && py < H;
-    unsigned long long kb[KB];
+    int px = (tile % A.tiles_x) * ADMS_TILE + tile_x(threadIdx.x), py = (tile / A.tiles_x) * ADMS_TILE + tile_y(threadIdx.x);
+    KeySink<KB> sink;
 #pragma unroll
-    for (int i = 0; i < KB; ++i) kb[i] = ADMS_EMPTY_KEY;
-    size_t t = (size_t)b * tiles_x * tiles_y + tile;
-    long long off = tile_off[t];
-    int cnt = tile_count[t];
-    const TriRec* rb = rec + (size_t)b * F;
-    const TriBin* bb = bin + (size_t)b * F;
-    bool overflow = off + cnt > capacity;
-    int n = overflow ? F : cnt;
-    if (overflow && threadIdx.x == 0) atomicAdd(overflow_ctr, 1ull);
-    for (int c0 = 0; c0 < n; c0 += 256) {
-        int m = min(256, n - c0);
-        __syncthreads();
-        if ((int)threadIdx.x < m) {
-            if (overflow) {
-                int id = c0 + threadIdx.x;
-                TriBin tb = bb[id];
-                if (tb.bx0 <= tb.bx1) sm[threadIdx.x] = rb[id];
-                else sm[threadIdx.x].valid = 0;
-            } else {
-                sm[threadIdx.x] = rb[list[off + c0 + threadIdx.x]];
-            }
-        }
-        __syncthreads();
-        for (int k = 0; k < m; ++k) {
-            const TriRec& r = sm[k];
-            if (!r.valid) continue;
-            if (px < r.bx0 || px > r.bx1 || py < r.by0 || py > r.by1) continue;
-            test_tri_kbuf<KB>(r, Sx, Sy, kb);
-        }
-    }
-    if (!inside) return;
-    size_t pix = ((size_t)b * H + py) * W + px, layer = (size_t)B * H * W;
+    for (int i = 0; i < KB; ++i) sink.kb[i] = ADMS_EMPTY_KEY;
+    size_t t = (size_t)b * A.tiles_x * A.tiles_y + tile;
+    raster_tile_walk<KB>(A, b, tile, A.tile_off[t], A.tile_count[t], sm, sink);
+    if (px >= A.W || py >= A.H) return;
+    size_t pix = ((size_t)b * A.H + py) * A.W + px, layer = (size_t)B * A.H * A.W;
 #pragma unroll
     for (int i = 0; i < KB; ++i)
-        if (i < L) keys[pix + (size_t)i * layer] = kb[i];
+        if (i < L) keys[pix + (size_t)i * layer] = sink.kb[i];
 }
+
+static TileLists tile_lists(const TriRec* rec, const int* list, long long capacity, long long records) {
+    return TileLists{list, reinterpret_cast<const int*>(rec + records), capacity,
+                     capacity + records * (long long)(sizeof(TriRec) / sizeof(int))};
+}
+
+struct RasterBatch {
+    TileArgs a[ADMS_BATCH_JOBS];
+    unsigned long long* keys[ADMS_BATCH_JOBS];
+};
 // persistent: block k takes items k, k + gridDim.x, ... (the items are equal
 // 16x16 tiles, so a static stride balances them without a shared counter); the
 // jobs' arguments are kernel parameters (up to 64 jobs per launch)
-__global__ void __launch_bounds__(256) k_raster_batch(const RasterBatch P, const WorkItem* __restrict__ items, int n,
-                                                      int job0) {
-    __shared__ TriRec sm[256];
+__global__ void __launch_bounds__(256) k_raster_batch(const __grid_constant__ RasterBatch P,
+                                                      const WorkItem* __restrict__ items, int n, int job0) {
+    __shared__ TileSmem sm;
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         WorkItem w = items[it];
-        const RasterJob& R = P.a[w.job - job0];
-        int tile = (w.y0 / ADMS_TILE) * R.tiles_x + w.x0 / ADMS_TILE;
-        raster_tile_body(R.rec, R.bin, R.F, R.W, R.H, R.tiles_x, R.tiles_y, R.tile_off, R.tile_count, R.list,
-                         R.capacity, R.keys, R.overflow_ctr, w.view, tile, sm);
+        const TileArgs& A = P.a[w.job - job0];
+        int tile = (w.y0 / ADMS_TILE) * A.tiles_x + w.x0 / ADMS_TILE;
+        raster_tile_body(A, P.keys[w.job - job0], w.view, tile, sm);
     }
 }
 
@@ -550,7 +645,12 @@ cudaError_t raster_tiles_batched(const RasterJob* args, const int* item_off, int
         int j1 = std::min(n_jobs, j0 + ADMS_BATCH_JOBS);
         int s0 = item_off[j0], n = item_off[j1] - s0;
         if (n <= 0) continue;
-        memcpy(P.a, args + j0, sizeof(RasterJob) * (j1 - j0));
+        for (int j = j0; j < j1; ++j) {
+            const RasterJob& r = args[j];
+            P.a[j - j0] = TileArgs{r.rec, r.bin, r.F, r.W, r.H, r.tiles_x, r.tiles_y, r.tile_off, r.tile_count,
+                                   tile_lists(r.rec, r.list, r.capacity, r.records), r.overflow_ctr};
+            P.keys[j - j0] = r.keys;
+        }
         k_raster_batch<<<std::min(blocks, n), 256, 0, st>>>(P, items + s0, n, j0);
         count_launches(1);
         cudaError_t e = cudaGetLastError();
@@ -576,36 +676,39 @@ cudaError_t raster_prepare(const RasterIn& in, RasterScratch& s, cudaStream_t st
     int bs = 256;
     k_transform<<<(B * V + bs - 1) / bs, bs, 0, st>>>(in.pos, V, in.views, B, W, H, s.clip, s.vs, s.scr,
                                                     s.total_pairs);
-    if (in.small_px > ADMS_SMALL_PX)
+    if (in.zfilter && in.small_px > ADMS_SMALL_PX)
         k_setup<true><<<(B * F + bs - 1) / bs, bs, 0, st>>>(in.tri, F, s.vs, V, B, W, H, tiles_x, tiles_y, s.rec,
-                                                          s.bin, s.asign, s.tile_count, in.keys, in.small_px, in.zfilter);
+                                                          s.bin, s.asign, s.tile_count, in.keys, in.small_px);
     else
         k_setup<false><<<(B * F + bs - 1) / bs, bs, 0, st>>>(in.tri, F, s.vs, V, B, W, H, tiles_x, tiles_y, s.rec,
-                                                           s.bin, s.asign, s.tile_count, in.keys, in.small_px, 0);
+                                                           s.bin, s.asign, s.tile_count, in.keys, in.small_px);
     k_list_alloc<<<(ntiles + bs - 1) / bs, bs, 0, st>>>(s.tile_count, ntiles, s.tile_off,
                                                        reinterpret_cast<unsigned long long*>(s.total_pairs));
-    k_bin_fill<<<(B * F + bs - 1) / bs, bs, 0, st>>>(s.bin, F, B, tiles_x, tiles_y, s.tile_off, s.tile_cursor,
-                                                   s.list, s.list_capacity, in.adj, s.asign, s.silmask);
+    k_bin_fill<<<(B * F + bs - 1) / bs, bs, 0, st>>>(s.rec, s.bin, F, B, tiles_x, tiles_y, s.tile_off, s.tile_cursor,
+                                                   tile_lists(s.rec, s.list, s.list_capacity, (long long)B * F),
+                                                   in.adj, s.asign, s.silmask);
     count_launches(4);
     return cudaGetLastError();
 }
 
+static TileArgs tile_args(const RasterIn& in, const RasterScratch& s) {
+    return TileArgs{s.rec, s.bin, in.F, in.W, in.H, (in.W + ADMS_TILE - 1) / ADMS_TILE,
+                    (in.H + ADMS_TILE - 1) / ADMS_TILE, s.tile_off, s.tile_count,
+                    tile_lists(s.rec, s.list, s.list_capacity, (long long)in.B * in.F), s.overflow_ctr};
+}
+
 cudaError_t raster_tiles(const RasterIn& in, RasterScratch& s, cudaStream_t st) {
-    int tiles_x = (in.W + ADMS_TILE - 1) / ADMS_TILE, tiles_y = (in.H + ADMS_TILE - 1) / ADMS_TILE;
-    dim3 grid(tiles_x * tiles_y, in.B);
-    k_raster<<<grid, 256, 0, st>>>(s.rec, s.bin, in.F, in.W, in.H, tiles_x, tiles_y, s.tile_off, s.tile_count, s.list,
-                                   s.list_capacity, in.keys, s.overflow_ctr);
+    TileArgs a = tile_args(in, s);
+    k_raster<<<dim3(a.tiles_x * a.tiles_y, in.B), 256, 0, st>>>(a, in.keys);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t raster_tiles_peeled(const RasterIn& in, RasterScratch& s, int L, cudaStream_t st) {
     if (L < 1 || L > 16) return cudaErrorInvalidValue;
-    int tiles_x = (in.W + ADMS_TILE - 1) / ADMS_TILE, tiles_y = (in.H + ADMS_TILE - 1) / ADMS_TILE;
-    dim3 grid(tiles_x * tiles_y, in.B);
-#define ADMS_KBUF_LAUNCH(KB)                                                                                        \
-    k_raster_kbuf<KB><<<grid, 256, 0, st>>>(s.rec, s.bin, in.F, in.W, in.H, tiles_x, tiles_y, s.tile_off,           \
-                                            s.tile_count, s.list, s.list_capacity, in.keys, L, in.B, s.overflow_ctr)
+    TileArgs a = tile_args(in, s);
+    dim3 grid(a.tiles_x * a.tiles_y, in.B);
+#define ADMS_KBUF_LAUNCH(KB) k_raster_kbuf<KB><<<grid, 256, 0, st>>>(a, in.keys, L, in.B)
     if (L <= 2) ADMS_KBUF_LAUNCH(2);
     else if (L <= 4) ADMS_KBUF_LAUNCH(4);
     else if (L <= 8) ADMS_KBUF_LAUNCH(8);

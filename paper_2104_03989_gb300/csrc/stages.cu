@@ -43,7 +43,7 @@ StageWork carve_work(unsigned char* base, size_t V, size_t F, size_t B, int H, i
     size_t ntiles = B * (size_t)((W + ADMS_TILE - 1) / ADMS_TILE) * (size_t)((H + ADMS_TILE - 1) / ADMS_TILE);
     w.s.scr = reinterpret_cast<float4*>(take(B * V * sizeof(float4)));
     w.s.vs = reinterpret_cast<VtxS*>(take(B * V * sizeof(VtxS)));
-    w.s.rec = reinterpret_cast<TriRec*>(take(B * F * sizeof(TriRec)));
+    w.s.rec = reinterpret_cast<TriRec*>(take(B * F * ADMS_REC_PAD * sizeof(TriRec)));
     w.s.bin = reinterpret_cast<TriBin*>(take(B * F * sizeof(TriBin)));
     w.s.asign = reinterpret_cast<int8_t*>(take(B * F));
     w.s.silmask = reinterpret_cast<uint8_t*>(take(B * F));
