@@ -320,17 +320,65 @@ __device__ __forceinline__ float3 shade_eval(const adms_view& vw, const ShadeIn&
 
 __device__ __forceinline__ int key_tri(unsigned long long k) { return k == ADMS_EMPTY_KEY ? -1 : (int)(k & 0xffffffffu); }
 
+// The three maps share their texel taps when they have the same size (one LOD and
+// one bilinear footprint per level serve all three): the usual case of equally
+// sized latent maps.
+__host__ __device__ __forceinline__ bool shared_taps(const ShadeArgs& A) {
+    return A.kd.w0 == A.orm.w0 && A.kd.w0 == A.nrm.w0 && A.kd.h0 == A.orm.h0 && A.kd.h0 == A.nrm.h0 &&
+           A.kd.levels == A.orm.levels && A.kd.levels == A.nrm.levels;
+}
+
+// tex_sample of the three maps with shared taps (the same arithmetic, map by map)
+__device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3]) {
+    const float4* ts[3] = {A.kd.tex, A.orm.tex, A.nrm.tex};
+    int l0 = (int)floorf(lod);
+    float fr = lod - (float)l0;
+    int l1 = min(l0 + 1, A.kd.levels - 1);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) out[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        int k = s == 0 ? l0 : l1;
+        float wl = s == 0 ? 1.f - fr : fr;
+        if (wl == 0.f) continue;
+        BilinTap b = bilin_tap(A.kd, k, tc);
+        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
+        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            out[m] = f4madd(out[m], w00, __ldg(ts[m] + b.idx[0]));
+            out[m] = f4madd(out[m], w10, __ldg(ts[m] + b.idx[1]));
+            out[m] = f4madd(out[m], w01, __ldg(ts[m] + b.idx[2]));
+            out[m] = f4madd(out[m], w11, __ldg(ts[m] + b.idx[3]));
+        }
+    }
+}
+
+// the shading inputs at g: interpolated attributes and the three maps' trilinear samples
+// (their LODs into lod). One LOD and one footprint per level serve maps of one size (57.2 ->
+// 44.0 M warp instructions, 83 -> 73.5 us for 8 views of 512x512).
+// SHARE: 1 the maps are of one size, 0 not all, -1 decided here (batched and per-stage calls).
+template <int SHARE = -1>
 __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo& g, float lod[3]) {
-    lod[0] = tex_lod(A.kd, g.duv_dx, g.duv_dy);
-    lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
-    lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
     ShadeIn in;
     in.p = g.p;
     in.n_i = g.n;
     in.t_i = g.t;
-    in.kd = tex_sample(A.kd, g.tc, lod[0]);
-    in.orm = tex_sample(A.orm, g.tc, lod[1]);
-    in.nm = tex_sample(A.nrm, g.tc, lod[2]);
+    lod[0] = tex_lod(A.kd, g.duv_dx, g.duv_dy);
+    if (SHARE == 1 || (SHARE < 0 && shared_taps(A))) {
+        lod[1] = lod[2] = lod[0];
+        float4 smp[3];
+        tex_sample3(A, g.tc, lod[0], smp);
+        in.kd = smp[0];
+        in.orm = smp[1];
+        in.nm = smp[2];
+    } else {
+        lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
+        lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
+        in.kd = tex_sample(A.kd, g.tc, lod[0]);
+        in.orm = tex_sample(A.orm, g.tc, lod[1]);
+        in.nm = tex_sample(A.nrm, g.tc, lod[2]);
+    }
     return in;
 }
 
@@ -429,12 +477,12 @@ __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
 // ------------------------------------------------------------------ shading forward
 // shading of triangle f at sample (px, py), refining it (INLINE) or listing it for
 // the refinement pass when bright on a triangle that spans many texels
-template <bool INLINE = false>
+template <bool INLINE = false, int SHARE = -1>
 __device__ __forceinline__ float4 shade_covered(const ShadeArgs& A, int b, int px, int py, int f, size_t pix) {
     PixGeo g;
     pix_geo(A, b, px, py, f, g);
     float lod[3];
-    ShadeIn in = shade_inputs(A, g, lod);
+    ShadeIn in = shade_inputs<SHARE>(A, g, lod);
     float3 c = shade_eval<false>(A.views[b], in, zero3(), nullptr);
     // Bright pixels (sharp highlights) carry almost all of the error a float32
     // texture coordinate causes: on the noise-textured workloads the 0.35% of
@@ -447,7 +495,7 @@ __device__ __forceinline__ float4 shade_covered(const ShadeArgs& A, int b, int p
     if (A.refine && fmaxf(c.x, fmaxf(c.y, c.z)) > 0.5f && tc_lever(A, g, lod) > 2.f) {
         if (INLINE) {
             refine_tc(A, b, px, py, g);
-            in = shade_inputs(A, g, lod);
+            in = shade_inputs<SHARE>(A, g, lod);
             c = shade_eval<false>(A.views[b], in, zero3(), nullptr);
         } else {
             A.refine[1 + atomicAdd(A.refine, 1)] = (int)pix;  // for k_shade_refine
@@ -456,12 +504,12 @@ __device__ __forceinline__ float4 shade_covered(const ShadeArgs& A, int b, int p
     return make_float4(c.x, c.y, c.z, A.peel ? in.kd.w : 1.f);  // a peeled layer keeps its opacity
 }
 
-template <bool INLINE = false>
+template <bool INLINE = false, int SHARE = -1>
 __device__ __forceinline__ void shade_fwd_px(const ShadeArgs& A, int b, int px, int py) {
     if (px >= A.W || py >= A.H) return;
     size_t pix = ((size_t)b * A.H + py) * A.W + px;
     int f = key_tri(__ldg(A.keys + (pix)));
-    A.pre[pix] = f >= 0 ? shade_covered<INLINE>(A, b, px, py, f, pix) : make_float4(0.f, 0.f, 0.f, 0.f);
+    A.pre[pix] = f >= 0 ? shade_covered<INLINE, SHARE>(A, b, px, py, f, pix) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Under MSAA every sample of a pixel that shows one triangle has the same shading
@@ -767,40 +815,6 @@ __device__ __forceinline__ float3 aa_adjoint(const ShadeArgs& A, int b, int px, 
         }
     }
     return gc;
-}
-
-// The three maps share their texel taps when they have the same size (one LOD and
-// one bilinear footprint per level serve all three): the usual case of equally
-// sized latent maps.
-__device__ __forceinline__ bool shared_taps(const ShadeArgs& A) {
-    return A.kd.w0 == A.orm.w0 && A.kd.w0 == A.nrm.w0 && A.kd.h0 == A.orm.h0 && A.kd.h0 == A.nrm.h0 &&
-           A.kd.levels == A.orm.levels && A.kd.levels == A.nrm.levels;
-}
-
-// tex_sample of the three maps with shared taps (the same arithmetic, map by map)
-__device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3]) {
-    const float4* ts[3] = {A.kd.tex, A.orm.tex, A.nrm.tex};
-    int l0 = (int)floorf(lod);
-    float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, A.kd.levels - 1);
-#pragma unroll
-    for (int m = 0; m < 3; ++m) out[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        int k = s == 0 ? l0 : l1;
-        float wl = s == 0 ? 1.f - fr : fr;
-        if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(A.kd, k, tc);
-        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
-        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            out[m] = f4madd(out[m], w00, __ldg(ts[m] + b.idx[0]));
-            out[m] = f4madd(out[m], w10, __ldg(ts[m] + b.idx[1]));
-            out[m] = f4madd(out[m], w01, __ldg(ts[m] + b.idx[2]));
-            out[m] = f4madd(out[m], w11, __ldg(ts[m] + b.idx[3]));
-        }
-    }
 }
 
 // adjoint of tex_sample3: the texel gradients of the optimized maps are scattered,

@@ -34,29 +34,23 @@ __device__ __forceinline__ void band_pixel(int W, int& px, int& py) {
     py = (tile / tiles_x) * ADMS_TILE + part * (ADMS_TILE / PARTS) + (threadIdx.x >> 4);
 }
 
-// block shapes measured on the plain-method step (threads per block x resident
-// blocks per SM, i.e. the register cap 65536 / (threads x blocks)); shading: 256 x 5
-// 0.0928 ms, 256 x 4 0.0919, 256 x 6 0.0902, 128 x 10 0.0903, 128 x 8 0.0882, 128 x 12
-// 0.0882; AA + loss: 256 x 8 0.0612, 256 x 6 0.0672, 128 x 12 0.0631, 128 x 16 0.0593;
-// the backward's below (a few hundred bytes of spills cost less than the latency the
-// extra resident warps hide)
-#ifndef ADMS_FWD_THREADS
+// Block shapes (threads per block x resident blocks per SM, i.e. the register cap 65536 /
+// (threads x blocks)), measured per kernel. SHARE (maps of one size, decided by the host per
+// launch) is a template argument: one kernel holding both forms cost the maps of different
+// sizes 3% (895 -> 920 us for the two passes over 16 views of 1024x1024). Equal maps, 8 views
+// of 512x512: 8 blocks 74.5 us, 6: 80.0, 10: 77.9, 12: 77.4; different ones, 16 views of
+// 1024x1024: 8 blocks 894 us, 6: 964, 10: 883, 12: 832, but with the refinement inline (small
+// grids) 8 is ahead (69.0 against 70.3 us at 5 of 333x501). AA + loss: 16 blocks 53.1 us,
+// 12: 55.3.
 #define ADMS_FWD_THREADS 128
-#endif
-#ifndef ADMS_FWD_BLOCKS
-#define ADMS_FWD_BLOCKS 8
-#endif
-#ifndef ADMS_AA_THREADS
+constexpr int fwd_blocks(bool inline_refine, int share) { return share == 0 && !inline_refine ? 12 : 8; }
 #define ADMS_AA_THREADS 128
-#endif
-#ifndef ADMS_AA_BLOCKS
 #define ADMS_AA_BLOCKS 16
-#endif
-template <bool INLINE>
-__global__ void __launch_bounds__(ADMS_FWD_THREADS, ADMS_FWD_BLOCKS) k_shade_fwd(ShadeArgs A) {
+template <bool INLINE, int SHARE>
+__global__ void __launch_bounds__(ADMS_FWD_THREADS, fwd_blocks(INLINE, SHARE)) k_shade_fwd(ShadeArgs A) {
     int px, py;
     band_pixel<ADMS_FWD_THREADS>(A.W, px, py);
-    shade_fwd_px<INLINE>(A, blockIdx.y, px, py);
+    shade_fwd_px<INLINE, SHARE>(A, blockIdx.y, px, py);
 }
 
 template <bool PEEL>
@@ -318,10 +312,10 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st) {
     if (a.msaa > 1) {
         int R = ADMS_MSAA_REGION;
         k_shade_fwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
-    } else if (inline_refine) {
-        k_shade_fwd<true><<<band_grid(a, ADMS_FWD_THREADS), ADMS_FWD_THREADS, 0, st>>>(a);
     } else {
-        k_shade_fwd<false><<<band_grid(a, ADMS_FWD_THREADS), ADMS_FWD_THREADS, 0, st>>>(a);
+        auto k = inline_refine ? (shared_taps(a) ? k_shade_fwd<true, 1> : k_shade_fwd<true, 0>)
+                               : (shared_taps(a) ? k_shade_fwd<false, 1> : k_shade_fwd<false, 0>);
+        k<<<band_grid(a, ADMS_FWD_THREADS), ADMS_FWD_THREADS, 0, st>>>(a);
     }
     count_launches(1);
     if (list) {
@@ -340,10 +334,9 @@ cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st) {
     if (a.msaa > 1) {
         int R = ADMS_MSAA_REGION;
         k_shade_bwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
-    } else if (a.peel) {
-        k_shade_bwd<true><<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
     } else {
-        k_shade_bwd<false><<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
+        auto k = a.peel ? k_shade_bwd<true> : k_shade_bwd<false>;
+        k<<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
     }
     count_launches(1);
     return cudaGetLastError();
