@@ -65,7 +65,7 @@ __device__ __forceinline__ double warp_sum_d(double x) {
 
 // (hi, lo) += (bhi, blo): hi the float32 sum, lo the rounding errors lost so far
 // (Knuth's TwoSum, no renormalisation, so an infinite or NaN hi stays what a plain
-// float32 sum gives). hi + lo carries about 46 bits over the few hundred terms of a block.
+// float32 sum gives). hi + lo carries about 46 bits over the few thousand terms of a block.
 __device__ __forceinline__ void comp_add(float& hi, float& lo, float bhi, float blo) {
     float s = __fadd_rn(hi, bhi);
     float bb = __fsub_rn(s, hi);
@@ -73,40 +73,34 @@ __device__ __forceinline__ void comp_add(float& hi, float& lo, float bhi, float 
     lo = __fadd_rn(__fadd_rn(lo, blo), e);
     hi = s;
 }
-// The sum of a block's per-pixel loss terms (three channels per thread), in thread 0.
-// Every thread of the block calls it; red: 2 floats per warp of shared memory.
-// Float64 runs at 1/64 of the float32 rate here: the warp sums in float64 held the FP64
-// pipe 73% busy and were most of the antialiasing kernel; the compensated float32 sums
-// cost 8 float32 operations a step instead of a 16-cycle DADD. Where the float32 sum is
-// not finite (a term is not, or the sum leaves float32's range) the block's sum is formed
-// in float64 as the terms stand.
-__device__ __forceinline__ double block_sum3(float a, float b, float c, float* red) {
-    float hi = a, lo = 0.f;
-    comp_add(hi, lo, b, 0.f);
-    comp_add(hi, lo, c, 0.f);
-    int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
+// A thread's running sum of its pixels' loss terms and the sum of a block's (in thread 0;
+// every thread calls it; red: 2 floats per warp of shared memory). Float64 runs at 1/64 of
+// the float32 rate here: the warp sums in float64 held the FP64 pipe 73% busy and were most
+// of the antialiasing kernel; the compensated sums cost 8 float32 operations a step instead
+// of a 16-cycle DADD. The terms are summed scaled by 2^-16 (exact), so that no block's sum
+// leaves float32's range unless one of its terms does.
+struct LossSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float a, float b, float c) {
+        comp_add(hi, lo, a * 0x1p-16f, 0.f);
+        comp_add(hi, lo, b * 0x1p-16f, 0.f);
+        comp_add(hi, lo, c * 0x1p-16f, 0.f);
+    }
+    __device__ __forceinline__ double block(float* red) {
+        int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        comp_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
-    if ((threadIdx.x & 31) == 0) {
-        red[2 * w] = hi;
-        red[2 * w + 1] = lo;
-    }
-    __syncthreads();
-    hi = red[0];
-    lo = red[1];
-    for (int k = 1; k < nw; ++k) comp_add(hi, lo, red[2 * k], red[2 * k + 1]);
-    if (isfinite(hi)) return threadIdx.x == 0 ? (double)hi + (double)lo : 0.0;
-    __syncthreads();  // the same branch for the whole block: red is the same for every thread
-    double d = warp_sum_d((double)a + (double)b + (double)c), s = 0.0;
-    for (int k = 0; k < nw; ++k) {
-        if (w == k && (threadIdx.x & 31) == 0) *reinterpret_cast<double*>(red) = d;
+        for (int o = 16; o > 0; o >>= 1)
+            comp_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+        if ((threadIdx.x & 31) == 0) {
+            red[2 * w] = hi;
+            red[2 * w + 1] = lo;
+        }
         __syncthreads();
-        s += *reinterpret_cast<double*>(red);
-        __syncthreads();
+        if (threadIdx.x != 0) return 0.0;
+        for (int k = 1; k < nw; ++k) comp_add(hi, lo, red[2 * k], red[2 * k + 1]);
+        return 65536.0 * (isfinite(hi) ? (double)hi + (double)lo : (double)hi);
     }
-    return s;
-}
+};
 
 // ------------------------------------------------------------------ double-float
 // hi + lo with |lo| <= ulp(hi) / 2: about 48 significant bits from float32

@@ -601,11 +601,14 @@ __device__ __forceinline__ float3 f3of(float4 a) { return f3(a.x, a.y, a.z); }
 // its blend over the composite behind it, alpha c + (1 - alpha) under (black
 // background behind the last layer; alpha 0 where the layer is empty)
 template <bool PEEL>
-__device__ __forceinline__ float3 layer_colour(const ShadeArgs& A, size_t pix) {
-    float4 p = A.pre[pix];
+__device__ __forceinline__ float3 layer_blend(const ShadeArgs& A, size_t pix, float4 p) {
     if (!PEEL) return f3of(p);
     float3 u = A.under ? f3of(A.under[pix]) : zero3();
     return p.w * f3of(p) + (1.f - p.w) * u;
+}
+template <bool PEEL>
+__device__ __forceinline__ float3 layer_colour(const ShadeArgs& A, size_t pix) {
+    return layer_blend<PEEL>(A, pix, A.pre[pix]);
 }
 
 // Gamma(log(max(x, 0) + 1)) with the sRGB Gamma of Sec. 5.3, and its
@@ -652,59 +655,76 @@ __device__ __forceinline__ void neighbour(int nbi, int px, int py, int& qx, int&
     qy = py + (nbi == 2 ? -1 : nbi == 3 ? 1 : 0);
 }
 
-// one block of pixels: AA, loss terms and dL/d(AA colour); the block's loss sum
-// goes to A.loss_acc (block-collective: every thread of the block calls it)
+// AA, loss terms and dL/d(AA colour) of one pixel; its loss terms go to sum. Issue-bound (83%
+// of the slots at 742 instructions a warp): the four neighbours share one copy of the pair
+// code, which only pixels beside another triangle enter, told by the keys' low words (the
+// neighbours' at constant offsets), and empty pixels read no colour. 8 views of 512x512 53 ->
+// 49 us, 16 of 1024x1024 (two passes) 703 -> 671, 16 passes over peeled layers 1023 -> 1005.
+// Strips of 2 or 4 rows per thread (ids reused downwards, a quarter of the block sums) lost
+// more in loads in flight than they saved (52 and 56 us), blocks of 256 threads too (51).
 // PEEL: A is a layer of a depth-peeled composite (A.peel set); a separate
 // instantiation keeps the opaque path's registers to its own needs
-template <bool PEEL = false>
-__device__ __forceinline__ void aa_loss_block(const ShadeArgs& A, int b, int px, int py, float* red) {
-    bool inside = px < A.W && py < A.H;
-    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
-    if (inside) {
-        size_t pix = ((size_t)b * A.H + py) * A.W + px;
-        unsigned long long kp = __ldg(A.keys + (pix));
-        float3 cp = layer_colour<PEEL>(A, pix);
-        float3 out = cp;
-        unsigned amask = 0;  // neighbours whose pair blends (tau != 1/2): the backward visits only these
-        if (A.aa) {
-#pragma unroll
-            for (int nbi = 0; nbi < 4; ++nbi) {
-                int qx, qy;
-                neighbour(nbi, px, py, qx, qy);
-                if (qx < 0 || qx >= A.W || qy < 0 || qy >= A.H) continue;
-                size_t qpix = ((size_t)b * A.H + qy) * A.W + qx;
-                PairInfo pi;
-                if (!pair_eval(A, b, px, py, kp, qx, qy, __ldg(A.keys + (qpix)), nbi < 2 ? 0 : 1, pi)) continue;
-                float om = pi.t.tau - 0.5f;
-                if (om != 0.f) amask |= 1u << nbi;
-                // the other pixel blends toward the owner when tau > 1/2, the owner toward it when tau < 1/2
-                bool p_target = om > 0.f ? !pi.p_owner : (om < 0.f ? pi.p_owner : false);
-                if (p_target) out += fabsf(om) * (layer_colour<PEEL>(A, qpix) - cp);
-            }
-        }
-        if (A.ref) {
-            const float* y = A.ref + pix * 3;
-            float y0 = y[0], y1 = y[1], y2 = y[2];
-            float g0 = 0.f, g1 = 0.f, g2 = 0.f;
-            // black on black (the background, half of most views) has no loss and no gradient in
-            // any of the losses: the warps that see nothing else skip their tone maps
-            if (out.x != 0.f || out.y != 0.f || out.z != 0.f || y0 != 0.f || y1 != 0.f || y2 != 0.f) {
-                l0 = loss_term(A.loss_kind, out.x, y0, &g0);
-                l1 = loss_term(A.loss_kind, out.y, y1, &g1);
-                l2 = loss_term(A.loss_kind, out.z, y2, &g2);
-            }
-            A.gprime[pix] = make_float4(g0 * A.loss_scale, g1 * A.loss_scale, g2 * A.loss_scale, __uint_as_float(amask));
-        }
-        if (A.out_img) {
-            A.out_img[pix * 3] = out.x;
-            A.out_img[pix * 3 + 1] = out.y;
-            A.out_img[pix * 3 + 2] = out.z;
-        }
-        if (A.acol) A.acol[pix] = make_float4(out.x, out.y, out.z, __uint_as_float(amask));
+template <bool PEEL>
+__device__ __forceinline__ void aa_pixel(const ShadeArgs& A, int b, int px, int py, LossSum& sum) {
+    if (px >= A.W || py >= A.H) return;
+    size_t pix = ((size_t)b * A.H + py) * A.W + px;
+    // triangle ids are the keys' low words (-1: empty)
+    const int* ids = reinterpret_cast<const int*>(A.keys);
+    int id = __ldg(ids + 2 * pix);
+    int up = py > 0 ? __ldg(ids + 2 * (pix - A.W)) : id, down = py + 1 < A.H ? __ldg(ids + 2 * (pix + A.W)) : id;
+    int left = px > 0 ? __ldg(ids + 2 * pix - 2) : id, right = px + 1 < A.W ? __ldg(ids + 2 * pix + 2) : id;
+    float4 own = id >= 0 ? A.pre[pix] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float y0 = 0.f, y1 = 0.f, y2 = 0.f;
+    if (A.ref) {
+        const float* y = A.ref + pix * 3;
+        y0 = y[0];
+        y1 = y[1];
+        y2 = y[2];
     }
+    float3 cp = layer_blend<PEEL>(A, pix, own);
+    float3 out = cp;
+    unsigned amask = 0;  // neighbours whose pair blends (tau != 1/2): the backward visits only these
+    unsigned todo = (left != id ? 1u : 0u) | (right != id ? 2u : 0u) | (up != id ? 4u : 0u) | (down != id ? 8u : 0u);
+    if (todo && A.aa) {
+        unsigned long long kp = __ldg(A.keys + pix);
+        for (; todo; todo &= todo - 1) {
+            int nbi = __ffs(todo) - 1;
+            int qx, qy;
+            neighbour(nbi, px, py, qx, qy);
+            size_t qpix = ((size_t)b * A.H + qy) * A.W + qx;
+            PairInfo pi;
+            if (!pair_eval(A, b, px, py, kp, qx, qy, __ldg(A.keys + qpix), nbi < 2 ? 0 : 1, pi)) continue;
+            float om = pi.t.tau - 0.5f;
+            if (om != 0.f) amask |= 1u << nbi;
+            // the other pixel blends toward the owner when tau > 1/2, the owner toward it when tau < 1/2
+            bool p_target = om > 0.f ? !pi.p_owner : (om < 0.f ? pi.p_owner : false);
+            if (p_target) out += fabsf(om) * (layer_colour<PEEL>(A, qpix) - cp);
+        }
+    }
+    if (A.ref) {
+        float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+        // black on black (the background, half of most views) has no loss and no gradient in
+        // any of the losses: the warps that see nothing else skip their tone maps
+        if (out.x != 0.f || out.y != 0.f || out.z != 0.f || y0 != 0.f || y1 != 0.f || y2 != 0.f) {
+            float l0 = loss_term(A.loss_kind, out.x, y0, &g0), l1 = loss_term(A.loss_kind, out.y, y1, &g1),
+                  l2 = loss_term(A.loss_kind, out.z, y2, &g2);
+            if (A.loss_acc) sum.add(l0, l1, l2);
+        }
+        A.gprime[pix] = make_float4(g0 * A.loss_scale, g1 * A.loss_scale, g2 * A.loss_scale, __uint_as_float(amask));
+    }
+    if (A.out_img) {
+        A.out_img[pix * 3] = out.x;
+        A.out_img[pix * 3 + 1] = out.y;
+        A.out_img[pix * 3 + 2] = out.z;
+    }
+    if (A.acol) A.acol[pix] = make_float4(out.x, out.y, out.z, __uint_as_float(amask));
+}
+
+// the block's loss sum into A.loss_acc (every thread of the block calls it)
+__device__ __forceinline__ void add_block_loss(const ShadeArgs& A, LossSum& sum, float* red) {
     if (!A.loss_acc) return;
     __syncthreads();  // red is free: a persistent block's last item has been summed
-    double s = block_sum3(l0, l1, l2, red);
+    double s = sum.block(red);
     if (threadIdx.x == 0 && s != 0.0) atomicAdd(A.loss_acc, s * (double)A.loss_scale);
 }
 

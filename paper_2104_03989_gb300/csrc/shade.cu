@@ -55,10 +55,12 @@ __global__ void __launch_bounds__(ADMS_FWD_THREADS, fwd_blocks(INLINE, SHARE)) k
 
 template <bool PEEL>
 __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(ShadeArgs A) {
-    __shared__ alignas(8) float red[ADMS_AA_THREADS / 16];
-    int px, py;
-    band_pixel<ADMS_AA_THREADS>(A.W, px, py);
-    aa_loss_block<PEEL>(A, blockIdx.y, px, py, red);
+    __shared__ float red[ADMS_AA_THREADS / 16];
+    int bx = (A.W + 31) / 32;  // a warp takes 32 columns of one row
+    LossSum sum;
+    aa_pixel<PEEL>(A, blockIdx.y, (blockIdx.x % bx) * 32 + (threadIdx.x & 31),
+                   (blockIdx.x / bx) * (ADMS_AA_THREADS / 32) + (threadIdx.x >> 5), sum);
+    add_block_loss(A, sum, red);
 }
 
 // resident blocks per SM of the fused backward (register cap 65536 / (threads x this))
@@ -224,24 +226,28 @@ __global__ void __launch_bounds__(256) k_refine_batch(const ShadeBatch P) {
 template <int KIND>
 __global__ void __launch_bounds__(256, KIND == 2 ? 3 : (KIND == 1 ? 8 : 5))
     k_pixels_batch(const ShadeBatch P, const WorkItem* __restrict__ items, int n, int tw, int job0) {
-    __shared__ alignas(8) float red[16];
+    __shared__ float red[16];
     __shared__ float rows[KIND == 2 ? 8 * 32 * ADMS_VROW : 1];
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         WorkItem w = items[it];
         const ShadeArgs& A = P.a[w.job - job0];
         int px = w.x0 + (int)threadIdx.x % tw, py = w.y0 + (int)threadIdx.x / tw;
         if (KIND == 0) shade_fwd_px(A, w.view, px, py);
-        else if (KIND == 1) aa_loss_block(A, w.view, px, py, red);
+        else if (KIND == 1) {
+            LossSum sum;
+            aa_pixel<false>(A, w.view, px, py, sum);
+            add_block_loss(A, sum, red);
+        }
         else shade_bwd_px(A, w.view, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
     }
 }
 
 // ------------------------------------------------------------------ supersample resolve
 __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
-    __shared__ alignas(8) float red[16];
+    __shared__ float red[16];
     long long n = (long long)r.B * r.H * r.W;
     long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
+    LossSum sum;
     if (pix < n) {
         int b = (int)(pix / ((long long)r.H * r.W));
         int rem = (int)(pix - (long long)b * r.H * r.W);
@@ -261,9 +267,9 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
         if (r.ref) {
             const float* y = r.ref + pix * 3;
             float g0, g1, g2;
-            l0 = loss_term(r.loss_kind, c.x, y[0], &g0);
-            l1 = loss_term(r.loss_kind, c.y, y[1], &g1);
-            l2 = loss_term(r.loss_kind, c.z, y[2], &g2);
+            float l0 = loss_term(r.loss_kind, c.x, y[0], &g0), l1 = loss_term(r.loss_kind, c.y, y[1], &g1),
+                  l2 = loss_term(r.loss_kind, c.z, y[2], &g2);
+            sum.add(l0, l1, l2);
             float k = r.loss_scale * inv;  // each sample carries 1 / s^2 of its pixel
             for (int sy = 0; sy < r.S; ++sy)
                 for (int sx = 0; sx < r.S; ++sx) {
@@ -273,7 +279,7 @@ __global__ void __launch_bounds__(256) k_resolve(ResolveArgs r) {
         }
     }
     if (!r.loss_acc) return;
-    double s = block_sum3(l0, l1, l2, red);
+    double s = sum.block(red);
     if (threadIdx.x == 0 && s != 0.0) atomicAdd(r.loss_acc, s * (double)r.loss_scale);
 }
 
@@ -325,8 +331,10 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st) {
-    if (a.peel) k_aa_loss<true><<<band_grid(a, ADMS_AA_THREADS), ADMS_AA_THREADS, 0, st>>>(a);
-    else k_aa_loss<false><<<band_grid(a, ADMS_AA_THREADS), ADMS_AA_THREADS, 0, st>>>(a);
+    int rows = ADMS_AA_THREADS / 32;
+    dim3 grid(((a.W + 31) / 32) * ((a.H + rows - 1) / rows), a.B);
+    auto k = a.peel ? k_aa_loss<true> : k_aa_loss<false>;
+    k<<<grid, ADMS_AA_THREADS, 0, st>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }
