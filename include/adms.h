@@ -318,6 +318,15 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
  * stay in the chain behind adms_param_view's gradient pointers).
  * ADMS_ERR_STATE for a texture that is not optimized. */
 adms_status adms_job_fold_gradients(adms_ctx* ctx, adms_job job, float* g_kd, float* g_orm, float* g_nrm);
+/* Hand a job's accumulated gradients over: each given output (device; positions
+ * [V][3], folded level-0 texture gradients [h][w][4] as adms_job_fold_gradients,
+ * displacement [h][w], skin weights [V][n_bones]; NULL entries skipped) receives
+ * its gradient times *scale (device scalar; NULL: 1), then every gradient buffer
+ * of the job is zeroed, as by adms_job_zero_gradients. Stream-ordered, no
+ * synchronisation. ADMS_ERR_STATE for a texture, displacement map or weights
+ * that the job does not optimize: nothing is then written or zeroed. */
+adms_status adms_job_take_gradients(adms_ctx* ctx, adms_job job, const float* scale, float* g_pos, float* g_kd,
+                                    float* g_orm, float* g_nrm, float* g_disp, float* g_skin_w);
 /* Zero every gradient buffer of a job (positions, displacement, textures). */
 adms_status adms_job_zero_gradients(adms_ctx* ctx, adms_job job);
 /* Rebuild the mip chains from level 0 (not for per-level textures, whose levels

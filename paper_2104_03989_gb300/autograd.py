@@ -23,6 +23,7 @@ import torch
 from . import binding as B
 
 TEXTURES = ("kd", "orm", "nrm")
+_TAKE = {"pos": "g_pos", "kd": "g_kd", "orm": "g_orm", "nrm": "g_nrm", "disp": "g_disp", "w": "g_skin_w"}
 
 
 def latents(ctx, job, names=None):
@@ -44,10 +45,27 @@ def invalidate(ctx, job):
     B.adms_job_invalidate(ctx.ctx, job)
 
 
+def _context_stream(ctx):
+    s = ctx.stream
+    return s if hasattr(s, "cuda_stream") else torch.cuda.ExternalStream(int(s))
+
+
+def _order(waiting, stream, tensors=()):
+    """Order a stream after another's work so far and keep the tensors' memory until the waiting one is through
+    with them (nothing to do when both are one stream)."""
+    if waiting.cuda_stream != stream.cuda_stream:
+        waiting.wait_stream(stream)
+        for t in tensors:
+            t.record_stream(waiting)
+
+
 class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def forward(fctx, ctx, job, views, refs, names, *tensors):
+        here, there = torch.cuda.current_stream(), _context_stream(ctx)
+        _order(there, here, (refs,))
         loss = ctx.forward_loss([job], [views], [refs])
+        _order(here, there)
         fctx.ctx, fctx.job, fctx.names = ctx, job, names
         fctx.shapes = [t.shape for t in tensors]
         return loss[0].clone()
@@ -55,18 +73,16 @@ class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def backward(fctx, g):
         ctx, job = fctx.ctx, fctx.job
+        here, there = torch.cuda.current_stream(), _context_stream(ctx)
+        scale = g.detach().to(torch.float32).contiguous()
+        grads = [torch.empty(shape, dtype=torch.float32, device=g.device) for shape in fctx.shapes]
+        _order(there, here, (scale, *grads))
         B.adms_job_zero_gradients(ctx.ctx, job)
         ctx.backward([job], recompute_raster=True)
-        p = ctx.params(job)
-        grads = []
-        for name, shape in zip(fctx.names, fctx.shapes):
-            if name in TEXTURES:
-                buf = torch.empty(shape, dtype=torch.float32, device=g.device)
-                B.adms_job_fold_gradients(ctx.ctx, job, **{"g_" + name: buf})
-            else:
-                buf = p["g_" + name].clone()
-            grads.append(buf * g)
-        B.adms_job_zero_gradients(ctx.ctx, job)
+        # times the incoming gradient, folded over the mip chains, the job's buffers left at
+        # zero: one pass over each, and nothing for the host to wait for
+        B.adms_job_take_gradients(ctx.ctx, job, scale, **{_TAKE[n]: buf for n, buf in zip(fctx.names, grads)})
+        _order(here, there)
         return (None, None, None, None, None, *grads)
 
 

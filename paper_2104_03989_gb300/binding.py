@@ -115,6 +115,7 @@ SIGNATURES = {
     "adms_optimizer_step": ([P, P, C.c_int32], C.c_int),
     "adms_job_keys": ([P, C.c_int32, P, C.c_size_t], C.c_int),
     "adms_job_fold_gradients": ([P, C.c_int32, P, P, P], C.c_int),
+    "adms_job_take_gradients": ([P, C.c_int32, P, P, P, P, P, P, P], C.c_int),
     "adms_job_zero_gradients": ([P, C.c_int32], C.c_int),
     "adms_job_invalidate": ([P, C.c_int32], C.c_int),
     "adms_laplacian": ([P, C.c_int32, P, P], C.c_int),
@@ -330,6 +331,12 @@ def adms_job_keys(ctx, job, out_keys):
 
 def adms_job_fold_gradients(ctx, job, g_kd=None, g_orm=None, g_nrm=None):
     _check(ctx, lib().adms_job_fold_gradients(ctx, job, ptr(g_kd), ptr(g_orm), ptr(g_nrm)))
+
+
+def adms_job_take_gradients(ctx, job, scale=None, g_pos=None, g_kd=None, g_orm=None, g_nrm=None, g_disp=None,
+                            g_skin_w=None):
+    _check(ctx, lib().adms_job_take_gradients(ctx, job, ptr(scale), ptr(g_pos), ptr(g_kd), ptr(g_orm), ptr(g_nrm),
+                                              ptr(g_disp), ptr(g_skin_w)))
 
 
 def adms_job_zero_gradients(ctx, job):

@@ -1853,24 +1853,70 @@ adms_status adms_job_fold_gradients(adms_ctx* ctx, adms_job job, float* g_kd, fl
     return ADMS_OK;
 }
 
-adms_status adms_job_zero_gradients(adms_ctx* ctx, adms_job job) {
-    Job* jp = get_job(ctx, job);
-    if (!jp) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
-    if (adms_status fs = flush_job(ctx, *jp)) return fs;  // its deferred texture step first
-    Job& j = *jp;
-    CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, ctx->stream));
+// zero a job's gradient buffers but for those that `taken` (bit 0 positions, 1 displacement,
+// 2 skin weights, 3 .. 5 textures) says are zero already
+static adms_status zero_gradients(adms_ctx* ctx, Job& j, unsigned taken) {
+    if (!(taken & 1u)) CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, ctx->stream));
     CK(cudaMemsetAsync(j.g_pos_acc, 0, sizeof(double) * 3 * j.V, ctx->stream));
     if (j.tess) {
         CK(cudaMemsetAsync(j.g_rpos, 0, sizeof(float) * 3 * j.V, ctx->stream));
         CK(cudaMemsetAsync(j.g_bpos_acc, 0, sizeof(double) * 3 * j.LV, ctx->stream));
     }
     if (j.skin) CK(cudaMemsetAsync(j.g_rpos, 0, sizeof(float) * 3 * j.V, ctx->stream));
-    if (j.g_skin_w) CK(cudaMemsetAsync(j.g_skin_w, 0, sizeof(float) * j.LV * j.SB, ctx->stream));
-    if (j.g_disp) CK(cudaMemsetAsync(j.g_disp, 0, sizeof(float) * j.dh * j.dw, ctx->stream));
+    if (j.g_skin_w && !(taken & 4u)) CK(cudaMemsetAsync(j.g_skin_w, 0, sizeof(float) * j.LV * j.SB, ctx->stream));
+    if (j.g_disp && !(taken & 2u)) CK(cudaMemsetAsync(j.g_disp, 0, sizeof(float) * j.dh * j.dw, ctx->stream));
     TexState* maps[3] = {&j.kd, &j.orm, &j.nrm};
     for (int m = 0; m < 3; ++m)
-        if (maps[m]->grad) CK(cudaMemsetAsync(maps[m]->grad, 0, sizeof(float4) * maps[m]->total, ctx->stream));
+        if (maps[m]->grad && !(taken & (8u << m)))
+            CK(cudaMemsetAsync(maps[m]->grad, 0, sizeof(float4) * maps[m]->total, ctx->stream));
     return ADMS_OK;
+}
+
+adms_status adms_job_zero_gradients(adms_ctx* ctx, adms_job job) {
+    Job* jp = get_job(ctx, job);
+    if (!jp) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
+    if (adms_status fs = flush_job(ctx, *jp)) return fs;  // its deferred texture step first
+    return zero_gradients(ctx, *jp, 0u);
+}
+
+adms_status adms_job_take_gradients(adms_ctx* ctx, adms_job job, const float* scale, float* g_pos, float* g_kd,
+                                    float* g_orm, float* g_nrm, float* g_disp, float* g_skin_w) {
+    Job* jp = get_job(ctx, job);
+    if (!jp) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
+    Job& j = *jp;
+    TexState* maps[3] = {&j.kd, &j.orm, &j.nrm};
+    float* outs[3] = {g_kd, g_orm, g_nrm};
+    for (int m = 0; m < 3; ++m)
+        if (outs[m] && !maps[m]->opt) return fail(ctx, ADMS_ERR_STATE, "texture is not optimized: no gradient");
+    if ((g_disp && !j.g_disp) || (g_skin_w && !j.g_skin_w))
+        return fail(ctx, ADMS_ERR_STATE, "displacement or skin weights are not optimized: no gradient");
+    if (adms_status fs = flush_job(ctx, j)) return fs;  // its deferred texture step first
+    unsigned taken = 0;
+    TexDev ts[3];
+    float4* to[3];
+    int n = 0;
+    for (int m = 0; m < 3; ++m) {
+        if (!outs[m]) continue;
+        TexDev t = maps[m]->dev();
+        if (maps[m]->per_level) t.levels = 1;  // level 0's own gradient; the chain is cleared below
+        else taken |= 8u << m;
+        ts[n] = t;
+        to[n++] = reinterpret_cast<float4*>(outs[m]);
+    }
+    CK(take_mip_gradients(ts, to, n, scale, ctx->stream));
+    FlatTake f{};
+    f.g[0] = j.g_pos;
+    f.out[0] = g_pos;
+    f.n[0] = g_pos ? (long long)j.LV * 3 : 0;
+    f.g[1] = j.g_disp;
+    f.out[1] = g_disp;
+    f.n[1] = g_disp ? (long long)j.dh * j.dw : 0;
+    f.g[2] = j.g_skin_w;
+    f.out[2] = g_skin_w;
+    f.n[2] = g_skin_w ? (long long)j.LV * j.SB : 0;
+    CK(take_flat_gradients(f, scale, ctx->stream));
+    taken |= (g_pos ? 1u : 0u) | (g_disp ? 2u : 0u) | (g_skin_w ? 4u : 0u);
+    return zero_gradients(ctx, j, taken);
 }
 
 adms_status adms_job_invalidate(adms_ctx* ctx, adms_job job) {

@@ -280,8 +280,18 @@ cudaError_t laplacian_backward(const LapArgs& a, cudaStream_t st);
 cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st);
 // a.g_pos = scale * dL_delta/dpos (overwrites) after laplacian_forward
 cudaError_t laplacian_gradient(const LapArgs& a, float scale, cudaStream_t st);
+#define ADMS_MIP_TEX 3  // textures per fold or rebuild launch (a job's maps)
 // level-0 texture gradient with the mip-chain adjoint folded in
 cudaError_t fold_mip_gradient(const TexDev& t, float4* out, cudaStream_t st);
+// the same for n <= 3 textures, times *scale (null: 1), the gradient chains then zero
+cudaError_t take_mip_gradients(const TexDev* ts, float4* const* outs, int n, const float* scale, cudaStream_t st);
+// out[k][0 .. n[k]) = g[k] times *scale (null: 1), g[k] = 0
+struct FlatTake {
+    float* g[3];
+    float* out[3];
+    long long n[3];
+};
+cudaError_t take_flat_gradients(const FlatTake& a, const float* scale, cudaStream_t st);
 
 struct SchedArgs {
     JobState* st;

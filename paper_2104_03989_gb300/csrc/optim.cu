@@ -637,18 +637,33 @@ cudaError_t adam_texture_and_mips(const TexDev& t, float4* m, float4* v, int cla
 // share every coarser texel: the levels' loads are issued together and reused four times, and
 // the levels' weights come as parameters. One texel per thread with its index divisions and
 // the weights rebuilt per level took 58.7 us for a 1024^2 map and 257 us for a 2048^2 one.
-struct FoldWeights {
-    float w[ADMS_MAX_LEVELS];
+//
+// With `take`, the written gradient is also multiplied by *scale (when given) and the read one
+// cleared: an autograd backward hands out dL/d(texture) = its incoming gradient times the
+// job's and leaves the job's buffers at zero, in the pass that reads them.
+struct FoldBatch {
+    TexDev t[ADMS_MIP_TEX];
+    float4* out[ADMS_MIP_TEX];
+    float w[ADMS_MIP_TEX][ADMS_MAX_LEVELS];
+    int block0[ADMS_MIP_TEX];
+    int n;
+    const float* scale;
+    int take;
 };
-__global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ TexDev t, const FoldWeights fw,
-                                                   float4* __restrict__ out) {
-    int x = 2 * (blockIdx.x * 32 + (threadIdx.x & 31)), y = 2 * (blockIdx.y * 8 + (threadIdx.x >> 5));
+__global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ FoldBatch P) {
+    int e = 0, block = blockIdx.x;
+    while (e + 1 < P.n && P.block0[e + 1] <= block) ++e;
+    const TexDev& t = P.t[e];
+    block -= P.block0[e];
+    int nbx = (t.w0 + 63) / 64;
+    int x = 2 * ((block % nbx) * 32 + (threadIdx.x & 31)), y = 2 * ((block / nbx) * 8 + (threadIdx.x >> 5));
     if (x >= t.w0 || y >= t.h0) return;
     bool bx = x + 1 < t.w0, by = y + 1 < t.h0;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     size_t i = (size_t)y * t.w0 + x;
     float4 g[4] = {t.grad[i], bx ? t.grad[i + 1] : zero, by ? t.grad[i + t.w0] : zero,
                    bx && by ? t.grad[i + t.w0 + 1] : zero};
+    float scale = P.scale ? *P.scale : 1.f;
 #pragma unroll
     for (int k0 = 1; k0 < ADMS_MAX_LEVELS; k0 += 5) {  // five levels' loads in flight at a time
         if (k0 >= t.levels) break;
@@ -662,23 +677,74 @@ __global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ TexDe
         for (int j = 0; j < 5; ++j)
             if (k0 + j < t.levels) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) g[q] = f4madd(g[q], fw.w[k0 + j], c[j]);
+                for (int q = 0; q < 4; ++q) g[q] = f4madd(g[q], P.w[e][k0 + j], c[j]);
             }
     }
-    out[i] = g[0];
-    if (bx) out[i + 1] = g[1];
-    if (by) out[i + t.w0] = g[2];
-    if (bx && by) out[i + t.w0 + 1] = g[3];
+    float4* out = P.out[e];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if ((q & 1 && !bx) || (q & 2 && !by)) continue;
+        size_t o = i + (q & 1) + (q & 2 ? t.w0 : 0);
+        out[o] = P.scale ? f4scale(g[q], scale) : g[q];
+        if (P.take) t.grad[o] = zero;
+    }
+}
+
+static cudaError_t fold_batch(const TexDev* ts, float4* const* outs, int n, const float* scale, bool take,
+                              cudaStream_t st) {
+    FoldBatch P;
+    P.n = n;
+    P.scale = scale;
+    P.take = take;
+    int blocks = 0;
+    for (int j = 0; j < n; ++j) {
+        const TexDev& t = ts[j];
+        P.t[j] = t;
+        P.out[j] = outs[j];
+        P.block0[j] = blocks;
+        blocks += ((t.w0 + 63) / 64) * ((t.h0 + 15) / 16);
+        P.w[j][0] = 1.f;
+        // the share of a level-k texel in each of its level-0 texels: the 2x2 / 2x1 box factors down the chain
+        for (int k = 1; k < ADMS_MAX_LEVELS; ++k)
+            P.w[j][k] = P.w[j][k - 1] / (float)(((t.w0 >> (k - 1)) > 1 ? 2 : 1) * ((t.h0 >> (k - 1)) > 1 ? 2 : 1));
+    }
+    if (n <= 0) return cudaSuccess;
+    k_fold_mips<<<blocks, 256, 0, st>>>(P);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 cudaError_t fold_mip_gradient(const TexDev& t, float4* out, cudaStream_t st) {
-    FoldWeights fw;
-    fw.w[0] = 1.f;
-    // the share of a level-k texel in each of its level-0 texels: the 2x2 / 2x1 box factors down the chain
-    for (int k = 1; k < ADMS_MAX_LEVELS; ++k)
-        fw.w[k] = fw.w[k - 1] / (float)(((t.w0 >> (k - 1)) > 1 ? 2 : 1) * ((t.h0 >> (k - 1)) > 1 ? 2 : 1));
-    dim3 grid((t.w0 + 63) / 64, (t.h0 + 15) / 16);
-    k_fold_mips<<<grid, 256, 0, st>>>(t, fw, out);
+    return fold_batch(&t, &out, 1, nullptr, false, st);
+}
+cudaError_t take_mip_gradients(const TexDev* ts, float4* const* outs, int n, const float* scale, cudaStream_t st) {
+    cudaError_t e = fold_batch(ts, outs, n, scale, true, st);
+    for (int j = 0; j < n && !e; ++j) {  // the coarser levels, once every reader is done
+        const TexDev& t = ts[j];
+        if (t.levels <= 1) continue;
+        int last = t.levels - 1;
+        size_t end = t.off[last] + (size_t)max(t.w0 >> last, 1) * max(t.h0 >> last, 1);
+        e = cudaMemsetAsync(t.grad + t.off[1], 0, (end - t.off[1]) * sizeof(float4), st);
+    }
+    return e;
+}
+
+// out = scale g, g = 0 over up to three flat gradients (positions, displacement, skin weights)
+__global__ void k_take_flat(const FlatTake a, const float* scale) {
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (i >= 0 && i < a.n[k]) {
+            a.out[k][i] = scale ? a.g[k][i] * *scale : a.g[k][i];
+            a.g[k][i] = 0.f;
+        }
+        i -= a.n[k];
+    }
+}
+cudaError_t take_flat_gradients(const FlatTake& a, const float* scale, cudaStream_t st) {
+    long long n = a.n[0] + a.n[1] + a.n[2];
+    if (n <= 0) return cudaSuccess;
+    k_take_flat<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, scale);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -712,7 +778,6 @@ __global__ void k_mip_level(float4* __restrict__ tex, int src_off, int ws, int h
 // thread's quad and the shuffles as in k_adam_tex_stream: level 0 is read once and nothing of
 // the chain is read back (HBM bound: 16 B per level-0 texel in, 5.3 out). A launch per level
 // took 36 us for a 1024^2 map (ten launches), three maps 110 us.
-#define ADMS_MIP_TEX 3
 struct MipBatch {
     TexDev t[ADMS_MIP_TEX];
     int tile0[ADMS_MIP_TEX];
