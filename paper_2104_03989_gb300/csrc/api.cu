@@ -171,10 +171,9 @@ struct BatchState {
 
 struct adms_ctx {
     cudaStream_t stream = 0;
-    // a second stream for the independent branches of a call (the vertex frame and
-    // the Laplacian beside the raster, the flat latents' Adam beside the textures'),
-    // forked from and joined back into `stream` within the call, so that a graph
-    // captured on `stream` holds both
+    // a second stream for the independent branches of a call (the flat latents' Adam beside
+    // the textures'), forked from and joined back into `stream` within the call, so that a
+    // graph captured on `stream` holds both
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // pipelined optimizer steps (adms_ctx_set_pipelining): a job's texture step is
@@ -551,35 +550,29 @@ SkinArgs skin_args(Job& j) {
     return a;
 }
 
-// The render positions (tessellated, skinned) on the context's stream, then the
-// vertex frame and, once per set of positions, the Laplacian on a branch beside
-// the raster: both need only the positions. *forked tells the caller to join the
-// branch before the shading.
-adms_status frame_branch(adms_ctx* ctx, Job& j, bool* forked) {
-    *forked = false;
-    if (j.frame_valid) return ADMS_OK;
-    if (j.tess) CK(TIMED(ST_FRAME, tess_forward(tess_args(j), ctx->stream)));
-    if (j.skin) CK(TIMED(ST_FRAME, skin_forward(skin_args(j), ctx->stream)));
-    cudaError_t e;
-    cudaStream_t bs = fork_branch(ctx, e);
-    CK(e);
-    *forked = true;
-    CK(TIMED(ST_FRAME, frame_forward(frame_args(j), bs)));
-    if (j.opt.optimize_pos && !j.lap_valid) {
-        CK(TIMED(ST_LAPLACIAN, laplacian_forward(lap_args(j), bs)));
-        j.lap_valid = true;
+// The render positions (tessellated, skinned) on the context's stream, and the raster's
+// preparation of a job whose views are in j.views: with the vertex frame and, once per set of
+// positions, the Laplacian where they are due. clear_grads: what a backward accumulates into
+// is cleared on the way, the render positions' gradient too.
+adms_status prep_job(adms_ctx* ctx, Job& j, bool clear_grads, bool clear_loss, PrepJob& p) {
+    if (!j.frame_valid) {
+        if (j.tess) CK(TIMED(ST_FRAME, tess_forward(tess_args(j), ctx->stream)));
+        if (j.skin) CK(TIMED(ST_FRAME, skin_forward(skin_args(j), ctx->stream)));
+        p.frame = true;
+        p.f = frame_args(j);
+        if (j.opt.optimize_pos && !j.lap_valid) {
+            p.lap = true;
+            p.l = lap_args(j);
+            p.add_clear(&j.st->lap_sum, sizeof(double));
+        }
     }
-    j.frame_valid = true;
-    return ADMS_OK;
-}
-
-// join_late: the context's stream waits for the late stream (the job's deferred
-// texture step) before the shading, the first kernel that reads the textures
-adms_status render_core(adms_ctx* ctx, Job& j, bool join_late = false) {
-    bool forked = false;
-    adms_status fs = frame_branch(ctx, j, &forked);
-    if (fs) return fs;
-    RasterIn in;
+    if (clear_loss) p.add_clear(&j.st->call_loss, sizeof(double));
+    if (clear_grads) {
+        p.add_clear(j.g_nrm, sizeof(double) * 6 * j.V);  // g_nrm and g_tan
+        if (j.tess || j.skin) p.add_clear(j.g_rpos, sizeof(float) * 3 * j.V);
+    }
+    p.s = &j.rs;
+    RasterIn& in = p.in;
     in.pos = j.rpos;
     in.tri = j.tri;
     in.adj = j.adj;
@@ -590,22 +583,34 @@ adms_status render_core(adms_ctx* ctx, Job& j, bool join_late = false) {
     in.W = j.W;
     in.H = j.H;
     in.keys = j.keys;
+    // depth peeling: all L layers in one tile pass (a k-buffer per sample), every triangle binned
+    in.small_px = j.L > 0 ? 0 : j.opt.raster_direct_px > 0 ? j.opt.raster_direct_px : ADMS_SMALL_PX;
+    in.zfilter = j.opt.raster_depth_filter;
+    return ADMS_OK;
+}
+
+// join_late: the context's stream waits for the late stream (the job's deferred
+// texture step) before the shading, the first kernel that reads the textures
+// after the launch of a job's preparation
+void prepared(Job& j, const PrepJob& p) {
+    if (p.frame) j.frame_valid = true;
+    if (p.lap) j.lap_valid = true;
+}
+
+adms_status render_core(adms_ctx* ctx, Job& j, bool clear_grads = false, bool clear_loss = false,
+                        bool join_late = false) {
+    PrepJob p;
+    adms_status ps = prep_job(ctx, j, clear_grads, clear_loss, p);
+    if (ps) return ps;
+    CK(TIMED(ST_RASTER_SETUP, raster_prepare(&p, 1, ctx->stream)));
+    prepared(j, p);
+    if (j.L > 0) CK(TIMED(ST_RASTER, raster_tiles_peeled(p.in, j.rs, j.L, ctx->stream)));
+    else CK(TIMED(ST_RASTER, raster_tiles(p.in, j.rs, ctx->stream)));
+    if (join_late) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_late_join, 0));
     if (j.L > 0) {
-        // all L peeling layers in one tile pass (a k-buffer per sample): every triangle binned
-        in.small_px = 0;
-        CK(TIMED(ST_RASTER_SETUP, raster_prepare(in, j.rs, ctx->stream)));
-        CK(TIMED(ST_RASTER, raster_tiles_peeled(in, j.rs, j.L, ctx->stream)));
-        if (forked) CK(join_branch(ctx));
-        if (join_late) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_late_join, 0));
         for (int l = 0; l < j.L; ++l) CK(TIMED(ST_SHADE, shade_forward(layer_args(j, l), ctx->stream)));
         return ADMS_OK;
     }
-    in.small_px = j.opt.raster_direct_px > 0 ? j.opt.raster_direct_px : ADMS_SMALL_PX;
-    in.zfilter = j.opt.raster_depth_filter;
-    CK(TIMED(ST_RASTER_SETUP, raster_prepare(in, j.rs, ctx->stream)));
-    CK(TIMED(ST_RASTER, raster_tiles(in, j.rs, ctx->stream)));
-    if (forked) CK(join_branch(ctx));
-    if (join_late) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_late_join, 0));
     CK(TIMED(ST_SHADE, shade_forward(shade_args(j), ctx->stream)));
     return ADMS_OK;
 }
@@ -937,31 +942,6 @@ adms_status job_create_impl(adms_ctx* ctx, const adms_mesh_desc* mesh, const adm
     return ADMS_OK;
 }
 
-// frame (and tessellation) plus the per-job raster preparation of a batched call
-// frame_branch and the raster setup of one job of a batch (*forked: join before
-// the batch's shading)
-adms_status frame_and_prepare(adms_ctx* ctx, Job& j, bool* forked) {
-    bool f = false;
-    adms_status fs = frame_branch(ctx, j, &f);
-    if (fs) return fs;
-    *forked = *forked || f;
-    RasterIn in;
-    in.pos = j.rpos;
-    in.tri = j.tri;
-    in.adj = j.adj;
-    in.views = j.views;
-    in.B = j.B;
-    in.V = j.V;
-    in.F = j.F;
-    in.W = j.W;
-    in.H = j.H;
-    in.keys = j.keys;
-    in.small_px = j.opt.raster_direct_px > 0 ? j.opt.raster_direct_px : ADMS_SMALL_PX;
-    in.zfilter = j.opt.raster_depth_filter;
-    CK(TIMED(ST_RASTER_SETUP, raster_prepare(in, j.rs, ctx->stream)));
-    return ADMS_OK;
-}
-
 template <typename T>
 adms_status batch_alloc(adms_ctx* ctx, BatchState& bs, T** out, size_t count) {
     size_t bytes = ((std::max<size_t>(count, 1) * sizeof(T)) + 255) & ~size_t(255);
@@ -1219,7 +1199,7 @@ static adms_status flush_job(adms_ctx* ctx, Job& j) {
     j.tex_pending = false;
     adms_status s = texture_adams(ctx, {&j}, ctx->stream);
     if (s) return s;
-    CK(TIMED(ST_SMALL, advance_step(j.st, ctx->stream)));
+    CK(TIMED(ST_SMALL, advance_step(&j.st, 1, ctx->stream)));
     return ADMS_OK;
 }
 static adms_status flush_all(adms_ctx* ctx) {
@@ -1244,7 +1224,7 @@ static adms_status fork_texture_step(adms_ctx* ctx, Job& j, bool* forked) {
     CK(cudaStreamWaitEvent(ctx->late, ctx->ev_late_fork, 0));
     adms_status s = texture_adams(ctx, {&j}, ctx->late);
     if (s) return s;
-    CK(advance_step(j.st, ctx->late));
+    CK(advance_step(&j.st, 1, ctx->late));
     CK(cudaEventRecord(ctx->ev_late_join, ctx->late));
     *forked = true;
     return ADMS_OK;
@@ -1637,8 +1617,8 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
     if (!ctx || !jobs || n_jobs <= 0 || !views || !views_per_job || !hw || !ref_rgb)
         return fail(ctx, ADMS_ERR_ARG, "invalid forward_loss arguments");
     size_t vofs = 0;
-    bool forked = false;  // a batch's frame branches, joined before its shading
     std::vector<Job*> js;
+    std::vector<PrepJob> preps(n_jobs > 1 ? n_jobs : 0);
     for (int k = 0; k < n_jobs; ++k) {
         Job* jp = get_job(ctx, jobs[k]);
         int B = views_per_job[k], H = hw[2 * k], W = hw[2 * k + 1];
@@ -1665,11 +1645,10 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
         j.loss_scale = (float)(1.0 / (3.0 * (double)norm_views * H * W));
         CK(cudaMemcpyAsync(j.views, views + vofs, sizeof(adms_view) * B, cudaMemcpyDefault, ctx->stream));
         vofs += B;
-        CK(cudaMemsetAsync(&j.st->call_loss, 0, sizeof(double), ctx->stream));
         if (n_jobs == 1) {
             bool late = false;  // the job's deferred texture step runs beside its frame and raster
             if ((s = fork_texture_step(ctx, j, &late))) return s;
-            if ((s = render_core(ctx, j, late))) return s;
+            if ((s = render_core(ctx, j, true, true, late))) return s;
             CK(wait_ref(ctx));
             if (j.L > 0) {
                 if ((s = peel_composite(ctx, j, j.ref, &j.st->call_loss, out_img ? out_img[k] : nullptr))) return s;
@@ -1684,28 +1663,29 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
             }
         } else {
             if ((s = flush_job(ctx, j))) return s;
-            if ((s = frame_and_prepare(ctx, j, &forked))) return s;
+            if ((s = prep_job(ctx, j, true, true, preps[k]))) return s;
         }
     }
     if (n_jobs > 1) {
-        // one persistent launch per stage over the tiles of every job and view
+        // one launch per stage over every job (the pixel stages over the tiles of every job and view)
         BatchState* bsp = nullptr;
         adms_status s = batch_upload(ctx, js, out_img, &bsp);
         if (s) return s;
         BatchState& bs = *bsp;
+        CK(TIMED(ST_RASTER_SETUP, raster_prepare(preps.data(), n_jobs, ctx->stream)));
+        for (int k = 0; k < n_jobs; ++k) prepared(*js[k], preps[k]);
         CK(TIMED(ST_RASTER, raster_tiles_batched(bs.h_rargs.data(), bs.rt_off.data(), n_jobs, bs.d_rt,
                                                  batch_grid(ctx, 3), ctx->stream)));
-        if (forked) CK(join_branch(ctx));
         CK(TIMED(ST_SHADE, pixels_batched(0, bs.h_args.data(), bs.px_off.data(), n_jobs, bs.d_px, ctx->tune_tw,
                                           batch_grid(ctx, 0), ctx->stream)));
         CK(wait_ref(ctx));
         CK(TIMED(ST_AA_LOSS, pixels_batched(1, bs.h_args.data(), bs.px_off.data(), n_jobs, bs.d_px, ctx->tune_tw,
                                             batch_grid(ctx, 1), ctx->stream)));
     }
-    for (int k = 0; k < n_jobs; ++k) {
-        CK(TIMED(ST_SMALL, finish_call_loss(js[k]->st, out_loss ? out_loss + k : nullptr, ctx->stream)));
-        js[k]->have_fwd = true;
-    }
+    std::vector<JobState*> sts;
+    for (Job* jp : js) sts.push_back(jp->st);
+    CK(TIMED(ST_SMALL, finish_call_loss(sts.data(), n_jobs, out_loss, ctx->stream)));
+    for (Job* jp : js) jp->have_fwd = true;
     return ADMS_OK;
 }
 
@@ -1724,7 +1704,7 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
         if (recompute_raster) {
             // rebuild keys, pre-AA colours and dL/d(AA colour) from the latents and the
             // caller's reference images instead of reading what the forward kept
-            adms_status s = render_core(ctx, j);
+            adms_status s = render_core(ctx, j, true);
             if (s) return s;
             CK(wait_ref(ctx));
             if (j.L > 0) {
@@ -1738,8 +1718,7 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
                 CK(TIMED(ST_AA_LOSS, aa_loss_forward(r, ctx->stream)));
             }
         }
-        CK(cudaMemsetAsync(j.g_nrm, 0, sizeof(double) * 6 * j.V, ctx->stream));  // g_nrm and g_tan
-        if (j.tess || j.skin) CK(cudaMemsetAsync(j.g_rpos, 0, sizeof(float) * 3 * j.V, ctx->stream));
+        // (the forward, or the recomputation above, cleared g_nrm, g_tan and g_rpos: prep_job)
         if (n_jobs == 1 && j.L > 0) {
             adms_status s = peel_backward(ctx, j);
             if (s) return s;
@@ -1757,9 +1736,11 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
         CK(TIMED(ST_SHADE_BWD, pixels_batched(2, bs.h_args.data(), bs.px_off.data(), n_jobs, bs.d_px, ctx->tune_tw,
                                               batch_grid(ctx, 2), ctx->stream)));
     }
+    std::vector<FrameArgs> frames;
+    for (Job* jp : js) frames.push_back(frame_args(*jp));
+    CK(TIMED(ST_FRAME_BWD, frame_backward(frames.data(), n_jobs, ctx->stream)));
     for (int k = 0; k < n_jobs; ++k) {
         Job& j = *js[k];
-        CK(TIMED(ST_FRAME_BWD, frame_backward(frame_args(j), ctx->stream)));
         if (j.tess) {
             // render positions -> base positions, base normals and displacement texels,
             // then the base normals' adjoint back to base positions
@@ -1792,26 +1773,27 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
     // weights, displacement) on a branch beside the textures: every job's tiled
     // textures in one launch; then, joined, the step counters. A pipelined context
     // issues the flat latents' updates here and defers the texture step.
+    std::vector<SchedArgs> sched;
+    std::vector<PosStepArgs> poss;
+    std::vector<JobState*> sts;
     for (Job* jp : js) {
         Job& j = *jp;
         if (j.opt.optimize_pos && !j.lap_valid) CK(TIMED(ST_LAPLACIAN, laplacian_forward(lap_args(j), ctx->stream)));
-        SchedArgs sa{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV};
-        CK(TIMED(ST_SMALL, schedule_step(sa, ctx->stream)));
+        sched.push_back(SchedArgs{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV});
+        if (j.opt.optimize_pos) poss.push_back(PosStepArgs{lap_args(j), j.pos, j.m_pos, j.v_pos});
+        sts.push_back(j.st);
     }
+    CK(TIMED(ST_SMALL, schedule_step(sched.data(), n_jobs, ctx->stream)));
     cudaStream_t bs = ctx->stream;
     if (!ctx->pipeline) {
         cudaError_t fe;
         bs = fork_branch(ctx, fe);
         CK(fe);
     }
+    if (!poss.empty()) CK(TIMED(ST_LAPLACIAN, position_step(poss.data(), (int)poss.size(), bs)));
     for (Job* jp : js) {
         Job& j = *jp;
-        if (j.opt.optimize_pos) {
-            CK(TIMED(ST_LAPLACIAN, laplacian_backward(lap_args(j), bs)));
-            CK(TIMED(ST_ADAM, adam_flat(j.pos, j.g_pos, j.m_pos, j.v_pos, (long long)j.LV * 3, j.st, bs)));
-        } else {
-            CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, bs));
-        }
+        if (!j.opt.optimize_pos) CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, bs));
         if (j.g_skin_w)
             CK(TIMED(ST_ADAM, adam_flat(j.skin_w, j.g_skin_w, j.m_skin_w, j.v_skin_w, (long long)j.LV * j.SB, j.st,
                                         bs, j.skin_lr_scale)));
@@ -1831,7 +1813,7 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
     adms_status s = texture_adams(ctx, js, ctx->stream);
     if (s) return s;
     CK(join_branch(ctx));
-    for (Job* jp : js) CK(TIMED(ST_SMALL, advance_step(jp->st, ctx->stream)));
+    CK(TIMED(ST_SMALL, advance_step(sts.data(), n_jobs, ctx->stream)));
     return ADMS_OK;
 }
 

@@ -16,6 +16,43 @@ namespace adms {
 inline std::atomic<long long> g_launches{0};
 inline void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+// Arguments of one launch over N jobs (blockIdx.y the job): a batched call's small per-job
+// kernels go out together, up to ADMS_BATCH_JOBS jobs' arguments in the parameter space (32 KB).
+template <typename A, int N>
+struct Pack {
+    A a[N];
+};
+#define ADMS_BATCH_JOBS 60
+// one launch for n arguments (kernel k1 for a single one, kn per ADMS_BATCH_JOBS otherwise),
+// grid.x the largest blocks(args)
+template <typename A, typename K1, typename KN, typename F>
+cudaError_t launch_packed(const A* args, int n, int threads, cudaStream_t st, K1 k1, KN kn, F blocks) {
+    static_assert(sizeof(Pack<A, ADMS_BATCH_JOBS>) <= 32764, "batched launch parameters exceed the kernel parameter space");
+    if (n == 1) {
+        Pack<A, 1> p;
+        p.a[0] = args[0];
+        int b = blocks(args[0]);
+        if (b <= 0) return cudaSuccess;
+        k1<<<b, threads, 0, st>>>(p);
+        count_launches(1);
+        return cudaGetLastError();
+    }
+    for (int j0 = 0; j0 < n; j0 += ADMS_BATCH_JOBS) {
+        Pack<A, ADMS_BATCH_JOBS> p;
+        int m = std::min(n - j0, ADMS_BATCH_JOBS), b = 0;
+        for (int j = 0; j < m; ++j) {
+            p.a[j] = args[j0 + j];
+            b = std::max(b, (int)blocks(p.a[j]));
+        }
+        if (b <= 0) continue;
+        kn<<<dim3(b, m), threads, 0, st>>>(p);
+        count_launches(1);
+        cudaError_t e = cudaGetLastError();
+        if (e) return e;
+    }
+    return cudaSuccess;
+}
+
 // transformed vertex of one view: snapped sub-pixel position, depth, usable flag
 struct VtxS {
     int X, Y;
@@ -75,8 +112,8 @@ struct RasterScratch {
 };
 
 cudaError_t raster_views(const RasterIn& in, RasterScratch& s, cudaStream_t st);
-// transform, setup, tile counts, scan and tile lists (in.keys may be null when
-// in.small_px is 0: nothing is then rasterized directly and the keys are untouched)
+// transform, setup, tile counts, list allocation and tile lists; with in.small_px = 0 nothing
+// is rasterized directly and the keys are untouched (in.keys may be null)
 cudaError_t raster_prepare(const RasterIn& in, RasterScratch& s, cudaStream_t st);
 // the per-tile z-buffer pass
 cudaError_t raster_tiles(const RasterIn& in, RasterScratch& s, cudaStream_t st);
@@ -152,10 +189,9 @@ cudaError_t resolve_loss(const ResolveArgs& r, cudaStream_t st);
 struct WorkItem {
     int job, view, x0, y0;
 };
-// Jobs per batched launch: their arguments travel in the launch's parameter
-// space (60 x 536 B, under the 32 KB limit), read-only and captured with the
+// Jobs per batched launch (ADMS_BATCH_JOBS): their arguments travel in the launch's
+// parameter space (60 x 536 B, under the 32 KB limit), read-only and captured with the
 // launch by a graph; larger job sets take one launch per 60 jobs.
-#define ADMS_BATCH_JOBS 60
 struct ShadeBatch {
     ShadeArgs a[ADMS_BATCH_JOBS];
 };
@@ -214,6 +250,8 @@ struct FrameArgs {
 };
 cudaError_t frame_forward(const FrameArgs& a, cudaStream_t st);
 cudaError_t frame_backward(const FrameArgs& a, cudaStream_t st);
+// of n jobs whose forward kept the normalisations (inv set), one launch
+cudaError_t frame_backward(const FrameArgs* as, int n, cudaStream_t st);
 
 // tessellation + displacement (latent base mesh -> render mesh) and its adjoint
 // dense skinning (Eq. 2) of the rest positions by the frame's bones
@@ -275,7 +313,25 @@ struct LapArgs {
     JobState* st;
 };
 cudaError_t laplacian_forward(const LapArgs& a, cudaStream_t st);
-cudaError_t laplacian_backward(const LapArgs& a, cudaStream_t st);
+
+// raster_prepare of n jobs, one launch per stage: the first also clears buffers the caller
+// names, the last also forms the vertex frames and Laplacians that are due
+#define ADMS_PREP_CLEARS 4
+struct PrepJob {
+    RasterIn in;
+    RasterScratch* s;
+    bool frame = false, lap = false;
+    FrameArgs f;
+    LapArgs l;  // st->lap_sum is cleared
+    void* clear[ADMS_PREP_CLEARS];       // 4-byte aligned
+    size_t clear_bytes[ADMS_PREP_CLEARS];  // multiples of 4
+    int n_clear = 0;
+    void add_clear(void* p, size_t bytes) {
+        clear[n_clear] = p;
+        clear_bytes[n_clear++] = bytes;
+    }
+};
+cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st);
 // *out = L_delta after laplacian_forward
 cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st);
 // a.g_pos = scale * dL_delta/dpos (overwrites) after laplacian_forward
@@ -299,7 +355,14 @@ struct SchedArgs {
     int has_pos;
     int n_verts;
 };
-cudaError_t schedule_step(const SchedArgs& a, cudaStream_t st);
+cudaError_t schedule_step(const SchedArgs* as, int n, cudaStream_t st);
+
+// the positions' step: g += lambda_t dL_delta/dpos (Eq. 4), Adam (no clamps), g = 0
+struct PosStepArgs {
+    LapArgs lap;
+    float *p, *m, *v;  // [V][3]
+};
+cudaError_t position_step(const PosStepArgs* as, int n, cudaStream_t st);
 
 // Adam on a flat float array (positions, displacement): no clamps
 cudaError_t adam_flat(float* p, float* g, float* m, float* v, long long n, const JobState* js, cudaStream_t st,
@@ -345,11 +408,11 @@ cudaError_t adam_encode_maps(const TexDev& t, const float4* m, const float4* v, 
 // Adam + mip rebuild of every listed texture (all adam_tiled, any jobs), one 32x32-texel
 // tile per block, one launch per ADMS_ADAM_TEX textures
 cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uint32_t extra_tx = 0);
-cudaError_t advance_step(JobState* js, cudaStream_t st);
+cudaError_t advance_step(JobState* const* js, int n, cudaStream_t st);
 // out[k] = the latched status of job k (stream-ordered; out: device [n])
 #define ADMS_STATUS_MAX 512
 cudaError_t gather_status(JobState* const* js, int n, int* out, cudaStream_t st);
-// out[j] = call_loss; img_loss += call_loss
-cudaError_t finish_call_loss(JobState* js, float* out, cudaStream_t st);
+// per job: out[k] = call_loss (out may be null); img_loss += call_loss
+cudaError_t finish_call_loss(JobState* const* js, int n, float* out, cudaStream_t st);
 
 }  // namespace adms

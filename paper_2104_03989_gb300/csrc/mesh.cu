@@ -4,75 +4,13 @@
 //
 // Both run one thread per vertex and gather over a vertex -> face (or one-ring)
 // CSR table, so results do not depend on atomic ordering.
-#include "kernels.cuh"
+#include "mesh.cuh"
 
 namespace adms {
 
-struct FaceFrame {
-    float3 e1, e2, fn, tv;
-    float d1y, d2y;
-    int sgn;
-    int idx[3];
-};
-
-__device__ __forceinline__ FaceFrame face_frame(const FrameArgs& a, int f) {
-    FaceFrame r;
-    int i0 = a.tri[3 * f], i1 = a.tri[3 * f + 1], i2 = a.tri[3 * f + 2];
-    r.idx[0] = i0;
-    r.idx[1] = i1;
-    r.idx[2] = i2;
-    float3 p0 = f3(a.pos[3 * i0], a.pos[3 * i0 + 1], a.pos[3 * i0 + 2]);
-    float3 p1 = f3(a.pos[3 * i1], a.pos[3 * i1 + 1], a.pos[3 * i1 + 2]);
-    float3 p2 = f3(a.pos[3 * i2], a.pos[3 * i2 + 1], a.pos[3 * i2 + 2]);
-    float2 u0 = a.uv[a.tri_uv[3 * f]], u1 = a.uv[a.tri_uv[3 * f + 1]], u2 = a.uv[a.tri_uv[3 * f + 2]];
-    r.e1 = p1 - p0;
-    r.e2 = p2 - p0;
-    r.fn = cross3(r.e1, r.e2);
-    float d1x = u1.x - u0.x, d2x = u2.x - u0.x;
-    r.d1y = u1.y - u0.y;
-    r.d2y = u2.y - u0.y;
-    float det = d1x * r.d2y - d2x * r.d1y;
-    r.sgn = det > 0.f ? 1 : (det < 0.f ? -1 : 0);
-    r.tv = r.d2y * r.e1 - r.d1y * r.e2;
-    return r;
-}
-
-// The gathers over a vertex's faces (or one-ring) run in batches of ADMS_GATHER:
-// the batch's loads are issued together (the last entry repeated past the end)
-// and summed in list order, so each sum keeps the order of a plain loop while the
-// dependent loads of a vertex take ceil(valence / ADMS_GATHER) round trips
-// instead of one per face.
-#define ADMS_GATHER 4
-
-// unnormalised vertex normal (sum of face normals) and tangent (sum of signed unit face tangents)
-__device__ __forceinline__ void vertex_sums(const FrameArgs& a, int v, float3& n, float3& t) {
-    n = zero3();
-    t = zero3();
-    int lo = a.vf_off[v], hi = a.vf_off[v + 1];
-    for (int j0 = lo; j0 < hi; j0 += ADMS_GATHER) {
-        FaceFrame ff[ADMS_GATHER];
-#pragma unroll
-        for (int q = 0; q < ADMS_GATHER; ++q) ff[q] = face_frame(a, a.vf_face[min(j0 + q, hi - 1)]);
-#pragma unroll
-        for (int q = 0; q < ADMS_GATHER; ++q) {
-            if (j0 + q < hi) {
-                n += ff[q].fn;
-                if (ff[q].sgn != 0) t += (float)ff[q].sgn * nrm3(ff[q].tv).y;
-            }
-        }
-    }
-}
-
 __global__ void k_frame_fwd(FrameArgs a) {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= a.V) return;
-    float3 n, t;
-    vertex_sums(a, v, n, t);
-    Nrm3 nn = nrm3(n), tn = nrm3(t);
-    a.vpos[v] = make_float4(a.pos[3 * v], a.pos[3 * v + 1], a.pos[3 * v + 2], 0.f);
-    a.vnrm[v] = make_float4(nn.y.x, nn.y.y, nn.y.z, 0.f);
-    a.vtan[v] = make_float4(tn.y.x, tn.y.y, tn.y.z, 0.f);
-    if (a.inv) a.inv[v] = make_float2(nn.big ? nn.inv : -nn.inv, tn.big ? tn.inv : -tn.inv);
+    if (v < a.V) frame_vertex(a, v);
 }
 
 // the normalisation of vertex c's normal (k = 0) or tangent (k = 1) sum as the
@@ -157,7 +95,9 @@ __global__ void k_frame_bwd2(FrameArgs a) {
 // incident faces s, s + 8, ... and forming their corners' normalisation adjoints
 // itself; the slots' sums are combined by shuffles in a fixed order
 #define ADMS_FRAME_SLOTS 8
-__global__ void k_frame_bwd_fused(FrameArgs a) {
+template <int N>
+__global__ void __launch_bounds__(128) k_frame_bwd_fused(const __grid_constant__ Pack<FrameArgs, N> P) {
+    const FrameArgs& a = P.a[N == 1 ? 0 : blockIdx.y];
     int gid = blockIdx.x * blockDim.x + threadIdx.x;
     int v = gid / ADMS_FRAME_SLOTS, slot = gid % ADMS_FRAME_SLOTS;
     bool valid = v < a.V;
@@ -195,12 +135,13 @@ cudaError_t frame_forward(const FrameArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+cudaError_t frame_backward(const FrameArgs* as, int n, cudaStream_t st) {
+    return launch_packed(as, n, 128, st, k_frame_bwd_fused<1>, k_frame_bwd_fused<ADMS_BATCH_JOBS>,
+                         [](const FrameArgs& a) { return (a.V * ADMS_FRAME_SLOTS + 127) / 128; });
+}
+
 cudaError_t frame_backward(const FrameArgs& a, cudaStream_t st) {
-    if (a.inv) {
-        k_frame_bwd_fused<<<(a.V * ADMS_FRAME_SLOTS + 127) / 128, 128, 0, st>>>(a);
-        count_launches(1);
-        return cudaGetLastError();
-    }
+    if (a.inv) return frame_backward(&a, 1, st);
     k_frame_bwd1<<<(a.V + 127) / 128, 128, 0, st>>>(a);
     k_frame_bwd2<<<(a.V + 127) / 128, 128, 0, st>>>(a);
     count_launches(2);
@@ -210,65 +151,7 @@ cudaError_t frame_backward(const FrameArgs& a, cudaStream_t st) {
 // ------------------------------------------------------------------ Laplacian (Eq. 4)
 __global__ void k_lap_fwd(LapArgs a) {
     __shared__ double red[4];
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double s = 0.0;
-    if (i < a.V) {
-        int lo = a.ring_off[i], hi = a.ring_off[i + 1];
-        float3 m = zero3();
-        for (int j0 = lo; j0 < hi; j0 += ADMS_GATHER) {
-            float3 pk[ADMS_GATHER];
-#pragma unroll
-            for (int q = 0; q < ADMS_GATHER; ++q) {
-                int k = a.ring[min(j0 + q, hi - 1)];
-                pk[q] = f3(a.pos[3 * k], a.pos[3 * k + 1], a.pos[3 * k + 2]);
-            }
-#pragma unroll
-            for (int q = 0; q < ADMS_GATHER; ++q)
-                if (j0 + q < hi) m += pk[q];
-        }
-        float inv = hi > lo ? 1.f / (float)(hi - lo) : 0.f;
-        float3 d = f3(a.pos[3 * i], a.pos[3 * i + 1], a.pos[3 * i + 2]) - inv * m;
-        if (a.delta_ref) d -= f3(a.delta_ref[3 * i], a.delta_ref[3 * i + 1], a.delta_ref[3 * i + 2]);
-        a.delta[3 * i] = d.x;
-        a.delta[3 * i + 1] = d.y;
-        a.delta[3 * i + 2] = d.z;
-        s = (double)dot3(d, d);
-    }
-    s = warp_sum_d(s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(&a.st->lap_sum, red[0] + red[1] + red[2] + red[3]);
-}
-
-// g -= sum over the one-ring i of vertex k of delta_i / |ring(i)| (the adjoint of
-// the one-ring means, gathered per vertex)
-__device__ __forceinline__ void ring_adjoint(const LapArgs& a, int k, float3& g) {
-    int lo = a.ring_off[k], hi = a.ring_off[k + 1];
-    for (int j0 = lo; j0 < hi; j0 += ADMS_GATHER) {
-        float inv[ADMS_GATHER];
-        float3 d[ADMS_GATHER];
-#pragma unroll
-        for (int q = 0; q < ADMS_GATHER; ++q) {
-            int i = a.ring[min(j0 + q, hi - 1)];
-            inv[q] = 1.f / (float)(a.ring_off[i + 1] - a.ring_off[i]);
-            d[q] = f3(a.delta[3 * i], a.delta[3 * i + 1], a.delta[3 * i + 2]);
-        }
-#pragma unroll
-        for (int q = 0; q < ADMS_GATHER; ++q)
-            if (j0 + q < hi) g -= inv[q] * d[q];
-    }
-}
-
-__global__ void k_lap_bwd(LapArgs a) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.V) return;
-    float lam = a.st->lam;
-    float scale = 2.f * lam / (float)a.V;
-    float3 g = f3(a.delta[3 * k], a.delta[3 * k + 1], a.delta[3 * k + 2]);
-    ring_adjoint(a, k, g);
-    a.g_pos[3 * k] += scale * g.x;
-    a.g_pos[3 * k + 1] += scale * g.y;
-    a.g_pos[3 * k + 2] += scale * g.z;
+    lap_vertex(a, blockIdx.x * blockDim.x + threadIdx.x, red);
 }
 
 cudaError_t laplacian_forward(const LapArgs& a, cudaStream_t st) {
@@ -301,12 +184,6 @@ cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st) {
 
 cudaError_t laplacian_gradient(const LapArgs& a, float scale, cudaStream_t st) {
     k_lap_grad_out<<<(a.V + 127) / 128, 128, 0, st>>>(a, scale);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t laplacian_backward(const LapArgs& a, cudaStream_t st) {
-    k_lap_bwd<<<(a.V + 127) / 128, 128, 0, st>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }

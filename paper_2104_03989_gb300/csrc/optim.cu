@@ -4,7 +4,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "kernels.cuh"
+#include "mesh.cuh"
 #include "bulk.cuh"
 
 namespace adms {
@@ -12,7 +12,7 @@ namespace adms {
 constexpr float kLog2_10 = 3.32192809488736234787f;
 
 // lambda_t (Eq. 5 text, recursive reading), lambda_0 heuristic, lr_t, bias corrections
-__global__ void k_schedule(SchedArgs a) {
+__device__ __forceinline__ void schedule_job(const SchedArgs& a) {
     JobState* s = a.st;
     int t = s->t;
     double l_img = s->img_loss;
@@ -45,19 +45,31 @@ __global__ void k_schedule(SchedArgs a) {
     s->img_loss = 0.0;
 }
 
-cudaError_t schedule_step(const SchedArgs& a, cudaStream_t st) {
-    k_schedule<<<1, 1, 0, st>>>(a);
-    count_launches(1);
-    return cudaGetLastError();
+// the scalar kernels: one block per job, one launch for the jobs of a call
+template <int N>
+__global__ void k_schedule(const __grid_constant__ Pack<SchedArgs, N> P) {
+    schedule_job(P.a[N == 1 ? 0 : blockIdx.y]);
+}
+cudaError_t schedule_step(const SchedArgs* as, int n, cudaStream_t st) {
+    return launch_packed(as, n, 1, st, k_schedule<1>, k_schedule<ADMS_BATCH_JOBS>, [](const SchedArgs&) { return 1; });
 }
 
-__global__ void k_advance(JobState* s) {
+template <int N>
+__global__ void k_advance(const __grid_constant__ Pack<JobState*, N> P) {
+    JobState* s = P.a[N == 1 ? 0 : blockIdx.y];
     s->t += 1;
     if (s->status_next) s->status = s->status_next;
 }
 
-__global__ void k_finish_call(JobState* s, float* out) {
-    if (out) *out = (float)s->call_loss;
+struct FinishArgs {
+    JobState* s;
+    float* out;
+};
+template <int N>
+__global__ void k_finish_call(const __grid_constant__ Pack<FinishArgs, N> P) {
+    const FinishArgs& a = P.a[N == 1 ? 0 : blockIdx.y];
+    JobState* s = a.s;
+    if (a.out) *a.out = (float)s->call_loss;
     s->img_loss += s->call_loss;
     if (!isfinite(s->call_loss)) s->status = ADMS_ERR_NONFINITE;  // latched: the optimizer skips the job
 }
@@ -77,15 +89,14 @@ cudaError_t gather_status(JobState* const* js, int n, int* out, cudaStream_t st)
     count_launches(1);
     return cudaGetLastError();
 }
-cudaError_t finish_call_loss(JobState* js, float* out, cudaStream_t st) {
-    k_finish_call<<<1, 1, 0, st>>>(js, out);
-    count_launches(1);
-    return cudaGetLastError();
+cudaError_t finish_call_loss(JobState* const* js, int n, float* out, cudaStream_t st) {
+    std::vector<FinishArgs> as(n);
+    for (int k = 0; k < n; ++k) as[k] = FinishArgs{js[k], out ? out + k : nullptr};
+    return launch_packed(as.data(), n, 1, st, k_finish_call<1>, k_finish_call<ADMS_BATCH_JOBS>,
+                         [](const FinishArgs&) { return 1; });
 }
-cudaError_t advance_step(JobState* js, cudaStream_t st) {
-    k_advance<<<1, 1, 0, st>>>(js);
-    count_launches(1);
-    return cudaGetLastError();
+cudaError_t advance_step(JobState* const* js, int n, cudaStream_t st) {
+    return launch_packed(js, n, 1, st, k_advance<1>, k_advance<ADMS_BATCH_JOBS>, [](JobState* const&) { return 1; });
 }
 
 // One Adam update. A job whose status is latched (a non-finite loss or gradient
@@ -129,6 +140,37 @@ cudaError_t adam_flat(float* p, float* g, float* m, float* v, long long n, const
     k_adam_flat<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, g, m, v, n, js, lr_scale);
     count_launches(1);
     return cudaGetLastError();
+}
+
+// The positions' step: one thread per vertex gathers the Laplacian's gradient and applies
+// Adam to its three coordinates (two launches and a pass over the gradient before). A latched
+// job is left as it is.
+template <int N>
+__global__ void __launch_bounds__(128) k_position_step(const __grid_constant__ Pack<PosStepArgs, N> P) {
+    const PosStepArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
+    const LapArgs& a = A.lap;
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= a.V || a.st->status) return;
+    float scale = 2.f * a.st->lam / (float)a.V;
+    float3 g = f3(a.delta[3 * k], a.delta[3 * k + 1], a.delta[3 * k + 2]);
+    ring_adjoint(a, k, g);
+    float lr = a.st->lr, bc1 = a.st->bc1, bc2 = a.st->bc2;
+    float gl[3] = {g.x, g.y, g.z};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        int i = 3 * k + c;
+        float gi = a.g_pos[i] + scale * gl[c];
+        float mm = A.m[i], vv = A.v[i];
+        latch_nonfinite(a.st, gi);
+        A.p[i] = adam1(A.p[i], gi, mm, vv, lr, bc1, bc2);
+        A.m[i] = mm;
+        A.v[i] = vv;
+        a.g_pos[i] = 0.f;
+    }
+}
+cudaError_t position_step(const PosStepArgs* as, int n, cudaStream_t st) {
+    return launch_packed(as, n, 128, st, k_position_step<1>, k_position_step<ADMS_BATCH_JOBS>,
+                         [](const PosStepArgs& a) { return (a.lap.V + 127) / 128; });
 }
 
 __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fminf(fmaxf(x, lo), hi); }

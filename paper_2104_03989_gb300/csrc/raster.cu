@@ -8,7 +8,7 @@
 //   covered: every edge of the positively wound triangle has E > 0, or E = 0 on a top/left edge
 //   d = (z0 + b1 (z1 - z0)) + b2 (z2 - z0), b1 = (float)E_20 / (float)A, b2 = (float)E_01 / (float)A
 //   key = (float_bits(d) << 32) | triangle id, minimum per pixel.
-#include "kernels.cuh"
+#include "mesh.cuh"
 
 namespace adms {
 
@@ -40,12 +40,11 @@ __device__ __forceinline__ DF df_affine(float c0, float s, DF q) {
 }
 
 // ---------------------------------------------------------------- transform
-__global__ void k_transform(const float* __restrict__ pos, int V, const adms_view* __restrict__ views, int B, int W,
-                            int H, float4* __restrict__ clip, VtxS* __restrict__ vs, float4* __restrict__ scr,
-                            long long* __restrict__ zero_total) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && zero_total) *zero_total = 0;  // the tile-list allocation's counter (k_list_alloc)
-    if (i >= B * V) return;
+// vertex i (view-major) of a job
+__device__ __forceinline__ void transform_vertex(const float* __restrict__ pos, int V,
+                                                 const adms_view* __restrict__ views, int W, int H,
+                                                 float4* __restrict__ clip, VtxS* __restrict__ vs,
+                                                 float4* __restrict__ scr, int i) {
     int b = i / V, v = i - b * V;
     const float* M = views[b].mvp;
     float x = pos[3 * v], y = pos[3 * v + 1], z = pos[3 * v + 2];
@@ -87,19 +86,70 @@ __global__ void k_transform(const float* __restrict__ pos, int V, const adms_vie
     vs[i] = o;
 }
 
+// The first launch of a raster pass: the first nb_vert blocks of a job transform its vertices,
+// the rest set its keys to empty and clear the tile counts and whatever else of 4-byte words
+// the pass needs at zero (four memset launches before).
+struct ClearSeg {
+    int* p;
+    long long n;
+};
+#define ADMS_BEGIN_CLEARS (ADMS_PREP_CLEARS + 3)
+struct BeginArgs {
+    const float* pos;
+    const adms_view* views;
+    float4* clip;
+    VtxS* vs;
+    float4* scr;
+    unsigned long long* keys;
+    long long n_keys;
+    ClearSeg z[ADMS_BEGIN_CLEARS];
+    int V, B, W, H, nb_vert, nb_fill;
+};
+template <int N>
+__global__ void __launch_bounds__(256) k_begin(const __grid_constant__ Pack<BeginArgs, N> P) {
+    const BeginArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
+    int blk = blockIdx.x;
+    if (blk < A.nb_vert) {
+        int i = blk * 256 + threadIdx.x;
+        if (i < A.B * A.V) transform_vertex(A.pos, A.V, A.views, A.W, A.H, A.clip, A.vs, A.scr, i);
+        return;
+    }
+    blk -= A.nb_vert;
+    if (blk >= A.nb_fill) return;
+    long long t = (long long)blk * 256 + threadIdx.x, step = (long long)A.nb_fill * 256;
+    if (reinterpret_cast<uintptr_t>(A.keys) & 15) {
+        for (long long i = t; i < A.n_keys; i += step) A.keys[i] = ADMS_EMPTY_KEY;
+    } else {
+        ulonglong2 e = make_ulonglong2(ADMS_EMPTY_KEY, ADMS_EMPTY_KEY);
+        for (long long i = t; i < A.n_keys / 2; i += step) reinterpret_cast<ulonglong2*>(A.keys)[i] = e;
+        if (t == 0 && (A.n_keys & 1)) A.keys[A.n_keys - 1] = ADMS_EMPTY_KEY;
+    }
+#pragma unroll
+    for (int k = 0; k < ADMS_BEGIN_CLEARS; ++k)
+        for (long long i = t; i < A.z[k].n; i += step) A.z[k].p[i] = 0;
+}
+
 // ---------------------------------------------------------------- tile-list allocation
 // Each tile's list segment [off, off + count) in the list buffer: a warp scans its 32
 // tiles' counts by shuffles and reserves their segments together with one 64-bit
-// atomicAdd on *total (zeroed by k_transform), so the segments lie in no particular
+// atomicAdd on *total (zeroed by k_begin), so the segments lie in no particular
 // order, as the entries inside a segment already do (the raster's per-pixel minimum
 // does not depend on either). Offsets saturate at INT_MAX (the list-capacity check
 // catches an overflow); *total ends exact. Many small blocks rather than one large
 // scan block: a 1024-thread block does not fit on an SM beside a resident
 // streamed-Adam block, which a pipelined step runs at the same time.
-__global__ void __launch_bounds__(256) k_list_alloc(const int* __restrict__ count, int n, int* __restrict__ off,
-                                                    unsigned long long* __restrict__ total) {
+struct AllocArgs {
+    const int* count;
+    int n;
+    int* off;
+    unsigned long long* total;
+};
+template <int N>
+__global__ void __launch_bounds__(256) k_list_alloc(const __grid_constant__ Pack<AllocArgs, N> P) {
+    const AllocArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
+    const int n = A.n;
     int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
-    long long c = i < n ? count[i] : 0;
+    long long c = i < n ? A.count[i] : 0;
     long long x = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -107,9 +157,9 @@ __global__ void __launch_bounds__(256) k_list_alloc(const int* __restrict__ coun
         if (lane >= o) x += y;
     }
     unsigned long long base = 0;
-    if (lane == 31 && x > 0) base = atomicAdd(total, (unsigned long long)x);
+    if (lane == 31 && x > 0) base = atomicAdd(A.total, (unsigned long long)x);
     base = __shfl_sync(0xffffffffu, base, 31);
-    if (i < n) off[i] = (int)min((long long)base + x - c, (long long)0x7fffffff);
+    if (i < n) A.off[i] = (int)min((long long)base + x - c, (long long)0x7fffffff);
 }
 
 // ---------------------------------------------------------------- edge functions
@@ -254,13 +304,28 @@ struct DirectTri {  // 80 bytes: 16-byte reads of consecutive slots touch distin
     unsigned zlo;
     int thr;             // thr_1 | thr_2 << 1
 };
-template <bool ZF>
-__global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
-    k_setup(const int* __restrict__ tri, int F, const VtxS* __restrict__ vs, int V, int B, int W, int H, int tiles_x,
-            int tiles_y, TriRec* __restrict__ rec, TriBin* __restrict__ bin, int8_t* __restrict__ asign,
-            int* __restrict__ tile_count, unsigned long long* __restrict__ keys, int small_px) {
+struct SetupArgs {
+    const int* tri;
+    const VtxS* vs;
+    TriRec* rec;
+    TriBin* bin;
+    int8_t* asign;
+    int* tile_count;
+    unsigned long long* keys;
+    int F, V, B, W, H, tiles_x, tiles_y, small_px, zfilter;
+};
+// ZF: compiled with the key read; taken where the job asks for it
+template <bool ZF, int N>
+__global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_constant__ Pack<SetupArgs, N> P) {
     __shared__ DirectTri slots[8][32];
+    const SetupArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
+    const int* __restrict__ tri = A.tri;
+    const VtxS* __restrict__ vs = A.vs;
+    unsigned long long* __restrict__ keys = A.keys;
+    const int F = A.F, V = A.V, B = A.B, W = A.W, H = A.H, tiles_x = A.tiles_x, tiles_y = A.tiles_y;
+    const bool zf = ZF && (N == 1 || A.zfilter);
     const unsigned full = 0xffffffffu;
+    if ((long long)blockIdx.x * blockDim.x >= (long long)B * F) return;
     int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     int npx = 0;  // samples of this lane's direct triangle
     DirectTri t;
@@ -274,9 +339,9 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
         int8_t sgn = 0;
         if (v0.ok && v1.ok && v2.ok) {
             int X[3] = {v0.X, v1.X, v2.X}, Y[3] = {v0.Y, v1.Y, v2.Y};
-            long long A = (long long)(X[1] - X[0]) * (Y[2] - Y[0]) - (long long)(Y[1] - Y[0]) * (X[2] - X[0]);
-            if (A != 0) {
-                sgn = A > 0 ? 1 : -1;
+            long long area = (long long)(X[1] - X[0]) * (Y[2] - Y[0]) - (long long)(Y[1] - Y[0]) * (X[2] - X[0]);
+            if (area != 0) {
+                sgn = area > 0 ? 1 : -1;
                 int minX = min(X[0], min(X[1], X[2])), maxX = max(X[0], max(X[1], X[2]));
                 int minY = min(Y[0], min(Y[1], Y[2])), maxY = max(Y[0], max(Y[1], Y[2]));
                 // samples at 256 i + 128; |X| <= 2^27, so the shifts round down without overflow
@@ -286,7 +351,7 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
                     bool near = maxX - minX <= ADMS_NEAR && maxY - minY <= ADMS_NEAR;
                     float dz1 = __fsub_rn(v1.z, v0.z), dz2 = __fsub_rn(v2.z, v0.z);
                     int w = ihi - ilo + 1, n = w * (jhi - jlo + 1);  // at most 2^28
-                    if (near && n <= small_px) {
+                    if (near && n <= A.small_px) {
                         npx = n;
                         Edges<int> e = make_edges<int>(X, Y);
                         near_pack(e, 256 * ilo + 128, 256 * jlo + 128, t.p, t.q);
@@ -296,7 +361,7 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
                         t.inv_w = w > 1 ? 0xffffffffu / (unsigned)w + 1u : 0u;
                         t.origin = ((long long)b * H + jlo) * W + ilo;
                         t.width = w;
-                        t.zlo = ZF ? key_floor(v0.z, v1.z, v2.z) : 0u;
+                        t.zlo = zf ? key_floor(v0.z, v1.z, v2.z) : 0u;
                         t.thr = e.thr[1] | (e.thr[2] << 1);
                     } else {
                         tb.bx0 = (short)ilo;
@@ -311,8 +376,8 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
                         r.dz2 = dz2;
                         r.near = near;
                         r.box = tb;
-                        rec[i] = r;
-                        int* tc = tile_count + (size_t)b * tiles_x * tiles_y;
+                        A.rec[i] = r;
+                        int* tc = A.tile_count + (size_t)b * tiles_x * tiles_y;
                         auto count = [&](int k) { atomicAdd(tc + k, 1); };
                         if (near) for_tiles(make_edges<int>(X, Y), tb, tiles_x, count);
                         else for_tiles(make_edges<long long>(X, Y), tb, tiles_x, count);
@@ -320,8 +385,8 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
                 }
             }
         }
-        asign[i] = sgn;
-        bin[i] = tb;
+        A.asign[i] = sgn;
+        A.bin[i] = tb;
     }
     unsigned direct = __ballot_sync(full, npx > 0);
     if (!direct) return;
@@ -350,7 +415,7 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
         if ((e0 | e1 | e2) < 0) continue;
         unsigned long long* a = keys + d.origin + (long long)y * W + x;
         unsigned long long cur = ADMS_EMPTY_KEY;
-        if (ZF) {
+        if (zf) {
             cur = __ldcg(a);
             if (d.zlo > (unsigned)(cur >> 32)) continue;
         }
@@ -358,7 +423,7 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS)
         unsigned long long key =
             depth_key(__int2float_rn(e1 + (d.thr & 1)), __int2float_rn(e2 + (d.thr >> 1)), __int_as_float(r.x),
                       __int_as_float(r.y), __int_as_float(r.z), __int_as_float(r.w), d.id);
-        if (ZF ? key < cur : key != ADMS_EMPTY_KEY) atomicMin(a, key);
+        if (zf ? key < cur : key != ADMS_EMPTY_KEY) atomicMin(a, key);
     }
 }
 
@@ -380,33 +445,67 @@ struct TileLists {
 // silhouette-edge mask, then its entries in the tile lists. Bit e of
 // silmask[b][f] is set when edge e of triangle f is a silhouette edge in view b:
 // no neighbour across it, or a neighbour whose snapped area has another sign.
-__global__ void k_bin_fill(const TriRec* __restrict__ rec, const TriBin* __restrict__ bin, int F, int B, int tiles_x,
-                           int tiles_y, const int* __restrict__ tile_off, int* __restrict__ tile_cursor,
-                           const TileLists lists, const int* __restrict__ adj, const int8_t* __restrict__ asign,
-                           uint8_t* __restrict__ silmask) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * F) return;
-    int b = i / F, f = i - b * F;
+//
+// FRAME: the launch also forms the vertex frame and the Laplacian where they are due (new
+// positions), in its first blocks: both need only the positions and take about as long as the
+// lists, so that neither costs a launch, a second stream or a join before the shading.
+struct FillArgs {
+    const TriRec* rec;
+    const TriBin* bin;
+    const int* tile_off;
+    int* tile_cursor;
+    TileLists lists;
+    const int* adj;
+    const int8_t* asign;
+    uint8_t* silmask;
+    int F, B, tiles_x, tiles_y;
+    int nb_frame, nb_lap, nb_fill;
+    FrameArgs f;
+    LapArgs l;
+};
+template <bool FRAME, int N>
+__global__ void __launch_bounds__(256) k_bin_fill(const __grid_constant__ Pack<FillArgs, N> P) {
+    const FillArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
+    int blk = blockIdx.x;
+    if (FRAME) {
+        __shared__ double red[8];
+        if (blk < A.nb_frame) {
+            int v = blk * 256 + threadIdx.x;
+            if (v < A.f.V) frame_vertex(A.f, v);
+            return;
+        }
+        blk -= A.nb_frame;
+        if (blk < A.nb_lap) {
+            lap_vertex(A.l, blk * 256 + threadIdx.x, red);
+            return;
+        }
+        blk -= A.nb_lap;
+    }
+    int i = blk * 256 + threadIdx.x;
+    if (i >= A.B * A.F) return;
+    int b = i / A.F, f = i - b * A.F;
     {
-        const int8_t* sg = asign + (size_t)b * F;
+        const int8_t* sg = A.asign + (size_t)b * A.F;
         int sf = sg[f];
         uint8_t msk = 0;
         if (sf != 0) {
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
-                int nb = adj[3 * f + e];
+                int nb = A.adj[3 * f + e];
                 if (nb < 0 || sg[nb] != sf) msk |= (uint8_t)(1u << e);
             }
         }
-        silmask[i] = msk;
+        A.silmask[i] = msk;
     }
-    TriBin tb = bin[i];
+    TriBin tb = A.bin[i];
     if (tb.bx0 > tb.bx1) return;
-    size_t tbase = (size_t)b * tiles_x * tiles_y;
-    TriRec r = rec[i];
-    auto fill = [&](int k) { lists.set((long long)tile_off[tbase + k] + atomicAdd(tile_cursor + tbase + k, 1), f); };
-    if (r.near) for_tiles(make_edges<int>(r.X, r.Y), tb, tiles_x, fill);
-    else for_tiles(make_edges<long long>(r.X, r.Y), tb, tiles_x, fill);
+    size_t tbase = (size_t)b * A.tiles_x * A.tiles_y;
+    TriRec r = A.rec[i];
+    auto fill = [&](int k) {
+        A.lists.set((long long)A.tile_off[tbase + k] + atomicAdd(A.tile_cursor + tbase + k, 1), f);
+    };
+    if (r.near) for_tiles(make_edges<int>(r.X, r.Y), tb, A.tiles_x, fill);
+    else for_tiles(make_edges<long long>(r.X, r.Y), tb, A.tiles_x, fill);
 }
 
 // ---------------------------------------------------------------- tiled raster
@@ -660,35 +759,92 @@ cudaError_t raster_tiles_batched(const RasterJob* args, const int* item_off, int
 }
 
 // ---------------------------------------------------------------- host launchers
-cudaError_t raster_prepare(const RasterIn& in, RasterScratch& s, cudaStream_t st) {
-    int B = in.B, V = in.V, F = in.F, W = in.W, H = in.H;
-    int tiles_x = (W + ADMS_TILE - 1) / ADMS_TILE, tiles_y = (H + ADMS_TILE - 1) / ADMS_TILE;
-    int ntiles = B * tiles_x * tiles_y;
-    cudaError_t e;
-    // without a key buffer (every triangle binned: small_px = 0) the keys are left to raster_tiles' caller
-    if (in.keys && (e = cudaMemsetAsync(in.keys, 0xFF, sizeof(unsigned long long) * B * H * W, st))) return e;
-    if (s.tile_cursor == s.tile_count + ntiles) {  // one buffer: counts, then cursors
-        if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * 2 * ntiles, st))) return e;
-    } else {
-        if ((e = cudaMemsetAsync(s.tile_count, 0, sizeof(int) * ntiles, st))) return e;
-        if ((e = cudaMemsetAsync(s.tile_cursor, 0, sizeof(int) * ntiles, st))) return e;
+cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
+    std::vector<BeginArgs> begin(n);
+    std::vector<SetupArgs> setup(n);
+    std::vector<AllocArgs> alloc(n);
+    std::vector<FillArgs> fill(n);
+    bool zf = false, frame = false;
+    for (int k = 0; k < n; ++k) {
+        const RasterIn& in = jobs[k].in;
+        RasterScratch& s = *jobs[k].s;
+        int tiles_x = (in.W + ADMS_TILE - 1) / ADMS_TILE, tiles_y = (in.H + ADMS_TILE - 1) / ADMS_TILE;
+        int ntiles = in.B * tiles_x * tiles_y;
+        BeginArgs& g = begin[k];
+        g.pos = in.pos;
+        g.views = in.views;
+        g.clip = s.clip;
+        g.vs = s.vs;
+        g.scr = s.scr;
+        g.V = in.V;
+        g.B = in.B;
+        g.W = in.W;
+        g.H = in.H;
+        g.keys = in.keys;
+        g.n_keys = in.keys && in.small_px > 0 ? (long long)in.B * in.H * in.W : 0;
+        int z = 0;
+        long long words = 0;
+        auto clear = [&](void* p, size_t bytes) {
+            g.z[z++] = ClearSeg{static_cast<int*>(p), (long long)(bytes / 4)};
+            words += (long long)(bytes / 4);
+        };
+        clear(s.tile_count, sizeof(int) * (size_t)ntiles);
+        clear(s.tile_cursor, sizeof(int) * (size_t)ntiles);
+        if (s.total_pairs) clear(s.total_pairs, sizeof(long long));
+        for (int c = 0; c < jobs[k].n_clear; ++c) clear(jobs[k].clear[c], jobs[k].clear_bytes[c]);
+        g.nb_vert = (in.B * in.V + 255) / 256;
+        // 16 stores of 16 bytes per thread for the keys, 16 of 4 for the rest
+        g.nb_fill = (int)std::max<long long>(1, std::max(g.n_keys / 2, words) / (256 * 16));
+        setup[k] = SetupArgs{in.tri, s.vs, s.rec, s.bin, s.asign, s.tile_count, in.keys, in.F, in.V, in.B, in.W, in.H,
+                             tiles_x, tiles_y, in.small_px, in.zfilter && in.small_px > ADMS_SMALL_PX};
+        zf = zf || setup[k].zfilter;
+        alloc[k] = AllocArgs{s.tile_count, ntiles, s.tile_off, reinterpret_cast<unsigned long long*>(s.total_pairs)};
+        FillArgs& f = fill[k];
+        f.rec = s.rec;
+        f.bin = s.bin;
+        f.tile_off = s.tile_off;
+        f.tile_cursor = s.tile_cursor;
+        f.lists = tile_lists(s.rec, s.list, s.list_capacity, (long long)in.B * in.F);
+        f.adj = in.adj;
+        f.asign = s.asign;
+        f.silmask = s.silmask;
+        f.F = in.F;
+        f.B = in.B;
+        f.tiles_x = tiles_x;
+        f.tiles_y = tiles_y;
+        f.nb_fill = (in.B * in.F + 255) / 256;
+        if (jobs[k].frame) {
+            f.f = jobs[k].f;
+            f.nb_frame = (f.f.V + 255) / 256;
+        }
+        if (jobs[k].lap) {
+            f.l = jobs[k].l;
+            f.nb_lap = (f.l.V + 255) / 256;
+        }
+        frame = frame || f.nb_frame || f.nb_lap;
     }
-    int bs = 256;
-    k_transform<<<(B * V + bs - 1) / bs, bs, 0, st>>>(in.pos, V, in.views, B, W, H, s.clip, s.vs, s.scr,
-                                                    s.total_pairs);
-    if (in.zfilter && in.small_px > ADMS_SMALL_PX)
-        k_setup<true><<<(B * F + bs - 1) / bs, bs, 0, st>>>(in.tri, F, s.vs, V, B, W, H, tiles_x, tiles_y, s.rec,
-                                                          s.bin, s.asign, s.tile_count, in.keys, in.small_px);
-    else
-        k_setup<false><<<(B * F + bs - 1) / bs, bs, 0, st>>>(in.tri, F, s.vs, V, B, W, H, tiles_x, tiles_y, s.rec,
-                                                           s.bin, s.asign, s.tile_count, in.keys, in.small_px);
-    k_list_alloc<<<(ntiles + bs - 1) / bs, bs, 0, st>>>(s.tile_count, ntiles, s.tile_off,
-                                                       reinterpret_cast<unsigned long long*>(s.total_pairs));
-    k_bin_fill<<<(B * F + bs - 1) / bs, bs, 0, st>>>(s.rec, s.bin, F, B, tiles_x, tiles_y, s.tile_off, s.tile_cursor,
-                                                   tile_lists(s.rec, s.list, s.list_capacity, (long long)B * F),
-                                                   in.adj, s.asign, s.silmask);
-    count_launches(4);
-    return cudaGetLastError();
+    constexpr int M = ADMS_BATCH_JOBS;
+    cudaError_t e = launch_packed(begin.data(), n, 256, st, k_begin<1>, k_begin<M>,
+                                  [](const BeginArgs& a) { return a.nb_vert + a.nb_fill; });
+    auto tri_blocks = [](const SetupArgs& a) { return (a.B * a.F + 255) / 256; };
+    if (!e)
+        e = zf ? launch_packed(setup.data(), n, 256, st, k_setup<true, 1>, k_setup<true, M>, tri_blocks)
+               : launch_packed(setup.data(), n, 256, st, k_setup<false, 1>, k_setup<false, M>, tri_blocks);
+    if (!e)
+        e = launch_packed(alloc.data(), n, 256, st, k_list_alloc<1>, k_list_alloc<M>,
+                          [](const AllocArgs& a) { return (a.n + 255) / 256; });
+    auto fill_blocks = [](const FillArgs& a) { return a.nb_frame + a.nb_lap + a.nb_fill; };
+    if (!e)
+        e = frame ? launch_packed(fill.data(), n, 256, st, k_bin_fill<true, 1>, k_bin_fill<true, M>, fill_blocks)
+                  : launch_packed(fill.data(), n, 256, st, k_bin_fill<false, 1>, k_bin_fill<false, M>, fill_blocks);
+    return e;
+}
+
+cudaError_t raster_prepare(const RasterIn& in, RasterScratch& s, cudaStream_t st) {
+    PrepJob j;
+    j.in = in;
+    j.s = &s;
+    return raster_prepare(&j, 1, st);
 }
 
 static TileArgs tile_args(const RasterIn& in, const RasterScratch& s) {
