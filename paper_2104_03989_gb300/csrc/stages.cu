@@ -150,6 +150,28 @@ __device__ __forceinline__ void corner_ids(const ShadeArgs& A, int f, PixGeo& g)
     }
 }
 
+// the three maps' trilinear samples at g's texture coordinate (LODs into lod)
+__device__ __forceinline__ void stage_samples(const ShadeArgs& A, const PixGeo& g, float lod[3], ShadeIn& in) {
+    in.p = g.p;
+    in.n_i = g.n;
+    in.t_i = g.t;
+    if (shared_taps(A)) {
+        lod[0] = lod[1] = lod[2] = tex_lod(A.kd, g.duv_dx, g.duv_dy);
+        float4 smp[3];
+        tex_sample3(A, g.tc, lod[0], smp);
+        in.kd = smp[0];
+        in.orm = smp[1];
+        in.nm = smp[2];
+    } else {
+        lod[0] = tex_lod(A.kd, g.duv_dx, g.duv_dy);
+        lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
+        lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
+        in.kd = tex_sample(A.kd, g.tc, lod[0]);
+        in.orm = tex_sample(A.orm, g.tc, lod[1]);
+        in.nm = tex_sample(A.nrm, g.tc, lod[2]);
+    }
+}
+
 // pre-antialiasing colour from the barycentrics buffer
 __global__ void __launch_bounds__(256) k_stage_shade_fwd(ShadeArgs A, const float2* __restrict__ rast,
                                                          const float4* __restrict__ rast_db) {
@@ -168,7 +190,8 @@ __global__ void __launch_bounds__(256) k_stage_shade_fwd(ShadeArgs A, const floa
     float2 bb = rast[pix];
     pix_attr<true>(A, g, bb.x, bb.y, rast_db[pix]);
     float lod[3];
-    ShadeIn in = shade_inputs(A, g, lod);
+    ShadeIn in;
+    stage_samples(A, g, lod, in);
     float3 c = shade_eval<false>(A.views[b], in, zero3(), nullptr);
     A.pre[pix] = make_float4(c.x, c.y, c.z, 1.f);
 }
@@ -201,7 +224,8 @@ __global__ void __launch_bounds__(256, 3) k_stage_shade_bwd(ShadeArgs A, const f
                 PixGeo g;
                 corner_ids(A, f, g);
                 pix_attr<true>(A, g, bb.x, bb.y, rast_db[pix]);
-                ShadeIn in = shade_inputs(A, g, lod);
+                ShadeIn in;
+                stage_samples(A, g, lod, in);
                 tc = g.tc;
                 shade_eval<true>(A.views[b], in, gc, &G);
             }
