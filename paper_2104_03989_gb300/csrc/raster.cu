@@ -292,6 +292,7 @@ __device__ __forceinline__ void near_pack(const Edges<int>& e, int Sx, int Sy, i
 // is below the stored one. The stored key only ever decreases, so a read that lags behind
 // other threads' updates can only let an unneeded atomicMin through. Without it (closed
 // surfaces, about two fragments per sample) the read would only add a round trip.
+#define ADMS_ROUNDS_MIN (1 << 18)
 #ifndef ADMS_SETUP_BLOCKS
 #define ADMS_SETUP_BLOCKS 4
 #endif
@@ -313,7 +314,40 @@ struct SetupArgs {
     int* tile_count;
     unsigned long long* keys;
     int F, V, B, W, H, tiles_x, tiles_y, small_px, zfilter;
+    // a round of a dense cloud (ZF): the triangles of groups c0 .. c0 + cw - 1 of every eight
+    // groups of eight, per_view threads per view; hiz: per tile the largest stored depth after
+    // the rounds before (null: none)
+    int c0, cw, per_view;
+    const unsigned* hiz;
 };
+
+// Whether every sample of the box shows something nearer than zlo: hiz[tile] is the largest
+// depth word stored in the tile some time ago, and stored keys only decrease.
+__device__ __forceinline__ bool box_hidden(const SetupArgs& A, int b, int bx0, int bx1, int by0, int by1,
+                                           unsigned zlo) {
+    const unsigned* h = A.hiz + (size_t)b * A.tiles_x * A.tiles_y;
+    for (int ty = by0 / ADMS_TILE; ty <= by1 / ADMS_TILE; ++ty)
+        for (int tx = bx0 / ADMS_TILE; tx <= bx1 / ADMS_TILE; ++tx)
+            if (zlo <= h[ty * A.tiles_x + tx]) return false;
+    return true;
+}
+// the largest depth word of each 16x16 tile's stored keys (all ones where a sample is empty),
+// a warp per tile
+__global__ void __launch_bounds__(256) k_tile_depth(const unsigned long long* __restrict__ keys, int n_tiles, int tiles_x,
+                                                    int tiles_y, int W, int H, unsigned* __restrict__ hiz) {
+    int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= n_tiles) return;
+    int per_view = tiles_x * tiles_y, b = t / per_view, r = t % per_view;
+    int x = (r % tiles_x) * ADMS_TILE + (lane & 15), y0 = (r / tiles_x) * ADMS_TILE + (lane >> 4);
+    unsigned m = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        int y = y0 + 2 * k;
+        if (x < W && y < H) m = max(m, (unsigned)(__ldcg(keys + ((size_t)b * H + y) * W + x) >> 32));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) hiz[t] = m;
+}
 // ZF: compiled with the key read; taken where the job asks for it
 template <bool ZF, int N>
 __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_constant__ Pack<SetupArgs, N> P) {
@@ -325,12 +359,15 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_c
     const int F = A.F, V = A.V, B = A.B, W = A.W, H = A.H, tiles_x = A.tiles_x, tiles_y = A.tiles_y;
     const bool zf = ZF && (N == 1 || A.zfilter);
     const unsigned full = 0xffffffffu;
-    if ((long long)blockIdx.x * blockDim.x >= (long long)B * F) return;
+    const int per_view = ZF && N == 1 ? A.per_view : F;
+    if ((long long)blockIdx.x * blockDim.x >= (long long)B * per_view) return;
     int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     int npx = 0;  // samples of this lane's direct triangle
     DirectTri t;
-    if (i < B * F) {
-        int b = i / F, f = i - b * F;
+    int b = i / per_view, f = i - b * per_view;
+    if (ZF && N == 1) f = 8 * ((f / (8 * A.cw)) * 8 + A.c0 + (f / 8) % A.cw) + (f & 7);
+    if (b < B && f < F) {
+        i = b * F + f;
         const VtxS* vb = vs + (size_t)b * V;
         VtxS v0 = vb[tri[3 * f]], v1 = vb[tri[3 * f + 1]], v2 = vb[tri[3 * f + 2]];
         TriBin tb;
@@ -351,7 +388,10 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_c
                     bool near = maxX - minX <= ADMS_NEAR && maxY - minY <= ADMS_NEAR;
                     float dz1 = __fsub_rn(v1.z, v0.z), dz2 = __fsub_rn(v2.z, v0.z);
                     int w = ihi - ilo + 1, n = w * (jhi - jlo + 1);  // at most 2^28
-                    if (near && n <= A.small_px) {
+                    unsigned zlo = zf ? key_floor(v0.z, v1.z, v2.z) : 0u;
+                    if (ZF && N == 1 && A.hiz && box_hidden(A, b, ilo, ihi, jlo, jhi, zlo)) {
+                        // nothing of it can be seen: no record, no samples
+                    } else if (near && n <= A.small_px) {
                         npx = n;
                         Edges<int> e = make_edges<int>(X, Y);
                         near_pack(e, 256 * ilo + 128, 256 * jlo + 128, t.p, t.q);
@@ -361,7 +401,7 @@ __global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_c
                         t.inv_w = w > 1 ? 0xffffffffu / (unsigned)w + 1u : 0u;
                         t.origin = ((long long)b * H + jlo) * W + ilo;
                         t.width = w;
-                        t.zlo = zf ? key_floor(v0.z, v1.z, v2.z) : 0u;
+                        t.zlo = zlo;
                         t.thr = e.thr[1] | (e.thr[2] << 1);
                     } else {
                         tb.bx0 = (short)ilo;
@@ -796,7 +836,7 @@ cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
         // 16 stores of 16 bytes per thread for the keys, 16 of 4 for the rest
         g.nb_fill = (int)std::max<long long>(1, std::max(g.n_keys / 2, words) / (256 * 16));
         setup[k] = SetupArgs{in.tri, s.vs, s.rec, s.bin, s.asign, s.tile_count, in.keys, in.F, in.V, in.B, in.W, in.H,
-                             tiles_x, tiles_y, in.small_px, in.zfilter && in.small_px > ADMS_SMALL_PX};
+                             tiles_x, tiles_y, in.small_px, in.zfilter && in.small_px > ADMS_SMALL_PX, 0, 8, in.F, nullptr};
         zf = zf || setup[k].zfilter;
         alloc[k] = AllocArgs{s.tile_count, ntiles, s.tile_off, reinterpret_cast<unsigned long long*>(s.total_pairs)};
         FillArgs& f = fill[k];
@@ -827,9 +867,28 @@ cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
     cudaError_t e = launch_packed(begin.data(), n, 256, st, k_begin<1>, k_begin<M>,
                                   [](const BeginArgs& a) { return a.nb_vert + a.nb_fill; });
     auto tri_blocks = [](const SetupArgs& a) { return (a.B * a.F + 255) / 256; };
-    if (!e)
+    if (!e && zf && n == 1 && (long long)setup[0].B * setup[0].F >= ADMS_ROUNDS_MIN) {
+        // tile_off holds the tiles' depths until the list allocation writes it
+        SetupArgs a = setup[0];
+        int nt = a.B * a.tiles_x * a.tiles_y;
+        unsigned* hiz = reinterpret_cast<unsigned*>(jobs[0].s->tile_off);
+        const int first[5] = {0, 1, 2, 4, 8};
+        for (int r = 0; r < 4 && !e; ++r) {
+            a.c0 = first[r];
+            a.cw = first[r + 1] - first[r];
+            a.per_view = (a.F + 63) / 64 * 8 * a.cw;
+            a.hiz = r ? hiz : nullptr;
+            e = launch_packed(&a, 1, 256, st, k_setup<true, 1>, k_setup<true, M>,
+                              [](const SetupArgs& q) { return (int)(((long long)q.B * q.per_view + 255) / 256); });
+            if (e || r == 3) break;
+            k_tile_depth<<<(nt + 7) / 8, 256, 0, st>>>(a.keys, nt, a.tiles_x, a.tiles_y, a.W, a.H, hiz);
+            count_launches(1);
+            e = cudaGetLastError();
+        }
+    } else if (!e) {
         e = zf ? launch_packed(setup.data(), n, 256, st, k_setup<true, 1>, k_setup<true, M>, tri_blocks)
                : launch_packed(setup.data(), n, 256, st, k_setup<false, 1>, k_setup<false, M>, tri_blocks);
+    }
     if (!e)
         e = launch_packed(alloc.data(), n, 256, st, k_list_alloc<1>, k_list_alloc<M>,
                           [](const AllocArgs& a) { return (a.n + 255) / 256; });
