@@ -707,9 +707,9 @@ __device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int t
 __device__ __forceinline__ void raster_tile_body(const TileArgs& A, unsigned long long* __restrict__ keys, int b,
                                                  int tile, TileSmem& sm) {
     size_t t = (size_t)b * A.tiles_x * A.tiles_y + tile;
-    long long off = A.tile_off[t];
     int cnt = A.tile_count[t];
     if (cnt == 0) return;  // no binned triangle: the small-triangle pass left the final keys
+    long long off = A.tile_off[t];
     int px = (tile % A.tiles_x) * ADMS_TILE + tile_x(threadIdx.x), py = (tile / A.tiles_x) * ADMS_TILE + tile_y(threadIdx.x);
     bool inside = px < A.W && py < A.H;
     size_t pix = ((size_t)b * A.H + py) * A.W + px;
@@ -722,6 +722,20 @@ __device__ __forceinline__ void raster_tile_body(const TileArgs& A, unsigned lon
 __global__ void __launch_bounds__(256) k_raster(const TileArgs A, unsigned long long* __restrict__ keys) {
     __shared__ TileSmem sm;
     raster_tile_body(A, keys, blockIdx.y, blockIdx.x, sm);
+}
+
+// the same for a mostly empty grid: block k takes tiles k, k + gridDim.x, ... of all views, up
+// to 32, reads their counts together and skips the empty ones
+__global__ void __launch_bounds__(256) k_raster_sparse(const TileArgs A, unsigned long long* __restrict__ keys,
+                                                       int n_tiles) {
+    __shared__ TileSmem sm;
+    long long t = blockIdx.x + (long long)(threadIdx.x & 31) * gridDim.x;
+    unsigned live = __ballot_sync(0xffffffffu, t < n_tiles && A.tile_count[t] > 0);
+    int per_view = A.tiles_x * A.tiles_y;
+    for (; live; live &= live - 1) {
+        int k = blockIdx.x + (__ffs(live) - 1) * gridDim.x;
+        raster_tile_body(A, keys, k / per_view, k % per_view, sm);
+    }
 }
 
 // Depth peeling in one pass (Sec. 5.2): per sample the L nearest fragments,
@@ -906,6 +920,7 @@ cudaError_t raster_prepare(const RasterIn& in, RasterScratch& s, cudaStream_t st
     return raster_prepare(&j, 1, st);
 }
 
+#define ADMS_RASTER_GRID 2048
 static TileArgs tile_args(const RasterIn& in, const RasterScratch& s) {
     return TileArgs{s.rec, s.bin, in.F, in.W, in.H, (in.W + ADMS_TILE - 1) / ADMS_TILE,
                     (in.H + ADMS_TILE - 1) / ADMS_TILE, s.tile_off, s.tile_count,
@@ -914,7 +929,15 @@ static TileArgs tile_args(const RasterIn& in, const RasterScratch& s) {
 
 cudaError_t raster_tiles(const RasterIn& in, RasterScratch& s, cudaStream_t st) {
     TileArgs a = tile_args(in, s);
-    k_raster<<<dim3(a.tiles_x * a.tiles_y, in.B), 256, 0, st>>>(a, in.keys);
+    // A job that rasterizes most of its triangles directly has mostly empty tiles: a grid of
+    // ADMS_RASTER_GRID blocks looks them over (16 views of 1024x1024 of a displaced mesh, two
+    // passes: 83 -> 16 us; 600k leaf quads 65 -> 36). Where the tiles hold work the hardware's
+    // block scheduling balances better (plain mesh, a block per tile 41.2 us, two tiles 45.4,
+    // four 48.0).
+    int n = a.tiles_x * a.tiles_y * in.B;
+    int per = in.small_px > ADMS_SMALL_PX ? std::min(n / ADMS_RASTER_GRID, 32) : 1;
+    if (per > 1) k_raster_sparse<<<(n + per - 1) / per, 256, 0, st>>>(a, in.keys, n);
+    else k_raster<<<dim3(a.tiles_x * a.tiles_y, in.B), 256, 0, st>>>(a, in.keys);
     count_launches(1);
     return cudaGetLastError();
 }
