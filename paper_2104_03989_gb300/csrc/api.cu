@@ -607,6 +607,14 @@ adms_status render_core(adms_ctx* ctx, Job& j, bool clear_grads = false, bool cl
     if (j.L > 0) CK(TIMED(ST_RASTER, raster_tiles_peeled(p.in, j.rs, j.L, ctx->stream)));
     else CK(TIMED(ST_RASTER, raster_tiles(p.in, j.rs, ctx->stream)));
     if (join_late) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_late_join, 0));
+    if (j.L > 1 && (long long)j.L * j.B * j.H * j.W < (1LL << 31)) {
+        // all layers in one launch; the composites' buffer, not written before the shading is
+        // done, holds the list of their pixels to refine (16 (L - 1) bytes per pixel: 4 L and more)
+        ShadeArgs a = layer_args(j, 0);
+        a.refine = reinterpret_cast<int*>(j.acc);
+        CK(TIMED(ST_SHADE, shade_forward(a, ctx->stream, j.L)));
+        return ADMS_OK;
+    }
     if (j.L > 0) {
         for (int l = 0; l < j.L; ++l) CK(TIMED(ST_SHADE, shade_forward(layer_args(j, l), ctx->stream)));
         return ADMS_OK;

@@ -166,7 +166,8 @@ struct ShadeArgs {
     double* g_clip;                  // per-stage calls: [B][V][4] d/d(clip coordinates), or null
 };
 
-cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st);
+// layers > 1: a.keys and a.pre hold that many slices (depth peeling), a.refine as many pixels
+cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers = 1);
 cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st);
 cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st);
 

@@ -449,9 +449,11 @@ __device__ __forceinline__ float tc_lever(const ShadeArgs& A, const PixGeo& g, c
 }
 
 // shading of one listed pixel again, with the refined texture coordinate and LOD
+// (a depth-peeled job's list counts its pixels layer after layer, A.B views each)
 __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
     int hw = A.H * A.W;
     int b = pix / hw, rem = pix - b * hw;
+    if (A.peel) b %= A.B;
     int py = rem / A.W, px = rem - py * A.W;
     int f = key_tri(__ldg(A.keys + (pix)));
     PixGeo g;
@@ -505,9 +507,9 @@ __device__ __forceinline__ float4 shade_covered(const ShadeArgs& A, int b, int p
 }
 
 template <bool INLINE = false, int SHARE = -1>
-__device__ __forceinline__ void shade_fwd_px(const ShadeArgs& A, int b, int px, int py) {
+__device__ __forceinline__ void shade_fwd_px(const ShadeArgs& A, int b, int px, int py, size_t layer = 0) {
     if (px >= A.W || py >= A.H) return;
-    size_t pix = ((size_t)b * A.H + py) * A.W + px;
+    size_t pix = layer + ((size_t)b * A.H + py) * A.W + px;  // layer: first pixel of a peeled layer
     int f = key_tri(__ldg(A.keys + (pix)));
     A.pre[pix] = f >= 0 ? shade_covered<INLINE, SHARE>(A, b, px, py, f, pix) : make_float4(0.f, 0.f, 0.f, 0.f);
 }

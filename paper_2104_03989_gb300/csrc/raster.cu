@@ -293,9 +293,10 @@ __device__ __forceinline__ void near_pack(const Edges<int>& e, int Sx, int Sy, i
 // other threads' updates can only let an unneeded atomicMin through. Without it (closed
 // surfaces, about two fragments per sample) the read would only add a round trip.
 #define ADMS_ROUNDS_MIN (1 << 18)
-#ifndef ADMS_SETUP_BLOCKS
-#define ADMS_SETUP_BLOCKS 4
-#endif
+// resident blocks per SM: 4 (5: 1% faster on the displaced mesh, 3% slower on 11k billboards),
+// 5 with the key read, whose latency the extra warps hide (the canopy's preparation 1.15 ->
+// 1.06 ms; 6: 1.07, 3: 1.29)
+constexpr int setup_blocks(bool zf) { return zf ? 5 : 4; }
 struct DirectTri {  // 80 bytes: 16-byte reads of consecutive slots touch distinct banks
     int4 p, q, r;
     int id;
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(256) k_tile_depth(const unsigned long long* __
 }
 // ZF: compiled with the key read; taken where the job asks for it
 template <bool ZF, int N>
-__global__ void __launch_bounds__(256, ADMS_SETUP_BLOCKS) k_setup(const __grid_constant__ Pack<SetupArgs, N> P) {
+__global__ void __launch_bounds__(256, setup_blocks(ZF)) k_setup(const __grid_constant__ Pack<SetupArgs, N> P) {
     __shared__ DirectTri slots[8][32];
     const SetupArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
     const int* __restrict__ tri = A.tri;
