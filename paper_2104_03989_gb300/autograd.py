@@ -64,11 +64,12 @@ class _RenderLoss(torch.autograd.Function):
     def forward(fctx, ctx, job, views, refs, names, *tensors):
         here, there = torch.cuda.current_stream(), _context_stream(ctx)
         _order(there, here, (refs,))
-        loss = ctx.forward_loss([job], [views], [refs])
+        loss = torch.empty((), dtype=torch.float32, device="cuda")
+        ctx.forward_loss([job], [views], [refs], out_loss=loss)
         _order(here, there)
         fctx.ctx, fctx.job, fctx.names = ctx, job, names
         fctx.shapes = [t.shape for t in tensors]
-        return loss[0].clone()
+        return loss
 
     @staticmethod
     def backward(fctx, g):
@@ -95,11 +96,11 @@ def render_loss(ctx, job, views, refs, lat):
 class _Laplacian(torch.autograd.Function):
     @staticmethod
     def forward(fctx, ctx, job, pos):
-        out = torch.zeros(1, dtype=torch.float32, device=pos.device)
+        out = torch.empty((), dtype=torch.float32, device=pos.device)
         grad = torch.empty_like(pos)
         B.adms_laplacian(ctx.ctx, job, out, grad)
         fctx.save_for_backward(grad)
-        return out[0].clone()
+        return out
 
     @staticmethod
     def backward(fctx, g):

@@ -589,17 +589,37 @@ adms_status prep_job(adms_ctx* ctx, Job& j, bool clear_grads, bool clear_loss, P
     return ADMS_OK;
 }
 
-// join_late: the context's stream waits for the late stream (the job's deferred
-// texture step) before the shading, the first kernel that reads the textures
+// One job's views into its buffer: pageable host memory goes with the launch of its
+// preparation (*by_launch, at most ADMS_PARAM_VIEWS views, not while a stream capture would
+// record the values), anything else is copied in stream order.
+adms_status put_views(adms_ctx* ctx, Job& j, const adms_view* views, int B, const adms_view** by_launch) {
+    *by_launch = nullptr;
+    if (B <= ADMS_PARAM_VIEWS && !ctx->capturing) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        cudaPointerAttributes pa;
+        bool free_stream = cudaStreamIsCapturing(ctx->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+        if (free_stream && cudaPointerGetAttributes(&pa, views) == cudaSuccess && pa.type == cudaMemoryTypeUnregistered) {
+            *by_launch = views;
+            return ADMS_OK;
+        }
+        (void)cudaGetLastError();  // a failed query is no error of this call: the copy below decides
+    }
+    CK(cudaMemcpyAsync(j.views, views, sizeof(adms_view) * B, cudaMemcpyDefault, ctx->stream));
+    return ADMS_OK;
+}
+
 // after the launch of a job's preparation
 void prepared(Job& j, const PrepJob& p) {
     if (p.frame) j.frame_valid = true;
     if (p.lap) j.lap_valid = true;
 }
 
+// join_late: the context's stream waits for the late stream (the job's deferred
+// texture step) before the shading, the first kernel that reads the textures
 adms_status render_core(adms_ctx* ctx, Job& j, bool clear_grads = false, bool clear_loss = false,
-                        bool join_late = false) {
+                        bool join_late = false, const adms_view* host_views = nullptr) {
     PrepJob p;
+    p.host_views = host_views;
     adms_status ps = prep_job(ctx, j, clear_grads, clear_loss, p);
     if (ps) return ps;
     CK(TIMED(ST_RASTER_SETUP, raster_prepare(&p, 1, ctx->stream)));
@@ -934,7 +954,11 @@ adms_status job_create_impl(adms_ctx* ctx, const adms_mesh_desc* mesh, const adm
     AL(j.g_nrm, (size_t)j.V * 6);  // the tangents' gradient follows: one clear per backward
     j.g_tan = j.g_nrm + (size_t)j.V * 3;
     AL(j.g_pos_acc, (size_t)j.V * 3);
-    AL(j.st, 1);
+    {
+        JobCell* cell = nullptr;
+        AL(cell, 1);
+        j.st = &cell->s;
+    }
     bool mips = mat->mips != 0;
     bool pl = j.opt.per_level_textures != 0;
     if (pl && !mips) return fail(ctx, ADMS_ERR_ARG, "per-level textures need mip chains");
@@ -1178,7 +1202,9 @@ extern "C" {
 // ------------------------------------------------------------------ texture steps
 // the Adam updates of the texture latents of jobs js (Eq. 4 moments, clamps, the mip
 // chain rebuilt) on stream st: every job's tiled textures in one launch
-static adms_status texture_adams(adms_ctx* ctx, const std::vector<Job*>& js, cudaStream_t st) {
+// advance (may be null): in the last launch, the job's step counter too where that launch is
+// the tiled textures' one (*advance then null), else it is left to the caller
+static adms_status texture_adams(adms_ctx* ctx, const std::vector<Job*>& js, cudaStream_t st, JobState** advance) {
     std::vector<TexAdam> tiled;
     for (Job* jp : js) {
         Job& j = *jp;
@@ -1197,7 +1223,10 @@ static adms_status texture_adams(adms_ctx* ctx, const std::vector<Job*>& js, cud
             }
         }
     }
-    if (!tiled.empty()) CK(TIMED(ST_ADAM, adam_textures_tiled(tiled, st, ctx->adam_extra_tx)));
+    if (tiled.empty()) return ADMS_OK;
+    JobState* adv = advance && tiled.size() <= ADMS_ADAM_TEX ? *advance : nullptr;
+    CK(TIMED(ST_ADAM, adam_textures_tiled(tiled, st, ctx->adam_extra_tx, adv)));
+    if (adv) *advance = nullptr;
     return ADMS_OK;
 }
 
@@ -1205,9 +1234,10 @@ static adms_status texture_adams(adms_ctx* ctx, const std::vector<Job*>& js, cud
 static adms_status flush_job(adms_ctx* ctx, Job& j) {
     if (!j.tex_pending) return ADMS_OK;
     j.tex_pending = false;
-    adms_status s = texture_adams(ctx, {&j}, ctx->stream);
+    JobState* adv = j.st;
+    adms_status s = texture_adams(ctx, {&j}, ctx->stream, &adv);
     if (s) return s;
-    CK(TIMED(ST_SMALL, advance_step(&j.st, 1, ctx->stream)));
+    if (adv) CK(TIMED(ST_SMALL, advance_step(&adv, 1, ctx->stream)));
     return ADMS_OK;
 }
 static adms_status flush_all(adms_ctx* ctx) {
@@ -1230,9 +1260,10 @@ static adms_status fork_texture_step(adms_ctx* ctx, Job& j, bool* forked) {
     j.tex_pending = false;
     CK(cudaEventRecord(ctx->ev_late_fork, ctx->stream));
     CK(cudaStreamWaitEvent(ctx->late, ctx->ev_late_fork, 0));
-    adms_status s = texture_adams(ctx, {&j}, ctx->late);
+    JobState* adv = j.st;
+    adms_status s = texture_adams(ctx, {&j}, ctx->late, &adv);
     if (s) return s;
-    CK(advance_step(&j.st, 1, ctx->late));
+    if (adv) CK(advance_step(&adv, 1, ctx->late));
     CK(cudaEventRecord(ctx->ev_late_join, ctx->late));
     *forked = true;
     return ADMS_OK;
@@ -1600,8 +1631,9 @@ adms_status adms_render_reference(adms_ctx* ctx, adms_job job, const adms_view* 
     j.W = W * j.S;
     j.PH = H;
     j.PW = W;
-    CK(cudaMemcpyAsync(j.views, views, sizeof(adms_view) * n_views, cudaMemcpyDefault, ctx->stream));
-    if ((s = render_core(ctx, j))) return s;
+    const adms_view* host_views = nullptr;
+    if ((s = put_views(ctx, j, views, n_views, &host_views))) return s;
+    if ((s = render_core(ctx, j, false, false, false, host_views))) return s;
     if (j.S > 1 || j.L > 0) {
         if ((s = j.L > 0 ? peel_composite(ctx, j, nullptr, nullptr, out_rgb)
                          : aa_resolve(ctx, j, nullptr, nullptr, out_rgb)))
@@ -1625,6 +1657,7 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
     if (!ctx || !jobs || n_jobs <= 0 || !views || !views_per_job || !hw || !ref_rgb)
         return fail(ctx, ADMS_ERR_ARG, "invalid forward_loss arguments");
     size_t vofs = 0;
+    bool finished = false;  // a single job's loss, by the last block of its AA + loss
     std::vector<Job*> js;
     std::vector<PrepJob> preps(n_jobs > 1 ? n_jobs : 0);
     for (int k = 0; k < n_jobs; ++k) {
@@ -1651,12 +1684,17 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
         j.ref = ref_rgb[k];
         int norm_views = j.opt.batch_views > 0 ? j.opt.batch_views : B;
         j.loss_scale = (float)(1.0 / (3.0 * (double)norm_views * H * W));
-        CK(cudaMemcpyAsync(j.views, views + vofs, sizeof(adms_view) * B, cudaMemcpyDefault, ctx->stream));
+        const adms_view* host_views = nullptr;
+        if (n_jobs == 1) {
+            if ((s = put_views(ctx, j, views, B, &host_views))) return s;
+        } else {
+            CK(cudaMemcpyAsync(j.views, views + vofs, sizeof(adms_view) * B, cudaMemcpyDefault, ctx->stream));
+        }
         vofs += B;
         if (n_jobs == 1) {
             bool late = false;  // the job's deferred texture step runs beside its frame and raster
             if ((s = fork_texture_step(ctx, j, &late))) return s;
-            if ((s = render_core(ctx, j, true, true, late))) return s;
+            if ((s = render_core(ctx, j, true, true, late, host_views))) return s;
             CK(wait_ref(ctx));
             if (j.L > 0) {
                 if ((s = peel_composite(ctx, j, j.ref, &j.st->call_loss, out_img ? out_img[k] : nullptr))) return s;
@@ -1667,7 +1705,7 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
                 a.ref = j.ref;
                 a.loss_acc = &j.st->call_loss;
                 a.out_img = out_img ? out_img[k] : nullptr;
-                CK(TIMED(ST_AA_LOSS, aa_loss_forward(a, ctx->stream)));
+                CK(TIMED(ST_AA_LOSS, aa_loss_forward(a, ctx->stream, j.st, out_loss, &finished)));
             }
         } else {
             if ((s = flush_job(ctx, j))) return s;
@@ -1692,7 +1730,7 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
     }
     std::vector<JobState*> sts;
     for (Job* jp : js) sts.push_back(jp->st);
-    CK(TIMED(ST_SMALL, finish_call_loss(sts.data(), n_jobs, out_loss, ctx->stream)));
+    if (!finished) CK(TIMED(ST_SMALL, finish_call_loss(sts.data(), n_jobs, out_loss, ctx->stream)));
     for (Job* jp : js) jp->have_fwd = true;
     return ADMS_OK;
 }
@@ -1776,39 +1814,49 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
         adms_status s = flush_job(ctx, *jp);  // a step not yet consumed by a forward_loss
         if (s) return s;
     }
-    // schedules per job (after the Laplacian when no forward computed it for these
-    // positions); then the flat latents (positions with the Laplacian term, skin
-    // weights, displacement) on a branch beside the textures: every job's tiled
-    // textures in one launch; then, joined, the step counters. A pipelined context
-    // issues the flat latents' updates here and defers the texture step.
+    // the schedules (after the Laplacian when no forward computed it for these positions), with
+    // the positions' step where they are optimized; then skin weights and displacement, if
+    // any, on a branch beside the textures; every job's tiled textures in one launch; then,
+    // joined, the step counters. A pipelined context issues the flat latents' updates here and
+    // defers the texture step.
     std::vector<SchedArgs> sched;
     std::vector<PosStepArgs> poss;
     std::vector<JobState*> sts;
+    ClearList fixed;  // gradients of positions that stay
+    bool flat = false;
     for (Job* jp : js) {
         Job& j = *jp;
         if (j.opt.optimize_pos && !j.lap_valid) CK(TIMED(ST_LAPLACIAN, laplacian_forward(lap_args(j), ctx->stream)));
-        sched.push_back(SchedArgs{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV});
-        if (j.opt.optimize_pos) poss.push_back(PosStepArgs{lap_args(j), j.pos, j.m_pos, j.v_pos});
+        SchedArgs sa{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV};
+        if (j.opt.optimize_pos) {
+            poss.push_back(PosStepArgs{lap_args(j), j.pos, j.m_pos, j.v_pos, sa});
+        } else {
+            sched.push_back(sa);
+            if (fixed.n == ADMS_CLEARS) {
+                CK(clear_buffers(fixed, ctx->stream));
+                fixed.n = 0;
+            }
+            fixed.add(j.g_pos, sizeof(float) * 3 * j.LV);
+        }
+        flat = flat || j.g_skin_w || (j.tess && j.opt.optimize_disp);
         sts.push_back(j.st);
     }
-    CK(TIMED(ST_SMALL, schedule_step(sched.data(), n_jobs, ctx->stream)));
+    if (!sched.empty()) CK(TIMED(ST_SMALL, schedule_step(sched.data(), (int)sched.size(), ctx->stream)));
+    CK(clear_buffers(fixed, ctx->stream));
+    if (!poss.empty()) CK(TIMED(ST_LAPLACIAN, position_step(poss.data(), (int)poss.size(), ctx->stream)));
     cudaStream_t bs = ctx->stream;
-    if (!ctx->pipeline) {
+    if (flat && !ctx->pipeline) {
         cudaError_t fe;
         bs = fork_branch(ctx, fe);
         CK(fe);
     }
-    if (!poss.empty()) CK(TIMED(ST_LAPLACIAN, position_step(poss.data(), (int)poss.size(), bs)));
     for (Job* jp : js) {
         Job& j = *jp;
-        if (!j.opt.optimize_pos) CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, bs));
         if (j.g_skin_w)
             CK(TIMED(ST_ADAM, adam_flat(j.skin_w, j.g_skin_w, j.m_skin_w, j.v_skin_w, (long long)j.LV * j.SB, j.st,
                                         bs, j.skin_lr_scale)));
-        if (j.tess) {
-            if (j.opt.optimize_disp)
-                CK(TIMED(ST_ADAM, adam_flat(j.disp, j.g_disp, j.m_disp, j.v_disp, (long long)j.dh * j.dw, j.st, bs)));
-        }
+        if (j.tess && j.opt.optimize_disp)
+            CK(TIMED(ST_ADAM, adam_flat(j.disp, j.g_disp, j.m_disp, j.v_disp, (long long)j.dh * j.dw, j.st, bs)));
     }
     for (Job* jp : js) {
         jp->frame_valid = false;
@@ -1818,10 +1866,12 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
         for (Job* jp : js) jp->tex_pending = true;
         return ADMS_OK;
     }
-    adms_status s = texture_adams(ctx, js, ctx->stream);
+    // a lone job without a branch ends its step in the textures' last launch
+    JobState* adv = n_jobs == 1 && !flat ? sts[0] : nullptr;
+    adms_status s = texture_adams(ctx, js, ctx->stream, adv ? &adv : nullptr);
     if (s) return s;
-    CK(join_branch(ctx));
-    CK(TIMED(ST_SMALL, advance_step(sts.data(), n_jobs, ctx->stream)));
+    if (flat) CK(join_branch(ctx));
+    if (adv || n_jobs > 1 || flat) CK(TIMED(ST_SMALL, advance_step(sts.data(), n_jobs, ctx->stream)));
     return ADMS_OK;
 }
 
@@ -1846,19 +1896,19 @@ adms_status adms_job_fold_gradients(adms_ctx* ctx, adms_job job, float* g_kd, fl
 // zero a job's gradient buffers but for those that `taken` (bit 0 positions, 1 displacement,
 // 2 skin weights, 3 .. 5 textures) says are zero already
 static adms_status zero_gradients(adms_ctx* ctx, Job& j, unsigned taken) {
-    if (!(taken & 1u)) CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, ctx->stream));
-    CK(cudaMemsetAsync(j.g_pos_acc, 0, sizeof(double) * 3 * j.V, ctx->stream));
-    if (j.tess) {
-        CK(cudaMemsetAsync(j.g_rpos, 0, sizeof(float) * 3 * j.V, ctx->stream));
-        CK(cudaMemsetAsync(j.g_bpos_acc, 0, sizeof(double) * 3 * j.LV, ctx->stream));
-    }
-    if (j.skin) CK(cudaMemsetAsync(j.g_rpos, 0, sizeof(float) * 3 * j.V, ctx->stream));
-    if (j.g_skin_w && !(taken & 4u)) CK(cudaMemsetAsync(j.g_skin_w, 0, sizeof(float) * j.LV * j.SB, ctx->stream));
-    if (j.g_disp && !(taken & 2u)) CK(cudaMemsetAsync(j.g_disp, 0, sizeof(float) * j.dh * j.dw, ctx->stream));
+    ClearList c;
+    if (!(taken & 1u)) c.add(j.g_pos, sizeof(float) * 3 * j.LV);
+    c.add(j.g_pos_acc, sizeof(double) * 3 * j.V);
+    if (j.tess || j.skin) c.add(j.g_rpos, sizeof(float) * 3 * j.V);
+    if (j.tess) c.add(j.g_bpos_acc, sizeof(double) * 3 * j.LV);
+    if (j.g_skin_w && !(taken & 4u)) c.add(j.g_skin_w, sizeof(float) * j.LV * j.SB);
+    if (j.g_disp && !(taken & 2u)) c.add(j.g_disp, sizeof(float) * j.dh * j.dw);
     TexState* maps[3] = {&j.kd, &j.orm, &j.nrm};
-    for (int m = 0; m < 3; ++m)
-        if (maps[m]->grad && !(taken & (8u << m)))
-            CK(cudaMemsetAsync(maps[m]->grad, 0, sizeof(float4) * maps[m]->total, ctx->stream));
+    for (int m = 0; m < 3; ++m) {  // (taken: level 0 is clear, the coarser levels follow)
+        size_t first = taken & (8u << m) ? (size_t)maps[m]->w * maps[m]->h : 0;
+        if (maps[m]->grad) c.add(maps[m]->grad + first, sizeof(float4) * (maps[m]->total - first));
+    }
+    CK(clear_buffers(c, ctx->stream));
     return ADMS_OK;
 }
 
@@ -1888,12 +1938,11 @@ adms_status adms_job_take_gradients(adms_ctx* ctx, adms_job job, const float* sc
     for (int m = 0; m < 3; ++m) {
         if (!outs[m]) continue;
         TexDev t = maps[m]->dev();
-        if (maps[m]->per_level) t.levels = 1;  // level 0's own gradient; the chain is cleared below
-        else taken |= 8u << m;
+        if (maps[m]->per_level) t.levels = 1;  // level 0's own gradient
+        taken |= 8u << m;
         ts[n] = t;
         to[n++] = reinterpret_cast<float4*>(outs[m]);
     }
-    CK(take_mip_gradients(ts, to, n, scale, ctx->stream));
     FlatTake f{};
     f.g[0] = j.g_pos;
     f.out[0] = g_pos;
@@ -1904,7 +1953,7 @@ adms_status adms_job_take_gradients(adms_ctx* ctx, adms_job job, const float* sc
     f.g[2] = j.g_skin_w;
     f.out[2] = g_skin_w;
     f.n[2] = g_skin_w ? (long long)j.LV * j.SB : 0;
-    CK(take_flat_gradients(f, scale, ctx->stream));
+    CK(take_gradients(ts, to, n, f, scale, ctx->stream));
     taken |= (g_pos ? 1u : 0u) | (g_disp ? 2u : 0u) | (g_skin_w ? 4u : 0u);
     return zero_gradients(ctx, j, taken);
 }

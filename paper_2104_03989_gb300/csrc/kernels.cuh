@@ -168,7 +168,10 @@ struct ShadeArgs {
 
 // layers > 1: a.keys and a.pre hold that many slices (depth peeling), a.refine as many pixels
 cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers = 1);
-cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st);
+// finish (may be null) of an opaque job of up to ADMS_FINISH_BLOCKS blocks: the last block also does
+// finish_call_loss(finish, out); *finished tells whether it will
+cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st, struct JobState* finish = nullptr, float* out = nullptr,
+                            bool* finished = nullptr);
 cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st);
 
 // per-pixel resolve of a supersampled render: pixel = mean of its s x s antialiased
@@ -303,6 +306,32 @@ struct JobState {
     int status_next;   // latched by the optimizer step's kernels, folded into status when t advances
 };
 
+static_assert(sizeof(JobState) == 64, "the job state is part of the checkpoint format");
+// a job's state and, beside it (not checkpointed), the block counters of the kernels whose last
+// block finishes for the job; zero between launches
+struct JobCell {
+    JobState s;
+    unsigned ticket[4];
+};
+enum { TICKET_LOSS = 0, TICKET_POS, TICKET_TEX };
+// true in the last of n blocks (in the one thread of each that calls it, after the block's
+// other threads' work is ordered before it by a barrier)
+__device__ __forceinline__ bool last_block(JobState* s, int which, unsigned n) {
+    __threadfence();
+    bool last = atomicInc(&reinterpret_cast<JobCell*>(s)->ticket[which], n - 1) == n - 1;
+    if (last) __threadfence();
+    return last;
+}
+
+// the end of a forward call: the loss to out (may be null) and to the step's sum; a NaN or
+// infinite one is latched (the optimizer skips the job)
+__device__ __forceinline__ void finish_job_loss(JobState* s, float* out) {
+    double loss = *reinterpret_cast<volatile double*>(&s->call_loss);
+    if (out) *out = (float)loss;
+    s->img_loss += loss;
+    if (!isfinite(loss)) s->status = ADMS_ERR_NONFINITE;
+}
+
 struct LapArgs {
     int V;
     const float* pos;       // [V][3]
@@ -327,11 +356,14 @@ struct PrepJob {
     void* clear[ADMS_PREP_CLEARS];       // 4-byte aligned
     size_t clear_bytes[ADMS_PREP_CLEARS];  // multiples of 4
     int n_clear = 0;
+    // the job's views in pageable host memory, to be copied into in.views; null: they are there
+    const adms_view* host_views = nullptr;
     void add_clear(void* p, size_t bytes) {
         clear[n_clear] = p;
         clear_bytes[n_clear++] = bytes;
     }
 };
+#define ADMS_PARAM_VIEWS 16  // views of a single job that travel as launch parameters
 cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st);
 // *out = L_delta after laplacian_forward
 cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st);
@@ -340,15 +372,29 @@ cudaError_t laplacian_gradient(const LapArgs& a, float scale, cudaStream_t st);
 #define ADMS_MIP_TEX 3  // textures per fold or rebuild launch (a job's maps)
 // level-0 texture gradient with the mip-chain adjoint folded in
 cudaError_t fold_mip_gradient(const TexDev& t, float4* out, cudaStream_t st);
-// the same for n <= 3 textures, times *scale (null: 1), the gradient chains then zero
-cudaError_t take_mip_gradients(const TexDev* ts, float4* const* outs, int n, const float* scale, cudaStream_t st);
-// out[k][0 .. n[k]) = g[k] times *scale (null: 1), g[k] = 0
+// the same for n <= 3 textures, times *scale (null: 1), their level-0 gradients then zero;
+// and, for flat gradients, out[k][0 .. n[k]) = g[k] times *scale, g[k] = 0
 struct FlatTake {
     float* g[3];
     float* out[3];
     long long n[3];
 };
-cudaError_t take_flat_gradients(const FlatTake& a, const float* scale, cudaStream_t st);
+cudaError_t take_gradients(const TexDev* ts, float4* const* outs, int n, const FlatTake& flat, const float* scale,
+                           cudaStream_t st);
+// several buffers to zero in one launch (4-byte words; 16-byte stores where aligned)
+struct ClearSeg {
+    int* p;
+    long long n;
+};
+#define ADMS_CLEARS 12
+struct ClearList {
+    ClearSeg z[ADMS_CLEARS];
+    int n = 0;
+    void add(void* p, size_t bytes) {
+        if (p && bytes) z[n++] = ClearSeg{static_cast<int*>(p), (long long)(bytes / 4)};
+    }
+};
+cudaError_t clear_buffers(const ClearList& c, cudaStream_t st);
 
 struct SchedArgs {
     JobState* st;
@@ -358,10 +404,12 @@ struct SchedArgs {
 };
 cudaError_t schedule_step(const SchedArgs* as, int n, cudaStream_t st);
 
-// the positions' step: g += lambda_t dL_delta/dpos (Eq. 4), Adam (no clamps), g = 0
+// the schedules of a job that optimizes its positions, and their step: g += lambda_t
+// dL_delta/dpos (Eq. 4), Adam (no clamps), g = 0
 struct PosStepArgs {
     LapArgs lap;
     float *p, *m, *v;  // [V][3]
+    SchedArgs sched;
 };
 cudaError_t position_step(const PosStepArgs* as, int n, cudaStream_t st);
 
@@ -408,7 +456,9 @@ cudaError_t adam_prepare();
 cudaError_t adam_encode_maps(const TexDev& t, const float4* m, const float4* v, CUtensorMap out[4]);
 // Adam + mip rebuild of every listed texture (all adam_tiled, any jobs), one 32x32-texel
 // tile per block, one launch per ADMS_ADAM_TEX textures
-cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uint32_t extra_tx = 0);
+// advance (may be null; one launch only): the job whose step ends with this call, as advance_step
+cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uint32_t extra_tx = 0,
+                                JobState* advance = nullptr);
 cudaError_t advance_step(JobState* const* js, int n, cudaStream_t st);
 // out[k] = the latched status of job k (stream-ordered; out: device [n])
 #define ADMS_STATUS_MAX 512

@@ -11,12 +11,21 @@ namespace adms {
 
 constexpr float kLog2_10 = 3.32192809488736234787f;
 
-// lambda_t (Eq. 5 text, recursive reading), lambda_0 heuristic, lr_t, bias corrections
-__device__ __forceinline__ void schedule_job(const SchedArgs& a) {
-    JobState* s = a.st;
+// lambda_t (Eq. 5 text, recursive reading), lambda_0 heuristic, lr_t, bias corrections of a
+// job's step, from its state; nothing is written
+struct Schedule {
+    float lam, lam0, lr, bc1, bc2, l_img, l_lap;
+    int status;
+};
+__device__ __forceinline__ Schedule schedule_of(const SchedArgs& a) {
+    const JobState* s = a.st;
+    Schedule o;
     int t = s->t;
     double l_img = s->img_loss;
     double l_lap = a.has_pos ? s->lap_sum / (double)a.n_verts : 0.0;
+    o.lam = s->lam;
+    o.lam0 = s->lam0;
+    o.status = s->status;
     if (a.has_pos) {
         if (t == 0) {
             double lam0 = a.lambda0_user;
@@ -25,40 +34,54 @@ __device__ __forceinline__ void schedule_job(const SchedArgs& a) {
                     lam0 = 0.25 * l_img / l_lap;
                 } else {
                     lam0 = 0.0;
-                    s->status = ADMS_ERR_ARG;
+                    o.status = ADMS_ERR_ARG;
                 }
             }
-            s->lam0 = (float)lam0;
-            s->lam = (float)lam0;
+            o.lam0 = (float)lam0;
+            o.lam = (float)lam0;
         } else {
             double lmin = 0.02 * (double)s->lam0;
-            s->lam = (float)(((double)s->lam - lmin) * (double)exp2f(-1e-6f * kLog2_10 * (float)t) + lmin);
+            o.lam = (float)(((double)s->lam - lmin) * (double)exp2f(-1e-6f * kLog2_10 * (float)t) + lmin);
         }
     }
     // float32 transcendentals: float64 ones cost ~10 us on one thread here; the
     // results are float32 and within a few ulp of the float64 values
-    s->lr = a.lr0 * exp2f(-0.0002f * kLog2_10 * (float)t);
-    s->bc1 = -expm1f((float)(t + 1) * log1pf(-0.1f));   // 1 - 0.9^(t+1)
-    s->bc2 = -expm1f((float)(t + 1) * log1pf(-0.001f)); // 1 - 0.999^(t+1)
-    s->last_img_loss = (float)l_img;
-    s->last_lap = (float)l_lap;
+    o.lr = a.lr0 * exp2f(-0.0002f * kLog2_10 * (float)t);
+    o.bc1 = -expm1f((float)(t + 1) * log1pf(-0.1f));   // 1 - 0.9^(t+1)
+    o.bc2 = -expm1f((float)(t + 1) * log1pf(-0.001f)); // 1 - 0.999^(t+1)
+    o.l_img = (float)l_img;
+    o.l_lap = (float)l_lap;
+    return o;
+}
+__device__ __forceinline__ void write_schedule(JobState* s, const Schedule& o) {
+    s->lam = o.lam;
+    s->lam0 = o.lam0;
+    s->lr = o.lr;
+    s->bc1 = o.bc1;
+    s->bc2 = o.bc2;
+    s->last_img_loss = o.l_img;
+    s->last_lap = o.l_lap;
+    s->status = o.status;
     s->img_loss = 0.0;
 }
 
 // the scalar kernels: one block per job, one launch for the jobs of a call
 template <int N>
 __global__ void k_schedule(const __grid_constant__ Pack<SchedArgs, N> P) {
-    schedule_job(P.a[N == 1 ? 0 : blockIdx.y]);
+    const SchedArgs& a = P.a[N == 1 ? 0 : blockIdx.y];
+    write_schedule(a.st, schedule_of(a));
 }
 cudaError_t schedule_step(const SchedArgs* as, int n, cudaStream_t st) {
     return launch_packed(as, n, 1, st, k_schedule<1>, k_schedule<ADMS_BATCH_JOBS>, [](const SchedArgs&) { return 1; });
 }
 
-template <int N>
-__global__ void k_advance(const __grid_constant__ Pack<JobState*, N> P) {
-    JobState* s = P.a[N == 1 ? 0 : blockIdx.y];
+__device__ __forceinline__ void advance_job(JobState* s) {
     s->t += 1;
     if (s->status_next) s->status = s->status_next;
+}
+template <int N>
+__global__ void k_advance(const __grid_constant__ Pack<JobState*, N> P) {
+    advance_job(P.a[N == 1 ? 0 : blockIdx.y]);
 }
 
 struct FinishArgs {
@@ -68,10 +91,7 @@ struct FinishArgs {
 template <int N>
 __global__ void k_finish_call(const __grid_constant__ Pack<FinishArgs, N> P) {
     const FinishArgs& a = P.a[N == 1 ? 0 : blockIdx.y];
-    JobState* s = a.s;
-    if (a.out) *a.out = (float)s->call_loss;
-    s->img_loss += s->call_loss;
-    if (!isfinite(s->call_loss)) s->status = ADMS_ERR_NONFINITE;  // latched: the optimizer skips the job
+    finish_job_loss(a.s, a.out);
 }
 
 struct StatusPtrs {
@@ -142,31 +162,42 @@ cudaError_t adam_flat(float* p, float* g, float* m, float* v, long long n, const
     return cudaGetLastError();
 }
 
-// The positions' step: one thread per vertex gathers the Laplacian's gradient and applies
-// Adam to its three coordinates (two launches and a pass over the gradient before). A latched
-// job is left as it is.
+// The schedules and the positions' step: one thread per vertex gathers the Laplacian's
+// gradient and applies Adam to its three coordinates. Each block works the schedules out from
+// the state of before the step; the last one writes them. (Three launches and a pass over the
+// gradient before.) A latched job is left as it is.
 template <int N>
 __global__ void __launch_bounds__(128) k_position_step(const __grid_constant__ Pack<PosStepArgs, N> P) {
+    __shared__ Schedule sh;
     const PosStepArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
     const LapArgs& a = A.lap;
+    int blocks = (a.V + 127) / 128;
+    if ((int)blockIdx.x >= blocks) return;
     int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.V || a.st->status) return;
-    float scale = 2.f * a.st->lam / (float)a.V;
-    float3 g = f3(a.delta[3 * k], a.delta[3 * k + 1], a.delta[3 * k + 2]);
-    ring_adjoint(a, k, g);
-    float lr = a.st->lr, bc1 = a.st->bc1, bc2 = a.st->bc2;
-    float gl[3] = {g.x, g.y, g.z};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        int i = 3 * k + c;
-        float gi = a.g_pos[i] + scale * gl[c];
-        float mm = A.m[i], vv = A.v[i];
-        latch_nonfinite(a.st, gi);
-        A.p[i] = adam1(A.p[i], gi, mm, vv, lr, bc1, bc2);
-        A.m[i] = mm;
-        A.v[i] = vv;
-        a.g_pos[i] = 0.f;
+    if (threadIdx.x == 0) sh = schedule_of(A.sched);
+    float3 g = zero3();
+    if (k < a.V) {
+        g = f3(a.delta[3 * k], a.delta[3 * k + 1], a.delta[3 * k + 2]);
+        ring_adjoint(a, k, g);
     }
+    __syncthreads();
+    if (k < a.V && !sh.status) {
+        float scale = 2.f * sh.lam / (float)a.V;
+        float lr = sh.lr, bc1 = sh.bc1, bc2 = sh.bc2;
+        float gl[3] = {g.x, g.y, g.z};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            int i = 3 * k + c;
+            float gi = a.g_pos[i] + scale * gl[c];
+            float mm = A.m[i], vv = A.v[i];
+            latch_nonfinite(a.st, gi);
+            A.p[i] = adam1(A.p[i], gi, mm, vv, lr, bc1, bc2);
+            A.m[i] = mm;
+            A.v[i] = vv;
+            a.g_pos[i] = 0.f;
+        }
+    }
+    if (threadIdx.x == 0 && last_block(a.st, TICKET_POS, blocks)) write_schedule(a.st, sh);
 }
 cudaError_t position_step(const PosStepArgs* as, int n, cudaStream_t st) {
     return launch_packed(as, n, 128, st, k_position_step<1>, k_position_step<ADMS_BATCH_JOBS>,
@@ -595,11 +626,15 @@ __device__ __forceinline__ void mip_top(const TexDev& t, float4* s) {
     }
 }
 
-__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_adam_mip_top(const __grid_constant__ TexAdamBatch P) {
+// advance: the job whose step this launch ends (the last block advances it), or null
+__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_adam_mip_top(const __grid_constant__ TexAdamBatch P,
+                                                                       JobState* advance) {
     __shared__ float4 s[ADMS_MIP_TOP_THREADS];
     const TexAdam& A = P.a[blockIdx.x];
-    if (A.js->status) return;
-    mip_top<true>(A.t, s);
+    if (!A.js->status) mip_top<true>(A.t, s);
+    if (!advance) return;
+    __syncthreads();  // every thread has read the status
+    if (threadIdx.x == 0 && last_block(advance, TICKET_TEX, gridDim.x)) advance_job(advance);
 }
 
 bool adam_tiled(const TexDev& t) { return t.levels > 5 && (t.w0 % 32) == 0 && (t.h0 % 32) == 0; }
@@ -632,7 +667,8 @@ cudaError_t adam_encode_maps(const TexDev& t, const float4* m, const float4* v, 
     return cudaSuccess;
 }
 
-cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uint32_t extra_tx) {
+cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uint32_t extra_tx, JobState* advance) {
+    if (advance && list.size() > ADMS_ADAM_TEX) return cudaErrorInvalidValue;
     static int sms = 0;
     if (!sms) {
         int dev = 0;
@@ -658,7 +694,7 @@ cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uin
         P.extra_tx = extra_tx;
         int blocks = std::min(tiles, std::max(1, sms * ADMS_ADAM_GRID_PCT / 100));
         k_adam_tex_stream<<<blocks, ADMS_ADAM_THREADS, sizeof(AdamSmem), st>>>(P, tiles);
-        k_adam_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P);
+        k_adam_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P, advance);
         count_launches(2);
         cudaError_t e = cudaGetLastError();
         if (e) return e;
@@ -691,9 +727,23 @@ struct FoldBatch {
     int n;
     const float* scale;
     int take;
+    int tex_blocks;  // the blocks after them take the flat gradients
+    FlatTake flat;
 };
 __global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ FoldBatch P) {
     int e = 0, block = blockIdx.x;
+    if (block >= P.tex_blocks) {
+        long long i = (long long)(block - P.tex_blocks) * 256 + threadIdx.x;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (i >= 0 && i < P.flat.n[k]) {
+                P.flat.out[k][i] = P.scale ? P.flat.g[k][i] * *P.scale : P.flat.g[k][i];
+                P.flat.g[k][i] = 0.f;
+            }
+            i -= P.flat.n[k];
+        }
+        return;
+    }
     while (e + 1 < P.n && P.block0[e + 1] <= block) ++e;
     const TexDev& t = P.t[e];
     block -= P.block0[e];
@@ -732,12 +782,13 @@ __global__ void __launch_bounds__(256) k_fold_mips(const __grid_constant__ FoldB
     }
 }
 
-static cudaError_t fold_batch(const TexDev* ts, float4* const* outs, int n, const float* scale, bool take,
-                              cudaStream_t st) {
+static cudaError_t fold_batch(const TexDev* ts, float4* const* outs, int n, const FlatTake* flat, const float* scale,
+                              bool take, cudaStream_t st) {
     FoldBatch P;
     P.n = n;
     P.scale = scale;
     P.take = take;
+    P.flat = flat ? *flat : FlatTake{};
     int blocks = 0;
     for (int j = 0; j < n; ++j) {
         const TexDev& t = ts[j];
@@ -750,43 +801,39 @@ static cudaError_t fold_batch(const TexDev* ts, float4* const* outs, int n, cons
         for (int k = 1; k < ADMS_MAX_LEVELS; ++k)
             P.w[j][k] = P.w[j][k - 1] / (float)(((t.w0 >> (k - 1)) > 1 ? 2 : 1) * ((t.h0 >> (k - 1)) > 1 ? 2 : 1));
     }
-    if (n <= 0) return cudaSuccess;
+    P.tex_blocks = blocks;
+    blocks += (int)((P.flat.n[0] + P.flat.n[1] + P.flat.n[2] + 255) / 256);
+    if (blocks <= 0) return cudaSuccess;
     k_fold_mips<<<blocks, 256, 0, st>>>(P);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t fold_mip_gradient(const TexDev& t, float4* out, cudaStream_t st) {
-    return fold_batch(&t, &out, 1, nullptr, false, st);
+    return fold_batch(&t, &out, 1, nullptr, nullptr, false, st);
 }
-cudaError_t take_mip_gradients(const TexDev* ts, float4* const* outs, int n, const float* scale, cudaStream_t st) {
-    cudaError_t e = fold_batch(ts, outs, n, scale, true, st);
-    for (int j = 0; j < n && !e; ++j) {  // the coarser levels, once every reader is done
-        const TexDev& t = ts[j];
-        if (t.levels <= 1) continue;
-        int last = t.levels - 1;
-        size_t end = t.off[last] + (size_t)max(t.w0 >> last, 1) * max(t.h0 >> last, 1);
-        e = cudaMemsetAsync(t.grad + t.off[1], 0, (end - t.off[1]) * sizeof(float4), st);
-    }
-    return e;
+cudaError_t take_gradients(const TexDev* ts, float4* const* outs, int n, const FlatTake& flat, const float* scale,
+                           cudaStream_t st) {
+    return fold_batch(ts, outs, n, &flat, scale, true, st);
 }
 
-// out = scale g, g = 0 over up to three flat gradients (positions, displacement, skin weights)
-__global__ void k_take_flat(const FlatTake a, const float* scale) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        if (i >= 0 && i < a.n[k]) {
-            a.out[k][i] = scale ? a.g[k][i] * *scale : a.g[k][i];
-            a.g[k][i] = 0.f;
-        }
-        i -= a.n[k];
+__global__ void __launch_bounds__(256) k_clear(const __grid_constant__ ClearList c) {
+    long long t = (long long)blockIdx.x * 256 + threadIdx.x, step = (long long)gridDim.x * 256;
+    for (int k = 0; k < c.n; ++k) {
+        int* p = c.z[k].p;
+        long long n = c.z[k].n, n4 = (reinterpret_cast<uintptr_t>(p) & 15) ? 0 : n / 4;
+        int4 zero = make_int4(0, 0, 0, 0);
+        for (long long i = t; i < n4; i += step) reinterpret_cast<int4*>(p)[i] = zero;
+        for (long long i = 4 * n4 + t; i < n; i += step) p[i] = 0;
     }
 }
-cudaError_t take_flat_gradients(const FlatTake& a, const float* scale, cudaStream_t st) {
-    long long n = a.n[0] + a.n[1] + a.n[2];
+cudaError_t clear_buffers(const ClearList& c, cudaStream_t st) {
+    long long n = 0;
+    for (int k = 0; k < c.n; ++k) n += c.z[k].n;
     if (n <= 0) return cudaSuccess;
-    k_take_flat<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, scale);
+    // eight 16-byte stores per thread, at most a few waves
+    int blocks = (int)std::min<long long>(std::max<long long>(n / (256 * 32), 1), 152 * 32);
+    k_clear<<<blocks, 256, 0, st>>>(c);
     count_launches(1);
     return cudaGetLastError();
 }

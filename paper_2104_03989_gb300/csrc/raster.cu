@@ -86,13 +86,16 @@ __device__ __forceinline__ void transform_vertex(const float* __restrict__ pos, 
     vs[i] = o;
 }
 
+// A single job's views in pageable host memory come with the launch: the vertices are
+// transformed from the parameters and block 0 writes them to the job's buffer for the kernels
+// that follow (a pageable copy costs the host 9 us).
+struct ViewSet {
+    adms_view v[ADMS_PARAM_VIEWS];
+    int n;
+};
 // The first launch of a raster pass: the first nb_vert blocks of a job transform its vertices,
 // the rest set its keys to empty and clear the tile counts and whatever else of 4-byte words
 // the pass needs at zero (four memset launches before).
-struct ClearSeg {
-    int* p;
-    long long n;
-};
 #define ADMS_BEGIN_CLEARS (ADMS_PREP_CLEARS + 3)
 struct BeginArgs {
     const float* pos;
@@ -106,12 +109,17 @@ struct BeginArgs {
     int V, B, W, H, nb_vert, nb_fill;
 };
 template <int N>
-__global__ void __launch_bounds__(256) k_begin(const __grid_constant__ Pack<BeginArgs, N> P) {
+__device__ __forceinline__ void begin_body(const Pack<BeginArgs, N>& P, const ViewSet* vs) {
     const BeginArgs& A = P.a[N == 1 ? 0 : blockIdx.y];
     int blk = blockIdx.x;
+    if (vs && blk == 0) {
+        int* to = reinterpret_cast<int*>(const_cast<adms_view*>(A.views));
+        const int* from = reinterpret_cast<const int*>(vs->v);
+        for (int i = threadIdx.x; i < vs->n * (int)(sizeof(adms_view) / 4); i += 256) to[i] = from[i];
+    }
     if (blk < A.nb_vert) {
         int i = blk * 256 + threadIdx.x;
-        if (i < A.B * A.V) transform_vertex(A.pos, A.V, A.views, A.W, A.H, A.clip, A.vs, A.scr, i);
+        if (i < A.B * A.V) transform_vertex(A.pos, A.V, vs ? vs->v : A.views, A.W, A.H, A.clip, A.vs, A.scr, i);
         return;
     }
     blk -= A.nb_vert;
@@ -127,6 +135,14 @@ __global__ void __launch_bounds__(256) k_begin(const __grid_constant__ Pack<Begi
 #pragma unroll
     for (int k = 0; k < ADMS_BEGIN_CLEARS; ++k)
         for (long long i = t; i < A.z[k].n; i += step) A.z[k].p[i] = 0;
+}
+template <int N>
+__global__ void __launch_bounds__(256) k_begin(const __grid_constant__ Pack<BeginArgs, N> P) {
+    begin_body(P, nullptr);
+}
+__global__ void __launch_bounds__(256) k_begin_views(const __grid_constant__ Pack<BeginArgs, 1> P,
+                                                     const __grid_constant__ ViewSet vs) {
+    begin_body(P, &vs);
 }
 
 // ---------------------------------------------------------------- tile-list allocation
@@ -879,8 +895,21 @@ cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
         frame = frame || f.nb_frame || f.nb_lap;
     }
     constexpr int M = ADMS_BATCH_JOBS;
-    cudaError_t e = launch_packed(begin.data(), n, 256, st, k_begin<1>, k_begin<M>,
-                                  [](const BeginArgs& a) { return a.nb_vert + a.nb_fill; });
+    cudaError_t e = cudaSuccess;
+    if (n == 1 && jobs[0].host_views) {
+        Pack<BeginArgs, 1> p;
+        p.a[0] = begin[0];
+        ViewSet vs;
+        vs.n = jobs[0].in.B;
+        if (vs.n > ADMS_PARAM_VIEWS) return cudaErrorInvalidValue;
+        memcpy(vs.v, jobs[0].host_views, sizeof(adms_view) * vs.n);
+        k_begin_views<<<begin[0].nb_vert + begin[0].nb_fill, 256, 0, st>>>(p, vs);
+        count_launches(1);
+        e = cudaGetLastError();
+    } else {
+        e = launch_packed(begin.data(), n, 256, st, k_begin<1>, k_begin<M>,
+                          [](const BeginArgs& a) { return a.nb_vert + a.nb_fill; });
+    }
     auto tri_blocks = [](const SetupArgs& a) { return (a.B * a.F + 255) / 256; };
     if (!e && zf && n == 1 && (long long)setup[0].B * setup[0].F >= ADMS_ROUNDS_MIN) {
         // tile_off holds the tiles' depths until the list allocation writes it

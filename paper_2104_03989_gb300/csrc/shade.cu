@@ -55,14 +55,16 @@ __global__ void __launch_bounds__(ADMS_FWD_THREADS, fwd_blocks(INLINE, SHARE)) k
     shade_fwd_px<INLINE, SHARE>(A, blockIdx.y, px, py, (size_t)blockIdx.z * ((size_t)A.B * A.H * A.W));
 }
 
-template <bool PEEL>
-__global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(ShadeArgs A) {
+// FINISH: the last block finishes the call's loss (a launch of its own otherwise)
+template <bool PEEL, bool FINISH>
+__global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(ShadeArgs A, JobState* fin, float* out) {
     __shared__ float red[ADMS_AA_THREADS / 16];
     int bx = (A.W + 31) / 32;  // a warp takes 32 columns of one row
     LossSum sum;
     aa_pixel<PEEL>(A, blockIdx.y, (blockIdx.x % bx) * 32 + (threadIdx.x & 31),
                    (blockIdx.x / bx) * (ADMS_AA_THREADS / 32) + (threadIdx.x >> 5), sum);
     add_block_loss(A, sum, red);
+    if (FINISH && threadIdx.x == 0 && last_block(fin, TICKET_LOSS, gridDim.x * gridDim.y)) finish_job_loss(fin, out);
 }
 
 // resident blocks per SM of the fused backward (register cap 65536 / (threads x this))
@@ -336,11 +338,16 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers) {
     }
     return cudaGetLastError();
 }
-cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st) {
+// up to this many blocks (one view of 512x512), where a pass is bound by the host's launches;
+// at 16384 blocks the counter costs what the launch does (49.4 us against 45.0 + 5.1)
+#define ADMS_FINISH_BLOCKS 2048
+cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st, JobState* finish, float* out, bool* finished) {
     int rows = ADMS_AA_THREADS / 32;
     dim3 grid(((a.W + 31) / 32) * ((a.H + rows - 1) / rows), a.B);
-    auto k = a.peel ? k_aa_loss<true> : k_aa_loss<false>;
-    k<<<grid, ADMS_AA_THREADS, 0, st>>>(a);
+    bool fin = finish && !a.peel && a.loss_acc && (long long)grid.x * grid.y <= ADMS_FINISH_BLOCKS;
+    if (finished) *finished = fin;
+    auto k = a.peel ? k_aa_loss<true, false> : fin ? k_aa_loss<false, true> : k_aa_loss<false, false>;
+    k<<<grid, ADMS_AA_THREADS, 0, st>>>(a, finish, out);
     count_launches(1);
     return cudaGetLastError();
 }

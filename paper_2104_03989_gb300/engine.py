@@ -180,7 +180,7 @@ class Context:
         vpj = [len(v) for v in views_list]
         hw = [(int(r.shape[1]), int(r.shape[2])) for r in refs]
         if out_loss is None:
-            out_loss = torch.zeros(len(jobs), dtype=torch.float32, device="cuda")
+            out_loss = torch.empty(len(jobs), dtype=torch.float32, device="cuda")  # written whole by the call
         B.adms_forward_loss(self.ctx, list(jobs), views, vpj, hw, refs, out_loss, out_img)
         self._keep["fwd"] = (views, refs)
         return out_loss
