@@ -328,24 +328,37 @@ __host__ __device__ __forceinline__ bool shared_taps(const ShadeArgs& A) {
            A.kd.levels == A.orm.levels && A.kd.levels == A.nrm.levels;
 }
 
-// tex_sample of the three maps with shared taps (the same arithmetic, map by map)
+// a map of one texel has that value everywhere: no footprint, no dependence on the coordinate
+__host__ __device__ __forceinline__ bool constant_map(const TexDev& t) { return t.w0 == 1 && t.h0 == 1; }
+
+// How a launch of its own kernel (SHARE) samples the maps: 1 all three share their taps, 2 orm
+// and nrm do (a base colour of a finer or coarser size, or a constant one), 0 every map has its own.
+__host__ __device__ __forceinline__ int share_of(const ShadeArgs& A) {
+    if (shared_taps(A)) return 1;
+    bool pair = A.orm.w0 == A.nrm.w0 && A.orm.h0 == A.nrm.h0 && A.orm.levels == A.nrm.levels;
+    return pair && !constant_map(A.nrm) ? 2 : 0;
+}
+
+// tex_sample of the maps FROM .. 2 with shared taps (the same arithmetic, map by map)
+template <int FROM = 0>
 __device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3]) {
     const float4* ts[3] = {A.kd.tex, A.orm.tex, A.nrm.tex};
+    const TexDev& t = FROM == 0 ? A.kd : A.orm;
     int l0 = (int)floorf(lod);
     float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, A.kd.levels - 1);
+    int l1 = min(l0 + 1, t.levels - 1);
 #pragma unroll
-    for (int m = 0; m < 3; ++m) out[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int m = FROM; m < 3; ++m) out[m] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         int k = s == 0 ? l0 : l1;
         float wl = s == 0 ? 1.f - fr : fr;
         if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(A.kd, k, tc);
+        BilinTap b = bilin_tap(t, k, tc);
         float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
         float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
+        for (int m = FROM; m < 3; ++m) {
             out[m] = f4madd(out[m], w00, __ldg(ts[m] + b.idx[0]));
             out[m] = f4madd(out[m], w10, __ldg(ts[m] + b.idx[1]));
             out[m] = f4madd(out[m], w01, __ldg(ts[m] + b.idx[2]));
@@ -354,10 +367,14 @@ __device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& 
     }
 }
 
+__device__ __forceinline__ float4 map_sample(const TexDev& t, const TexCoord& tc, float lod) {
+    return constant_map(t) ? __ldg(t.tex) : tex_sample(t, tc, lod);
+}
+
 // the shading inputs at g: interpolated attributes and the three maps' trilinear samples
 // (their LODs into lod). One LOD and one footprint per level serve maps of one size (57.2 ->
 // 44.0 M warp instructions, 83 -> 73.5 us for 8 views of 512x512).
-// SHARE: 1 the maps are of one size, 0 not all, -1 decided here (batched and per-stage calls).
+// SHARE: share_of, -1 decided here between 1 and 0 (batched and per-stage calls).
 template <int SHARE = -1>
 __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo& g, float lod[3]) {
     ShadeIn in;
@@ -372,12 +389,19 @@ __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo
         in.kd = smp[0];
         in.orm = smp[1];
         in.nm = smp[2];
+    } else if (SHARE == 2) {
+        lod[1] = lod[2] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
+        float4 smp[3];
+        tex_sample3<1>(A, g.tc, lod[1], smp);
+        in.kd = map_sample(A.kd, g.tc, lod[0]);
+        in.orm = smp[1];
+        in.nm = smp[2];
     } else {
         lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
         lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
-        in.kd = tex_sample(A.kd, g.tc, lod[0]);
-        in.orm = tex_sample(A.orm, g.tc, lod[1]);
-        in.nm = tex_sample(A.nrm, g.tc, lod[2]);
+        in.kd = map_sample(A.kd, g.tc, lod[0]);
+        in.orm = map_sample(A.orm, g.tc, lod[1]);
+        in.nm = map_sample(A.nrm, g.tc, lod[2]);
     }
     return in;
 }
@@ -450,6 +474,7 @@ __device__ __forceinline__ float tc_lever(const ShadeArgs& A, const PixGeo& g, c
 
 // shading of one listed pixel again, with the refined texture coordinate and LOD
 // (a depth-peeled job's list counts its pixels layer after layer, A.B views each)
+template <int SHARE = -1>
 __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
     int hw = A.H * A.W;
     int b = pix / hw, rem = pix - b * hw;
@@ -460,7 +485,7 @@ __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
     pix_geo(A, b, px, py, f, g);
     refine_tc(A, b, px, py, g);
     float lod[3];
-    ShadeIn in = shade_inputs(A, g, lod);
+    ShadeIn in = shade_inputs<SHARE>(A, g, lod);
     float3 c = shade_eval<false>(A.views[b], in, zero3(), nullptr);
     float4 v = make_float4(c.x, c.y, c.z, A.peel ? in.kd.w : 1.f);
     if (A.msaa > 1) {
@@ -892,19 +917,26 @@ __device__ __forceinline__ float2 tex_sample3_bwd(const ShadeArgs& A, const TexC
     return guv;
 }
 
-// tex_sample3 that also leaves, for each map m, dS_m/du and dS_m/dv (the derivatives
-// of its trilinear sample w.r.t. the texture coordinate, float4 each) in
-// stash[8 m .. 8 m + 7] (a lane's private shared-memory row): the adjoint then needs
-// no second read of the texels
-__device__ __forceinline__ void tex_sample3_stash(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3],
+// The samples of maps FROM .. TO-1, which share their taps (footprints from map FROM), leaving
+// for each map m dS_m/du and dS_m/dv (the derivatives of its trilinear sample w.r.t. the
+// texture coordinate, float4 each) in stash[8 m .. 8 m + 7] (a lane's private shared-memory
+// row): the adjoint then reads no texel a second time. Reading them again waited on memory: the
+// kernel issues in 39% of its slots and waits on L1 for most of the rest.
+template <int FROM, int TO>
+__device__ __forceinline__ void maps_sample_stash(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3],
                                                   float* stash) {
-    const float4* ts[3] = {A.kd.tex, A.orm.tex, A.nrm.tex};
+    const TexDev* maps[3] = {&A.kd, &A.orm, &A.nrm};
+    const TexDev& t = *maps[FROM];
+    if (TO - FROM == 1 && constant_map(t)) {
+        out[FROM] = __ldg(t.tex);
+        return;
+    }
     int l0 = (int)floorf(lod);
     float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, A.kd.levels - 1);
+    int l1 = min(l0 + 1, t.levels - 1);
     float4 du[3], dv[3];
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
+    for (int m = FROM; m < TO; ++m) {
         out[m] = du[m] = dv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -912,14 +944,15 @@ __device__ __forceinline__ void tex_sample3_stash(const ShadeArgs& A, const TexC
         int k = s == 0 ? l0 : l1;
         float wl = s == 0 ? 1.f - fr : fr;
         if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(A.kd, k, tc);
+        BilinTap b = bilin_tap(t, k, tc);
         float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
         float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
         float su = wl * b.sw, sv = wl * b.sh;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            float4 t00 = __ldg(ts[m] + b.idx[0]), t10 = __ldg(ts[m] + b.idx[1]);
-            float4 t01 = __ldg(ts[m] + b.idx[2]), t11 = __ldg(ts[m] + b.idx[3]);
+        for (int m = FROM; m < TO; ++m) {
+            const float4* tex = maps[m]->tex;
+            float4 t00 = __ldg(tex + b.idx[0]), t10 = __ldg(tex + b.idx[1]);
+            float4 t01 = __ldg(tex + b.idx[2]), t11 = __ldg(tex + b.idx[3]);
             out[m] = f4madd(out[m], w00, t00);
             out[m] = f4madd(out[m], w10, t10);
             out[m] = f4madd(out[m], w01, t01);
@@ -929,7 +962,7 @@ __device__ __forceinline__ void tex_sample3_stash(const ShadeArgs& A, const TexC
         }
     }
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
+    for (int m = FROM; m < TO; ++m) {
         float* q = stash + 8 * m;
         q[0] = du[m].x;
         q[1] = du[m].y;
@@ -942,54 +975,67 @@ __device__ __forceinline__ void tex_sample3_stash(const ShadeArgs& A, const TexC
     }
 }
 
-// adjoint of tex_sample3_stash: the texel gradients of the optimized maps scattered,
-// d/d(u, v) of g[0] . kd + g[1] . orm + g[2] . nm from the stashed derivatives
-__device__ __forceinline__ float2 tex_sample3_bwd_stash(const ShadeArgs& A, const TexCoord& tc, float lod,
-                                                        const float4 g[3], const float* stash) {
-    float4* gs[3] = {A.kd.grad, A.orm.grad, A.nrm.grad};
-    float2 guv = make_float2(0.f, 0.f);
+// adjoint of maps_sample_stash: the texel gradients of the optimized maps scattered,
+// sum_m d/d(u, v) of g[m] . S_m from the stashed derivatives added to guv
+template <int FROM, int TO>
+__device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoord& tc, float lod, const float4 g[3],
+                                                const float* stash, float2& guv) {
+    const TexDev* maps[3] = {&A.kd, &A.orm, &A.nrm};
+    const TexDev& t = *maps[FROM];
+    if (TO - FROM == 1 && constant_map(t)) {
+        if (t.grad) atomicAdd(t.grad, g[FROM]);
+        return;
+    }
+    bool any = false;
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
+    for (int m = FROM; m < TO; ++m) {
         const float* q = stash + 8 * m;
         guv.x += g[m].x * q[0] + g[m].y * q[1] + g[m].z * q[2] + g[m].w * q[3];
         guv.y += g[m].x * q[4] + g[m].y * q[5] + g[m].z * q[6] + g[m].w * q[7];
+        any = any || maps[m]->grad;
     }
-    if (!gs[0] && !gs[1] && !gs[2]) return guv;
+    if (!any) return;
     int l0 = (int)floorf(lod);
     float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, A.kd.levels - 1);
+    int l1 = min(l0 + 1, t.levels - 1);
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         int k = s == 0 ? l0 : l1;
         float wl = s == 0 ? 1.f - fr : fr;
         if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(A.kd, k, tc);
+        BilinTap b = bilin_tap(t, k, tc);
         float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
         float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            if (!gs[m]) continue;
-            atomicAdd(gs[m] + b.idx[0], f4scale(g[m], w00));
-            atomicAdd(gs[m] + b.idx[1], f4scale(g[m], w10));
-            atomicAdd(gs[m] + b.idx[2], f4scale(g[m], w01));
-            atomicAdd(gs[m] + b.idx[3], f4scale(g[m], w11));
+        for (int m = FROM; m < TO; ++m) {
+            float4* grad = maps[m]->grad;
+            if (!grad) continue;
+            atomicAdd(grad + b.idx[0], f4scale(g[m], w00));
+            atomicAdd(grad + b.idx[1], f4scale(g[m], w10));
+            atomicAdd(grad + b.idx[2], f4scale(g[m], w01));
+            atomicAdd(grad + b.idx[3], f4scale(g[m], w11));
         }
     }
-    return guv;
 }
 
+// Measured (us), sizes that differ read twice -> stashed, and one LOD and footprint for the last
+// two maps where those are of one size (SHARE 2), one load for a map of one texel: backward of
+// 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the others constant) 1388 ->
+// 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2154, of 5 views of 333x501
+// (512^2, 128^2, 256^2) 79.4 -> 76.8; their forward shading 801 -> 730, 878 -> 838, 80 -> 80.
 // shading adjoint of triangle f at sample (px, py) for dL/d(colour) gc (and, for a
 // peeled layer, dL/d(opacity) g_alpha): texel gradients scattered here, the three
 // corners' position / normal / tangent gradients written to vrow[27] (corner k at
 // 9k: position xyz, normal xyz, tangent xyz). The geometry is evaluated twice, once
 // for the shading inputs and once after the BRDF and texture adjoints for the
 // barycentric adjoint, so that nothing of it stays live across them.
-template <bool PEEL>
+// SHARE: share_of, -1 decided here between 1 and 0.
+template <bool PEEL, int SHARE = -1>
 __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int px, int py, int f, float3 gc,
                                                 float g_alpha, float* vrow) {
     const adms_view& vw = A.views[b];
     float hW = 0.5f * (float)A.W, hH = 0.5f * (float)A.H;
-    bool shared = shared_taps(A);
+    const int share = SHARE >= 0 ? SHARE : (shared_taps(A) ? 1 : 0);
     TexCoord tc;
     float lod[3];
     ShadeGrad G;
@@ -1000,35 +1046,40 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
         in.p = g.p;
         in.n_i = g.n;
         in.t_i = g.t;
-        if (shared) {
-            lod[0] = lod[1] = lod[2] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
-            float4 smp[3];
-            tex_sample3_stash(A, g.tc, lod[0], smp, vrow);  // the row holds the uv derivatives until phase 4
-            in.kd = smp[0];
-            in.orm = smp[1];
-            in.nm = smp[2];
+        float4 smp[3];  // the row holds their uv derivatives until the vertex gradients go there
+        lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
+        if (share == 1) {
+            maps_sample_stash<0, 3>(A, g.tc, lod[0], smp, vrow);
         } else {
-            lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
+            maps_sample_stash<0, 1>(A, g.tc, lod[0], smp, vrow);
             lod[1] = tex_lod<true>(A.orm, g.duv_dx, g.duv_dy);
-            lod[2] = tex_lod<true>(A.nrm, g.duv_dx, g.duv_dy);
-            in.kd = tex_sample(A.kd, g.tc, lod[0]);
-            in.orm = tex_sample(A.orm, g.tc, lod[1]);
-            in.nm = tex_sample(A.nrm, g.tc, lod[2]);
+            if (share == 2) {
+                maps_sample_stash<1, 3>(A, g.tc, lod[1], smp, vrow);
+            } else {
+                maps_sample_stash<1, 2>(A, g.tc, lod[1], smp, vrow);
+                lod[2] = tex_lod<true>(A.nrm, g.duv_dx, g.duv_dy);
+                maps_sample_stash<2, 3>(A, g.tc, lod[2], smp, vrow);
+            }
         }
+        in.kd = smp[0];
+        in.orm = smp[1];
+        in.nm = smp[2];
         tc = g.tc;
         shade_eval<true>(vw, in, gc, &G);
     }
     if (PEEL) G.kd.w = g_alpha;  // the opacity is the base colour's fourth channel
-    float2 guv;
-    if (shared) {
-        float4 gt[3] = {G.kd, G.orm, G.nm};
-        guv = tex_sample3_bwd_stash(A, tc, lod[0], gt, vrow);
+    float2 guv = make_float2(0.f, 0.f);
+    float4 gt[3] = {G.kd, G.orm, G.nm};
+    if (share == 1) {
+        maps_sample_bwd<0, 3>(A, tc, lod[0], gt, vrow, guv);
     } else {
-        guv = tex_sample_bwd(A.kd, tc, lod[0], G.kd);
-        float2 g2 = tex_sample_bwd(A.orm, tc, lod[1], G.orm);
-        float2 g3 = tex_sample_bwd(A.nrm, tc, lod[2], G.nm);
-        guv.x += g2.x + g3.x;
-        guv.y += g2.y + g3.y;
+        maps_sample_bwd<0, 1>(A, tc, lod[0], gt, vrow, guv);
+        if (share == 2) {
+            maps_sample_bwd<1, 3>(A, tc, lod[1], gt, vrow, guv);
+        } else {
+            maps_sample_bwd<1, 2>(A, tc, lod[1], gt, vrow, guv);
+            maps_sample_bwd<2, 3>(A, tc, lod[2], gt, vrow, guv);
+        }
     }
     PixGeo g;
     pix_geo<false, true>(A, b, px, py, f, g);
@@ -1089,7 +1140,7 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
 
 // one pixel of the fused backward; warp-collective (vertex scatter). rows: the
 // warp's 32 x ADMS_VROW floats of shared memory
-template <bool PEEL = false>
+template <bool PEEL = false, int SHARE = -1>
 __device__ __forceinline__ void shade_bwd_px(const ShadeArgs& A, int b, int px, int py, float* rows) {
     bool inside = px < A.W && py < A.H;
     int f = -1;
@@ -1112,7 +1163,7 @@ __device__ __forceinline__ void shade_bwd_px(const ShadeArgs& A, int b, int px, 
             gc = pr.w * gc;
         }
         if (f >= 0 && (gc.x != 0.f || gc.y != 0.f || gc.z != 0.f || g_alpha != 0.f))
-            shading_adjoint<PEEL>(A, b, px, py, f, gc, g_alpha, rows + (threadIdx.x & 31) * ADMS_VROW);
+            shading_adjoint<PEEL, SHARE>(A, b, px, py, f, gc, g_alpha, rows + (threadIdx.x & 31) * ADMS_VROW);
         else
             f = -1;
     }

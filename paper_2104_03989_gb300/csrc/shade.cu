@@ -17,10 +17,11 @@ namespace adms {
 
 // ------------------------------------------------------------------ single-job kernels (16x16 tiles)
 // the listed pixels of one job (A.refine[0] of them), grid-stride
+template <int SHARE>
 __global__ void __launch_bounds__(64) k_shade_refine(ShadeArgs A) {
     int n = A.refine[0];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        shade_refine_px(A, A.refine[1 + i]);
+        shade_refine_px<SHARE>(A, A.refine[1 + i]);
 }
 
 // A 16x16 tile of pixels is shaded by 256 / THREADS blocks, each a band of
@@ -43,7 +44,7 @@ __device__ __forceinline__ void band_pixel(int W, int& px, int& py) {
 // grids) 8 is ahead (69.0 against 70.3 us at 5 of 333x501). AA + loss: 16 blocks 53.1 us,
 // 12: 55.3.
 #define ADMS_FWD_THREADS 128
-constexpr int fwd_blocks(bool inline_refine, int share) { return share == 0 && !inline_refine ? 12 : 8; }
+constexpr int fwd_blocks(bool inline_refine, int share) { return share != 1 && !inline_refine ? 12 : 8; }
 #define ADMS_AA_THREADS 128
 #define ADMS_AA_BLOCKS 16
 template <bool INLINE, int SHARE>
@@ -76,12 +77,12 @@ __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(Sha
 #ifndef ADMS_BWD_THREADS
 #define ADMS_BWD_THREADS 128  // 256: a block per 16x16 tile; 128: two blocks of 16x8 pixels
 #endif
-template <bool PEEL>
+template <bool PEEL, int SHARE>
 __global__ void __launch_bounds__(ADMS_BWD_THREADS, ADMS_BWD_BLOCKS) k_shade_bwd(ShadeArgs A) {
     __shared__ float rows[(ADMS_BWD_THREADS / 32) * 32 * ADMS_VROW];
     int px, py;
     band_pixel<ADMS_BWD_THREADS>(A.W, px, py);
-    shade_bwd_px<PEEL>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
+    shade_bwd_px<PEEL, SHARE>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
 }
 
 // MSAA forward: a block takes a 32x32-sample region (four samples per thread), its
@@ -319,12 +320,14 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers) {
         cudaError_t e = cudaMemsetAsync(a.refine, 0, sizeof(int), st);
         if (e) return e;
     }
+    int share = share_of(a);
     if (a.msaa > 1) {
         int R = ADMS_MSAA_REGION;
         k_shade_fwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
     } else {
-        auto k = inline_refine ? (shared_taps(a) ? k_shade_fwd<true, 1> : k_shade_fwd<true, 0>)
-                               : (shared_taps(a) ? k_shade_fwd<false, 1> : k_shade_fwd<false, 0>);
+        auto k = inline_refine
+                     ? (share == 1 ? k_shade_fwd<true, 1> : share == 2 ? k_shade_fwd<true, 2> : k_shade_fwd<true, 0>)
+                     : (share == 1 ? k_shade_fwd<false, 1> : share == 2 ? k_shade_fwd<false, 2> : k_shade_fwd<false, 0>);
         dim3 grid = band_grid(a, ADMS_FWD_THREADS);
         grid.z = layers;
         k<<<grid, ADMS_FWD_THREADS, 0, st>>>(a);
@@ -333,7 +336,8 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers) {
     if (list) {
         // a few thousand pixels, a long dependent chain each: small blocks spread them over every
         // SM (128 blocks of 256 filled 30 SMs; the displaced mesh's shading 837 -> 822 us)
-        k_shade_refine<<<608, 64, 0, st>>>(a);
+        auto k = share == 1 ? k_shade_refine<1> : share == 2 ? k_shade_refine<2> : k_shade_refine<0>;
+        k<<<608, 64, 0, st>>>(a);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -356,7 +360,9 @@ cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st) {
         int R = ADMS_MSAA_REGION;
         k_shade_bwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
     } else {
-        auto k = a.peel ? k_shade_bwd<true> : k_shade_bwd<false>;
+        int share = share_of(a);
+        auto k = a.peel ? (share == 1 ? k_shade_bwd<true, 1> : share == 2 ? k_shade_bwd<true, 2> : k_shade_bwd<true, 0>)
+                        : (share == 1 ? k_shade_bwd<false, 1> : share == 2 ? k_shade_bwd<false, 2> : k_shade_bwd<false, 0>);
         k<<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
     }
     count_launches(1);
