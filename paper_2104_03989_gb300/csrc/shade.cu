@@ -228,15 +228,20 @@ __global__ void __launch_bounds__(256) k_refine_batch(const ShadeBatch P) {
         shade_refine_px(A, A.refine[1 + i]);
 }
 
+// Two blocks of 128 threads take a tile, as in the single-job kernels: shorter tails and finer
+// register rounding (eight uneven jobs: backward 498 -> 484 us, shading 206 -> 190, AA + loss 143
+// -> 135 against blocks of 256). The grid and the tuned blocks per SM stay in tiles.
+constexpr int batch_blocks(int kind) { return kind == 2 ? ADMS_BWD_BLOCKS : kind == 1 ? ADMS_AA_BLOCKS : 10; }
 template <int KIND>
-__global__ void __launch_bounds__(256, KIND == 2 ? 3 : (KIND == 1 ? 8 : 5))
+__global__ void __launch_bounds__(128, batch_blocks(KIND))
     k_pixels_batch(const ShadeBatch P, const WorkItem* __restrict__ items, int n, int tw, int job0) {
-    __shared__ float red[16];
-    __shared__ float rows[KIND == 2 ? 8 * 32 * ADMS_VROW : 1];
-    for (int it = blockIdx.x; it < n; it += gridDim.x) {
-        WorkItem w = items[it];
+    __shared__ float red[8];
+    __shared__ float rows[KIND == 2 ? 4 * 32 * ADMS_VROW : 1];
+    for (int it = blockIdx.x; it < 2 * n; it += gridDim.x) {
+        WorkItem w = items[it >> 1];
         const ShadeArgs& A = P.a[w.job - job0];
-        int px = w.x0 + (int)threadIdx.x % tw, py = w.y0 + (int)threadIdx.x / tw;
+        int t = (int)threadIdx.x + 128 * (it & 1);
+        int px = w.x0 + t % tw, py = w.y0 + t / tw;
         if (KIND == 0) shade_fwd_px(A, w.view, px, py);
         else if (KIND == 1) {
             LossSum sum;
@@ -369,13 +374,14 @@ cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// in tiles (256 pixels, two blocks of the pixel kernels) per SM, as pixels_batched's blocks are
 int batched_occupancy(int kind) {
     if (kind == 3) return raster_batch_occupancy();
     int n = 0;
-    cudaError_t e = kind == 0   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<0>, 256, 0)
-                    : kind == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<1>, 256, 0)
-                                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<2>, 256, 0);
-    return e == cudaSuccess && n > 0 ? n : 1;
+    cudaError_t e = kind == 0   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<0>, 128, 0)
+                    : kind == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<1>, 128, 0)
+                                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pixels_batch<2>, 128, 0);
+    return e == cudaSuccess && n > 1 ? n / 2 : 1;
 }
 
 cudaError_t pixels_batched(int kind, const ShadeArgs* args, const int* item_off, int n_jobs, const WorkItem* items,
@@ -386,15 +392,15 @@ cudaError_t pixels_batched(int kind, const ShadeArgs* args, const int* item_off,
         int s0 = item_off[j0], n = item_off[j1] - s0;
         if (n <= 0) continue;
         memcpy(P.a, args + j0, sizeof(ShadeArgs) * (j1 - j0));
-        int g = std::min(blocks, n);
+        int g = 2 * std::min(blocks, n);
         if (kind == 0) {
             k_refine_reset<<<1, ADMS_BATCH_JOBS, 0, st>>>(P, j1 - j0);
-            k_pixels_batch<0><<<g, 256, 0, st>>>(P, items + s0, n, tw, j0);
+            k_pixels_batch<0><<<g, 128, 0, st>>>(P, items + s0, n, tw, j0);
             k_refine_batch<<<dim3(64, j1 - j0), 256, 0, st>>>(P);
             count_launches(2);
         }
-        else if (kind == 1) k_pixels_batch<1><<<g, 256, 0, st>>>(P, items + s0, n, tw, j0);
-        else k_pixels_batch<2><<<g, 256, 0, st>>>(P, items + s0, n, tw, j0);
+        else if (kind == 1) k_pixels_batch<1><<<g, 128, 0, st>>>(P, items + s0, n, tw, j0);
+        else k_pixels_batch<2><<<g, 128, 0, st>>>(P, items + s0, n, tw, j0);
         count_launches(1);
         cudaError_t e = cudaGetLastError();
         if (e) return e;
