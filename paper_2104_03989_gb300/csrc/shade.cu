@@ -24,15 +24,19 @@ __global__ void __launch_bounds__(64) k_shade_refine(ShadeArgs A) {
         shade_refine_px<SHARE>(A, A.refine[1 + i]);
 }
 
-// A 16x16 tile of pixels is shaded by 256 / THREADS blocks, each a band of
-// 16 x (THREADS / 16) rows; thread t takes column t % 16 of row t / 16 of its band.
-template <int THREADS>
+// A 16x16 tile of pixels is shaded by 256 / THREADS blocks, each a band of 16 x (THREADS / 16)
+// rows. COLS: columns of a warp, 8 (a warp takes 8x4 pixels) or 16 (16x2). A compact warp meets
+// fewer triangles and texels: forward 94.2 -> 92.3 us (8 views of 512x512 of a dense mesh) and 836
+// -> 822 (peeled layers, two passes), backward 1193 -> 1183 (16 of 1024x1024); the peeled layers'
+// backward is better in rows (2257 against 2290 us).
+template <int THREADS, int COLS>
 __device__ __forceinline__ void band_pixel(int W, int& px, int& py) {
-    constexpr int PARTS = 256 / THREADS;
+    constexpr int PARTS = 256 / THREADS, ACROSS = ADMS_TILE / COLS, ROWS = 32 / COLS;
     int tiles_x = (W + ADMS_TILE - 1) / ADMS_TILE;
     int tile = blockIdx.x / PARTS, part = blockIdx.x % PARTS;
-    px = (tile % tiles_x) * ADMS_TILE + (threadIdx.x & 15);
-    py = (tile / tiles_x) * ADMS_TILE + part * (ADMS_TILE / PARTS) + (threadIdx.x >> 4);
+    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    px = (tile % tiles_x) * ADMS_TILE + COLS * (warp % ACROSS) + lane % COLS;
+    py = (tile / tiles_x) * ADMS_TILE + part * (ADMS_TILE / PARTS) + ROWS * (warp / ACROSS) + lane / COLS;
 }
 
 // Block shapes (threads per block x resident blocks per SM, i.e. the register cap 65536 /
@@ -41,8 +45,9 @@ __device__ __forceinline__ void band_pixel(int W, int& px, int& py) {
 // sizes 3% (895 -> 920 us for the two passes over 16 views of 1024x1024). Equal maps, 8 views
 // of 512x512: 8 blocks 74.5 us, 6: 80.0, 10: 77.9, 12: 77.4; different ones, 16 views of
 // 1024x1024: 8 blocks 894 us, 6: 964, 10: 883, 12: 832, but with the refinement inline (small
-// grids) 8 is ahead (69.0 against 70.3 us at 5 of 333x501). AA + loss: 16 blocks 53.1 us,
-// 12: 55.3.
+// grids) 8 is ahead (69.0 against 70.3 us at 5 of 333x501). AA + loss: 16 blocks; 12 are
+// ahead where few warps enter the pair loop (5 of 333x501: 32.4 against 34.4 us) and behind where
+// many do (600k leaf quads 69.8 against 66.2, peeled layers 961 against 912).
 #define ADMS_FWD_THREADS 128
 constexpr int fwd_blocks(bool inline_refine, int share) { return share != 1 && !inline_refine ? 12 : 8; }
 #define ADMS_AA_THREADS 128
@@ -50,7 +55,7 @@ constexpr int fwd_blocks(bool inline_refine, int share) { return share != 1 && !
 template <bool INLINE, int SHARE>
 __global__ void __launch_bounds__(ADMS_FWD_THREADS, fwd_blocks(INLINE, SHARE)) k_shade_fwd(ShadeArgs A) {
     int px, py;
-    band_pixel<ADMS_FWD_THREADS>(A.W, px, py);
+    band_pixel<ADMS_FWD_THREADS, 8>(A.W, px, py);
     // blockIdx.z: the layer of a depth-peeled job (the layers' shading is independent; a launch
     // and a refinement pass per layer left eight tails and eight nearly empty passes, 15 us each)
     shade_fwd_px<INLINE, SHARE>(A, blockIdx.y, px, py, (size_t)blockIdx.z * ((size_t)A.B * A.H * A.W));
@@ -81,7 +86,7 @@ template <bool PEEL, int SHARE>
 __global__ void __launch_bounds__(ADMS_BWD_THREADS, ADMS_BWD_BLOCKS) k_shade_bwd(ShadeArgs A) {
     __shared__ float rows[(ADMS_BWD_THREADS / 32) * 32 * ADMS_VROW];
     int px, py;
-    band_pixel<ADMS_BWD_THREADS>(A.W, px, py);
+    band_pixel<ADMS_BWD_THREADS, PEEL ? 16 : 8>(A.W, px, py);
     shade_bwd_px<PEEL, SHARE>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
 }
 
