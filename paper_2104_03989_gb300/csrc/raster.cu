@@ -575,16 +575,24 @@ __global__ void __launch_bounds__(256) k_bin_fill(const __grid_constant__ Pack<F
 // conversions and 17 of 32 lanes active in 16x2 strips, at 69.9 us for 8 views of 512x512 of
 // 5000 triangles before; 47.5 us now (58% issue, 22 lanes, 28.6 M against 50.4 M warp
 // instructions). The k-buffer form on 11k billboards with 8 layers: 6.06 ms (its tile lists
-// had overflowed) -> 0.45 ms.
+// had overflowed) -> 0.41 ms, 0.24 with the classes below.
 //
 // Each pixel starts from the key left by the small-triangle pass. A tile whose list did
 // not fit scans every binned triangle of its view instead.
+// BUCKETS > 1 (the k-buffer): the walk takes each staging warp's triangles front to back in
+// four classes of their depth floor, and a lane whose buffer is full of nearer fragments passes
+// a triangle over by the floor alone. Of 70 fragments a sample of 11k billboards, in list order
+// about 25 entered a buffer of 8 and every one was divided out (313 M warp instructions a launch,
+// 77% issue): two passes over 8 views of 512x512 817 -> 470 us. The keys do not depend on the order.
+template <int BUCKETS>
 struct TileSmem {
     int4 p[256], q[256], r[256];  // near_pack at the tile's first sample; q.w: flags
-    int4 s[256];                  // large triangles only
+    int4 s[256];                  // large triangles; .w: the depth floor (BUCKETS > 1)
     int id[256];
-    unsigned mask[8][8];  // [8x4 block][staging warp]
+    unsigned mask[BUCKETS][8][8];  // [class][8x4 block][staging warp]
 };
+template <int KB>
+constexpr int depth_buckets = KB > 1 ? 4 : 1;
 #define ADMS_LARGE 8  // q.w: bits 0-2 thresholds, bit 3 large
 
 // minimum key / the KB smallest keys in kb[0] < kb[1] < ... (the keys of one sample are
@@ -621,7 +629,8 @@ __device__ __forceinline__ int tile_y(int tid) { return (tid >> 6) * 4 + ((tid >
 
 template <int KB>
 __device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int tile, long long off, int cnt,
-                                                 TileSmem& sm, KeySink<KB>& sink) {
+                                                 TileSmem<depth_buckets<KB>>& sm, KeySink<KB>& sink) {
+    constexpr int BUCKETS = depth_buckets<KB>;
     int tx = tile % A.tiles_x, ty = tile / A.tiles_x;
     int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int lx = tile_x(tid), ly = tile_y(tid);
@@ -635,7 +644,7 @@ __device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int t
     for (int c0 = 0; c0 < n; c0 += 256) {
         int m = min(256, n - c0);
         __syncthreads();
-        unsigned mask = 0;
+        unsigned mask = 0, zlo = 0;
         if (tid < m) {
             int f = overflow ? c0 + tid : A.lists.get(off + c0 + tid);
             TriBin tb = overflow ? bb[f] : rb[f].box;
@@ -681,40 +690,55 @@ __device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int t
                 sm.r[tid] = make_int4(__float_as_int(area), __float_as_int(t.z0), __float_as_int(t.dz1),
                                       __float_as_int(t.dz2));
                 sm.id[tid] = f;
+                if (BUCKETS > 1) {
+                    zlo = key_floor(t.z0, t.z0 + t.dz1, t.z0 + t.dz2);
+                    sm.s[tid].w = (int)zlo;
+                }
             }
         }
+        int bucket = 0;
+        if (BUCKETS > 1) {
+            unsigned near = __reduce_min_sync(0xffffffffu, mask ? zlo : 0xffffffffu);
+            unsigned far = __reduce_max_sync(0xffffffffu, mask ? zlo : 0u);
+            unsigned step = (far - near) / BUCKETS + 1;  // (no triangle in the warp: no bit is set below)
+            bucket = (zlo >= near + step) + (zlo >= near + 2 * step) + (zlo >= near + 3 * step);
+        }
 #pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            unsigned mw = __ballot_sync(0xffffffffu, (mask >> w) & 1u);
-            if (lane == w) sm.mask[w][warp] = mw;
+        for (int k = 0; k < 8 * BUCKETS; ++k) {
+            unsigned mw = __ballot_sync(0xffffffffu, (mask >> (k & 7)) & (bucket == k >> 3 ? 1u : 0u));
+            if (lane == k) sm.mask[k >> 3][k & 7][warp] = mw;
         }
         __syncthreads();
-        for (int g = 0; g < m; g += 32) {
-            for (unsigned mm = sm.mask[warp][g >> 5]; mm; mm &= mm - 1) {
-                int j = g + __ffs(mm) - 1;
-                int4 p = sm.p[j], q = sm.q[j];
-                float f1, f2;
-                if (!(q.w & ADMS_LARGE)) {
-                    int e0 = p.x + p.y * lx + p.z * ly, e1 = q.x + q.y * lx + q.z * ly, e2 = near_third(p.w, e0, e1);
-                    if ((e0 | e1 | e2) < 0) continue;
-                    f1 = __int2float_rn(e1 + ((q.w >> 1) & 1));
-                    f2 = __int2float_rn(e2 + (q.w >> 2));
-                } else {
-                    int4 s = sm.s[j];
-                    long long E0 = ((long long)p.y << 32) | (unsigned)p.x, E1 = ((long long)p.w << 32) | (unsigned)p.z;
-                    long long E2 = ((long long)q.y << 32) | (unsigned)q.x;
-                    int dx = 256 * lx, dy = 256 * ly;
-                    long long e0 = E0 + (long long)q.z * dx + (long long)s.x * dy;
-                    long long e1 = E1 + (long long)s.y * dx + (long long)s.z * dy;
-                    // a_2 = -(a_0 + a_1): the edges of a closed triangle
-                    long long e2 = E2 - ((long long)q.z + s.y) * dx - ((long long)s.x + s.z) * dy;
-                    if (e0 < (q.w & 1) || e1 < ((q.w >> 1) & 1) || e2 < ((q.w >> 2) & 1)) continue;
-                    f1 = __ll2float_rn(e1);
-                    f2 = __ll2float_rn(e2);
+        for (int k = 0; k < BUCKETS; ++k) {
+            for (int g = 0; g < m; g += 32) {
+                for (unsigned mm = sm.mask[k][warp][g >> 5]; mm; mm &= mm - 1) {
+                    int j = g + __ffs(mm) - 1;
+                    if (BUCKETS > 1 && (unsigned)sm.s[j].w > (unsigned)(sink.kb[KB - 1] >> 32)) continue;
+                    int4 p = sm.p[j], q = sm.q[j];
+                    float f1, f2;
+                    if (!(q.w & ADMS_LARGE)) {
+                        int e0 = p.x + p.y * lx + p.z * ly, e1 = q.x + q.y * lx + q.z * ly,
+                            e2 = near_third(p.w, e0, e1);
+                        if ((e0 | e1 | e2) < 0) continue;
+                        f1 = __int2float_rn(e1 + ((q.w >> 1) & 1));
+                        f2 = __int2float_rn(e2 + (q.w >> 2));
+                    } else {
+                        int4 s = sm.s[j];
+                        long long E0 = ((long long)p.y << 32) | (unsigned)p.x, E1 = ((long long)p.w << 32) | (unsigned)p.z;
+                        long long E2 = ((long long)q.y << 32) | (unsigned)q.x;
+                        int dx = 256 * lx, dy = 256 * ly;
+                        long long e0 = E0 + (long long)q.z * dx + (long long)s.x * dy;
+                        long long e1 = E1 + (long long)s.y * dx + (long long)s.z * dy;
+                        // a_2 = -(a_0 + a_1): the edges of a closed triangle
+                        long long e2 = E2 - ((long long)q.z + s.y) * dx - ((long long)s.x + s.z) * dy;
+                        if (e0 < (q.w & 1) || e1 < ((q.w >> 1) & 1) || e2 < ((q.w >> 2) & 1)) continue;
+                        f1 = __ll2float_rn(e1);
+                        f2 = __ll2float_rn(e2);
+                    }
+                    int4 r = sm.r[j];
+                    sink.take(depth_key(f1, f2, __int_as_float(r.x), __int_as_float(r.y), __int_as_float(r.z),
+                                        __int_as_float(r.w), sm.id[j]));
                 }
-                int4 r = sm.r[j];
-                sink.take(depth_key(f1, f2, __int_as_float(r.x), __int_as_float(r.y), __int_as_float(r.z),
-                                    __int_as_float(r.w), sm.id[j]));
             }
         }
     }
@@ -722,7 +746,7 @@ __device__ __forceinline__ void raster_tile_walk(const TileArgs& A, int b, int t
 
 // one 16x16 tile of one view: the minimum key per pixel
 __device__ __forceinline__ void raster_tile_body(const TileArgs& A, unsigned long long* __restrict__ keys, int b,
-                                                 int tile, TileSmem& sm) {
+                                                 int tile, TileSmem<1>& sm) {
     size_t t = (size_t)b * A.tiles_x * A.tiles_y + tile;
     int cnt = A.tile_count[t];
     if (cnt == 0) return;  // no binned triangle: the small-triangle pass left the final keys
@@ -737,7 +761,7 @@ __device__ __forceinline__ void raster_tile_body(const TileArgs& A, unsigned lon
 }
 
 __global__ void __launch_bounds__(256) k_raster(const TileArgs A, unsigned long long* __restrict__ keys) {
-    __shared__ TileSmem sm;
+    __shared__ TileSmem<1> sm;
     raster_tile_body(A, keys, blockIdx.y, blockIdx.x, sm);
 }
 
@@ -745,7 +769,7 @@ __global__ void __launch_bounds__(256) k_raster(const TileArgs A, unsigned long 
 // to 32, reads their counts together and skips the empty ones
 __global__ void __launch_bounds__(256) k_raster_sparse(const TileArgs A, unsigned long long* __restrict__ keys,
                                                        int n_tiles) {
-    __shared__ TileSmem sm;
+    __shared__ TileSmem<1> sm;
     long long t = blockIdx.x + (long long)(threadIdx.x & 31) * gridDim.x;
     unsigned live = __ballot_sync(0xffffffffu, t < n_tiles && A.tile_count[t] > 0);
     int per_view = A.tiles_x * A.tiles_y;
@@ -764,7 +788,7 @@ __global__ void __launch_bounds__(256) k_raster_sparse(const TileArgs A, unsigne
 template <int KB>
 __global__ void __launch_bounds__(256) k_raster_kbuf(const TileArgs A, unsigned long long* __restrict__ keys, int L,
                                                      int B) {
-    __shared__ TileSmem sm;
+    __shared__ TileSmem<depth_buckets<KB>> sm;
     int b = blockIdx.y, tile = blockIdx.x;
     int px = (tile % A.tiles_x) * ADMS_TILE + tile_x(threadIdx.x), py = (tile / A.tiles_x) * ADMS_TILE + tile_y(threadIdx.x);
     KeySink<KB> sink;
@@ -793,7 +817,7 @@ struct RasterBatch {
 // jobs' arguments are kernel parameters (up to 64 jobs per launch)
 __global__ void __launch_bounds__(256) k_raster_batch(const __grid_constant__ RasterBatch P,
                                                       const WorkItem* __restrict__ items, int n, int job0) {
-    __shared__ TileSmem sm;
+    __shared__ TileSmem<1> sm;
     for (int it = blockIdx.x; it < n; it += gridDim.x) {
         WorkItem w = items[it];
         const TileArgs& A = P.a[w.job - job0];
