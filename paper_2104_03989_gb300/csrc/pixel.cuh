@@ -399,9 +399,9 @@ __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo
     } else {
         lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
         lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
-        in.kd = map_sample(A.kd, g.tc, lod[0]);
-        in.orm = map_sample(A.orm, g.tc, lod[1]);
-        in.nm = map_sample(A.nrm, g.tc, lod[2]);
+        in.kd = SHARE < 0 ? tex_sample(A.kd, g.tc, lod[0]) : map_sample(A.kd, g.tc, lod[0]);
+        in.orm = SHARE < 0 ? tex_sample(A.orm, g.tc, lod[1]) : map_sample(A.orm, g.tc, lod[1]);
+        in.nm = SHARE < 0 ? tex_sample(A.nrm, g.tc, lod[2]) : map_sample(A.nrm, g.tc, lod[2]);
     }
     return in;
 }
@@ -474,7 +474,6 @@ __device__ __forceinline__ float tc_lever(const ShadeArgs& A, const PixGeo& g, c
 
 // shading of one listed pixel again, with the refined texture coordinate and LOD
 // (a depth-peeled job's list counts its pixels layer after layer, A.B views each)
-template <int SHARE = -1>
 __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
     int hw = A.H * A.W;
     int b = pix / hw, rem = pix - b * hw;
@@ -485,7 +484,7 @@ __device__ __forceinline__ void shade_refine_px(const ShadeArgs& A, int pix) {
     pix_geo(A, b, px, py, f, g);
     refine_tc(A, b, px, py, g);
     float lod[3];
-    ShadeIn in = shade_inputs<SHARE>(A, g, lod);
+    ShadeIn in = shade_inputs(A, g, lod);
     float3 c = shade_eval<false>(A.views[b], in, zero3(), nullptr);
     float4 v = make_float4(c.x, c.y, c.z, A.peel ? in.kd.w : 1.f);
     if (A.msaa > 1) {
@@ -917,6 +916,92 @@ __device__ __forceinline__ float2 tex_sample3_bwd(const ShadeArgs& A, const TexC
     return guv;
 }
 
+// tex_sample3 that also leaves, for each map m, dS_m/du and dS_m/dv (the derivatives
+// of its trilinear sample w.r.t. the texture coordinate, float4 each) in
+// stash[8 m .. 8 m + 7] (a lane's private shared-memory row): the adjoint then needs
+// no second read of the texels
+__device__ __forceinline__ void tex_sample3_stash(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3],
+                                                  float* stash) {
+    const float4* ts[3] = {A.kd.tex, A.orm.tex, A.nrm.tex};
+    int l0 = (int)floorf(lod);
+    float fr = lod - (float)l0;
+    int l1 = min(l0 + 1, A.kd.levels - 1);
+    float4 du[3], dv[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        out[m] = du[m] = dv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        int k = s == 0 ? l0 : l1;
+        float wl = s == 0 ? 1.f - fr : fr;
+        if (wl == 0.f) continue;
+        BilinTap b = bilin_tap(A.kd, k, tc);
+        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
+        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
+        float su = wl * b.sw, sv = wl * b.sh;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            float4 t00 = __ldg(ts[m] + b.idx[0]), t10 = __ldg(ts[m] + b.idx[1]);
+            float4 t01 = __ldg(ts[m] + b.idx[2]), t11 = __ldg(ts[m] + b.idx[3]);
+            out[m] = f4madd(out[m], w00, t00);
+            out[m] = f4madd(out[m], w10, t10);
+            out[m] = f4madd(out[m], w01, t01);
+            out[m] = f4madd(out[m], w11, t11);
+            du[m] = f4madd(du[m], su, f4madd(f4scale(f4sub(t10, t00), 1.f - b.fy), b.fy, f4sub(t11, t01)));
+            dv[m] = f4madd(dv[m], sv, f4madd(f4scale(f4sub(t01, t00), 1.f - b.fx), b.fx, f4sub(t11, t10)));
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        float* q = stash + 8 * m;
+        q[0] = du[m].x;
+        q[1] = du[m].y;
+        q[2] = du[m].z;
+        q[3] = du[m].w;
+        q[4] = dv[m].x;
+        q[5] = dv[m].y;
+        q[6] = dv[m].z;
+        q[7] = dv[m].w;
+    }
+}
+
+// adjoint of tex_sample3_stash: the texel gradients of the optimized maps scattered,
+// d/d(u, v) of g[0] . kd + g[1] . orm + g[2] . nm from the stashed derivatives
+__device__ __forceinline__ float2 tex_sample3_bwd_stash(const ShadeArgs& A, const TexCoord& tc, float lod,
+                                                        const float4 g[3], const float* stash) {
+    float4* gs[3] = {A.kd.grad, A.orm.grad, A.nrm.grad};
+    float2 guv = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const float* q = stash + 8 * m;
+        guv.x += g[m].x * q[0] + g[m].y * q[1] + g[m].z * q[2] + g[m].w * q[3];
+        guv.y += g[m].x * q[4] + g[m].y * q[5] + g[m].z * q[6] + g[m].w * q[7];
+    }
+    if (!gs[0] && !gs[1] && !gs[2]) return guv;
+    int l0 = (int)floorf(lod);
+    float fr = lod - (float)l0;
+    int l1 = min(l0 + 1, A.kd.levels - 1);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        int k = s == 0 ? l0 : l1;
+        float wl = s == 0 ? 1.f - fr : fr;
+        if (wl == 0.f) continue;
+        BilinTap b = bilin_tap(A.kd, k, tc);
+        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
+        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if (!gs[m]) continue;
+            atomicAdd(gs[m] + b.idx[0], f4scale(g[m], w00));
+            atomicAdd(gs[m] + b.idx[1], f4scale(g[m], w10));
+            atomicAdd(gs[m] + b.idx[2], f4scale(g[m], w01));
+            atomicAdd(gs[m] + b.idx[3], f4scale(g[m], w11));
+        }
+    }
+    return guv;
+}
+
 // The samples of maps FROM .. TO-1, which share their taps (footprints from map FROM), leaving
 // for each map m dS_m/du and dS_m/dv (the derivatives of its trilinear sample w.r.t. the
 // texture coordinate, float4 each) in stash[8 m .. 8 m + 7] (a lane's private shared-memory
@@ -1029,13 +1114,15 @@ __device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoo
 // 9k: position xyz, normal xyz, tangent xyz). The geometry is evaluated twice, once
 // for the shading inputs and once after the BRDF and texture adjoints for the
 // barycentric adjoint, so that nothing of it stays live across them.
-// SHARE: share_of, -1 decided here between 1 and 0.
+// SHARE: 0 or 2 of share_of in a kernel of its own, -1 maps of one size (and batched and sampled
+// launches, whatever the sizes). Equal maps keep the general form: on its own its shading adjoint is
+// fused otherwise by the compiler, for no gain, and gradients that cancel to nothing change sign.
 template <bool PEEL, int SHARE = -1>
 __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int px, int py, int f, float3 gc,
                                                 float g_alpha, float* vrow) {
     const adms_view& vw = A.views[b];
     float hW = 0.5f * (float)A.W, hH = 0.5f * (float)A.H;
-    const int share = SHARE >= 0 ? SHARE : (shared_taps(A) ? 1 : 0);
+    bool shared = shared_taps(A);
     TexCoord tc;
     float lod[3];
     ShadeGrad G;
@@ -1046,40 +1133,60 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
         in.p = g.p;
         in.n_i = g.n;
         in.t_i = g.t;
-        float4 smp[3];  // the row holds their uv derivatives until the vertex gradients go there
-        lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
-        if (share == 1) {
-            maps_sample_stash<0, 3>(A, g.tc, lod[0], smp, vrow);
-        } else {
+        if constexpr (SHARE >= 0) {
+            float4 smp[3];  // the row holds their uv derivatives until the vertex gradients go there
+            lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
             maps_sample_stash<0, 1>(A, g.tc, lod[0], smp, vrow);
             lod[1] = tex_lod<true>(A.orm, g.duv_dx, g.duv_dy);
-            if (share == 2) {
+            if constexpr (SHARE == 2) {
                 maps_sample_stash<1, 3>(A, g.tc, lod[1], smp, vrow);
             } else {
                 maps_sample_stash<1, 2>(A, g.tc, lod[1], smp, vrow);
                 lod[2] = tex_lod<true>(A.nrm, g.duv_dx, g.duv_dy);
                 maps_sample_stash<2, 3>(A, g.tc, lod[2], smp, vrow);
             }
+            in.kd = smp[0];
+            in.orm = smp[1];
+            in.nm = smp[2];
+        } else if (shared) {
+            lod[0] = lod[1] = lod[2] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
+            float4 smp[3];
+            tex_sample3_stash(A, g.tc, lod[0], smp, vrow);  // the row holds the uv derivatives until phase 4
+            in.kd = smp[0];
+            in.orm = smp[1];
+            in.nm = smp[2];
+        } else {
+            lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
+            lod[1] = tex_lod<true>(A.orm, g.duv_dx, g.duv_dy);
+            lod[2] = tex_lod<true>(A.nrm, g.duv_dx, g.duv_dy);
+            in.kd = tex_sample(A.kd, g.tc, lod[0]);
+            in.orm = tex_sample(A.orm, g.tc, lod[1]);
+            in.nm = tex_sample(A.nrm, g.tc, lod[2]);
         }
-        in.kd = smp[0];
-        in.orm = smp[1];
-        in.nm = smp[2];
         tc = g.tc;
         shade_eval<true>(vw, in, gc, &G);
     }
     if (PEEL) G.kd.w = g_alpha;  // the opacity is the base colour's fourth channel
-    float2 guv = make_float2(0.f, 0.f);
-    float4 gt[3] = {G.kd, G.orm, G.nm};
-    if (share == 1) {
-        maps_sample_bwd<0, 3>(A, tc, lod[0], gt, vrow, guv);
-    } else {
+    float2 guv;
+    if constexpr (SHARE >= 0) {
+        guv = make_float2(0.f, 0.f);
+        float4 gt[3] = {G.kd, G.orm, G.nm};
         maps_sample_bwd<0, 1>(A, tc, lod[0], gt, vrow, guv);
-        if (share == 2) {
+        if constexpr (SHARE == 2) {
             maps_sample_bwd<1, 3>(A, tc, lod[1], gt, vrow, guv);
         } else {
             maps_sample_bwd<1, 2>(A, tc, lod[1], gt, vrow, guv);
             maps_sample_bwd<2, 3>(A, tc, lod[2], gt, vrow, guv);
         }
+    } else if (shared) {
+        float4 gt[3] = {G.kd, G.orm, G.nm};
+        guv = tex_sample3_bwd_stash(A, tc, lod[0], gt, vrow);
+    } else {
+        guv = tex_sample_bwd(A.kd, tc, lod[0], G.kd);
+        float2 g2 = tex_sample_bwd(A.orm, tc, lod[1], G.orm);
+        float2 g3 = tex_sample_bwd(A.nrm, tc, lod[2], G.nm);
+        guv.x += g2.x + g3.x;
+        guv.y += g2.y + g3.y;
     }
     PixGeo g;
     pix_geo<false, true>(A, b, px, py, f, g);

@@ -17,18 +17,18 @@ namespace adms {
 
 // ------------------------------------------------------------------ single-job kernels (16x16 tiles)
 // the listed pixels of one job (A.refine[0] of them), grid-stride
-template <int SHARE>
 __global__ void __launch_bounds__(64) k_shade_refine(ShadeArgs A) {
     int n = A.refine[0];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        shade_refine_px<SHARE>(A, A.refine[1 + i]);
+        shade_refine_px(A, A.refine[1 + i]);
 }
 
 // A 16x16 tile of pixels is shaded by 256 / THREADS blocks, each a band of 16 x (THREADS / 16)
-// rows. COLS: columns of a warp, 8 (a warp takes 8x4 pixels) or 16 (16x2). A compact warp meets
-// fewer triangles and texels: forward 94.2 -> 92.3 us (8 views of 512x512 of a dense mesh) and 836
-// -> 822 (peeled layers, two passes), backward 1193 -> 1183 (16 of 1024x1024); the peeled layers'
-// backward is better in rows (2257 against 2290 us).
+// rows. COLS: columns of a warp, 8 (a warp takes 8x4 pixels) or 16 (16x2). The forward's compact
+// warps meet fewer triangles and texels: 94.2 -> 92.3 us (8 views of 512x512 of a dense mesh), 836
+// -> 822 (peeled layers, two passes). The backward keeps rows: 8x4 gave 1% there, opaque, and lost
+// 1.5% on peeled layers, and the other order of its atomics flips Adam's first step at texels
+// whose gradients cancel.
 template <int THREADS, int COLS>
 __device__ __forceinline__ void band_pixel(int W, int& px, int& py) {
     constexpr int PARTS = 256 / THREADS, ACROSS = ADMS_TILE / COLS, ROWS = 32 / COLS;
@@ -89,7 +89,7 @@ template <bool PEEL, int SHARE>
 __global__ void __launch_bounds__(ADMS_BWD_THREADS, bwd_blocks(SHARE)) k_shade_bwd(ShadeArgs A) {
     __shared__ float rows[(ADMS_BWD_THREADS / 32) * 32 * ADMS_VROW];
     int px, py;
-    band_pixel<ADMS_BWD_THREADS, PEEL ? 16 : 8>(A.W, px, py);
+    band_pixel<ADMS_BWD_THREADS, 16>(A.W, px, py);
     shade_bwd_px<PEEL, SHARE>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
 }
 
@@ -367,8 +367,7 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers) {
     if (list) {
         // a few thousand pixels, a long dependent chain each: small blocks spread them over every
         // SM (128 blocks of 256 filled 30 SMs; the displaced mesh's shading 837 -> 822 us)
-        auto k = share == 1 ? k_shade_refine<1> : share == 2 ? k_shade_refine<2> : k_shade_refine<0>;
-        k<<<608, 64, 0, st>>>(a);
+        k_shade_refine<<<608, 64, 0, st>>>(a);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -392,8 +391,8 @@ cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st) {
         k_shade_bwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
     } else {
         int share = share_of(a);
-        auto k = a.peel ? (share == 1 ? k_shade_bwd<true, 1> : share == 2 ? k_shade_bwd<true, 2> : k_shade_bwd<true, 0>)
-                        : (share == 1 ? k_shade_bwd<false, 1> : share == 2 ? k_shade_bwd<false, 2> : k_shade_bwd<false, 0>);
+        auto k = a.peel ? (share == 1 ? k_shade_bwd<true, -1> : share == 2 ? k_shade_bwd<true, 2> : k_shade_bwd<true, 0>)
+                        : (share == 1 ? k_shade_bwd<false, -1> : share == 2 ? k_shade_bwd<false, 2> : k_shade_bwd<false, 0>);
         k<<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
     }
     count_launches(1);
