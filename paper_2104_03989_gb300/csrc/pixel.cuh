@@ -1103,11 +1103,12 @@ __device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoo
     }
 }
 
-// Measured (us), sizes that differ read twice -> stashed, and one LOD and footprint for the last
+// Measured (us), maps of different sizes, texels read twice -> derivatives stashed, and one LOD and footprint for the last
 // two maps where those are of one size (SHARE 2), one load for a map of one texel: backward of
 // 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the others constant) 1388 ->
-// 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2154, of 5 views of 333x501
+// 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of 5 views of 333x501
 // (512^2, 128^2, 256^2) 79.4 -> 76.8; their forward shading 801 -> 730, 878 -> 838, 80 -> 80.
+//
 // shading adjoint of triangle f at sample (px, py) for dL/d(colour) gc (and, for a
 // peeled layer, dL/d(opacity) g_alpha): texel gradients scattered here, the three
 // corners' position / normal / tangent gradients written to vrow[27] (corner k at
