@@ -328,7 +328,7 @@ __host__ __device__ __forceinline__ bool shared_taps(const ShadeArgs& A) {
            A.kd.levels == A.orm.levels && A.kd.levels == A.nrm.levels;
 }
 
-// a map of one texel has that value everywhere: no footprint, no dependence on the coordinate
+// a map of one texel: no dependence on the coordinate (used by the adjoint, see shading_adjoint)
 __host__ __device__ __forceinline__ bool constant_map(const TexDev& t) { return t.w0 == 1 && t.h0 == 1; }
 
 // How a launch of its own kernel (SHARE) samples the maps: 1 all three share their taps, 2 orm
@@ -367,10 +367,6 @@ __device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& 
     }
 }
 
-__device__ __forceinline__ float4 map_sample(const TexDev& t, const TexCoord& tc, float lod) {
-    return constant_map(t) ? __ldg(t.tex) : tex_sample(t, tc, lod);
-}
-
 // the shading inputs at g: interpolated attributes and the three maps' trilinear samples
 // (their LODs into lod). One LOD and one footprint per level serve maps of one size (57.2 ->
 // 44.0 M warp instructions, 83 -> 73.5 us for 8 views of 512x512).
@@ -393,15 +389,15 @@ __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo
         lod[1] = lod[2] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
         float4 smp[3];
         tex_sample3<1>(A, g.tc, lod[1], smp);
-        in.kd = map_sample(A.kd, g.tc, lod[0]);
+        in.kd = tex_sample(A.kd, g.tc, lod[0]);
         in.orm = smp[1];
         in.nm = smp[2];
     } else {
         lod[1] = tex_lod(A.orm, g.duv_dx, g.duv_dy);
         lod[2] = tex_lod(A.nrm, g.duv_dx, g.duv_dy);
-        in.kd = SHARE < 0 ? tex_sample(A.kd, g.tc, lod[0]) : map_sample(A.kd, g.tc, lod[0]);
-        in.orm = SHARE < 0 ? tex_sample(A.orm, g.tc, lod[1]) : map_sample(A.orm, g.tc, lod[1]);
-        in.nm = SHARE < 0 ? tex_sample(A.nrm, g.tc, lod[2]) : map_sample(A.nrm, g.tc, lod[2]);
+        in.kd = tex_sample(A.kd, g.tc, lod[0]);
+        in.orm = tex_sample(A.orm, g.tc, lod[1]);
+        in.nm = tex_sample(A.nrm, g.tc, lod[2]);
     }
     return in;
 }
@@ -1103,11 +1099,13 @@ __device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoo
     }
 }
 
-// Measured (us), maps of different sizes, texels read twice -> derivatives stashed, and one LOD and footprint for the last
-// two maps where those are of one size (SHARE 2), one load for a map of one texel: backward of
-// 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the others constant) 1388 ->
-// 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of 5 views of 333x501
-// (512^2, 128^2, 256^2) 79.4 -> 76.8; their forward shading 801 -> 730, 878 -> 838, 80 -> 80.
+// Measured (us), maps of different sizes: texels read twice -> derivatives stashed, one LOD and
+// footprint for the last two maps where those are of one size (SHARE 2), one load for a map of
+// one texel: backward of 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the
+// others constant) 1388 -> 1183, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of
+// 5 views of 333x501 (512^2, 128^2, 256^2) 79.4 -> 77. The forward takes the pair's form (878 -> 822
+// for the layers), but reads a map of one texel as any other: the texel itself (730 instead of 800 us) is
+// not the rounded sum of its four weights, and a colour that moves by an ulp can turn an L1 loss.
 //
 // shading adjoint of triangle f at sample (px, py) for dL/d(colour) gc (and, for a
 // peeled layer, dL/d(opacity) g_alpha): texel gradients scattered here, the three
