@@ -1102,7 +1102,7 @@ __device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoo
 // Measured (us), maps of different sizes: texels read twice -> derivatives stashed, one LOD and
 // footprint for the last two maps where those are of one size (SHARE 2), one load for a map of
 // one texel: backward of 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the
-// others constant) 1388 -> 1183, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of
+// others constant) 1388 -> 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of
 // 5 views of 333x501 (512^2, 128^2, 256^2) 79.4 -> 77. The forward takes the pair's form (878 -> 822
 // for the layers), but reads a map of one texel as any other: the texel itself (730 instead of 800 us) is
 // not the rounded sum of its four weights, and a colour that moves by an ulp can turn an L1 loss.

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(Sha
 #define ADMS_BWD_THREADS 128  // 256: a block per 16x16 tile; 128: two blocks of 16x8 pixels
 #endif
 // SHARE 2 at 7: eight peeled layers 2169 -> 2115 us, 8 opaque views of 512x512 180.2 -> 178.6;
-// the other forms lose (maps of three sizes 76.3 -> 77.6, one map and constants 1183 -> 1190)
+// the other forms lose (maps of three sizes 76.3 -> 77.6, one map and constants 0.6% slower)
 constexpr int bwd_blocks(int share) { return share == 2 ? ADMS_BWD_BLOCKS + 1 : ADMS_BWD_BLOCKS; }
 template <bool PEEL, int SHARE>
 __global__ void __launch_bounds__(ADMS_BWD_THREADS, bwd_blocks(SHARE)) k_shade_bwd(ShadeArgs A) {
