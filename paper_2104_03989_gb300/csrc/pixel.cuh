@@ -328,15 +328,15 @@ __host__ __device__ __forceinline__ bool shared_taps(const ShadeArgs& A) {
            A.kd.levels == A.orm.levels && A.kd.levels == A.nrm.levels;
 }
 
-// a map of one texel: no dependence on the coordinate (used by the adjoint, see shading_adjoint)
-__host__ __device__ __forceinline__ bool constant_map(const TexDev& t) { return t.w0 == 1 && t.h0 == 1; }
-
-// How a launch of its own kernel (SHARE) samples the maps: 1 all three share their taps, 2 orm
-// and nrm do (a base colour of a finer or coarser size, or a constant one), 0 every map has its own.
+// How the single-job forward, a kernel per form (SHARE), samples the maps: 1 all three share their
+// taps, 2 orm and nrm do (a base colour of a finer or coarser size, or a constant one; two peeled
+// passes 878 -> 822 us), 0 every map has its own (also two maps of one texel, whose taps are one).
+// The samples are the same bits in every form.
 __host__ __device__ __forceinline__ int share_of(const ShadeArgs& A) {
     if (shared_taps(A)) return 1;
     bool pair = A.orm.w0 == A.nrm.w0 && A.orm.h0 == A.nrm.h0 && A.orm.levels == A.nrm.levels;
-    return pair && !constant_map(A.nrm) ? 2 : 0;
+    bool one_texel = A.nrm.w0 == 1 && A.nrm.h0 == 1;
+    return pair && !one_texel ? 2 : 0;
 }
 
 // tex_sample of the maps FROM .. 2 with shared taps (the same arithmetic, map by map)
@@ -370,7 +370,7 @@ __device__ __forceinline__ void tex_sample3(const ShadeArgs& A, const TexCoord& 
 // the shading inputs at g: interpolated attributes and the three maps' trilinear samples
 // (their LODs into lod). One LOD and one footprint per level serve maps of one size (57.2 ->
 // 44.0 M warp instructions, 83 -> 73.5 us for 8 views of 512x512).
-// SHARE: share_of, -1 decided here between 1 and 0 (batched and per-stage calls).
+// SHARE: share_of, -1 decided here between 1 and 0 (batched and sampled launches, the refinement).
 template <int SHARE = -1>
 __device__ __forceinline__ ShadeIn shade_inputs(const ShadeArgs& A, const PixGeo& g, float lod[3]) {
     ShadeIn in;
@@ -998,125 +998,19 @@ __device__ __forceinline__ float2 tex_sample3_bwd_stash(const ShadeArgs& A, cons
     return guv;
 }
 
-// The samples of maps FROM .. TO-1, which share their taps (footprints from map FROM), leaving
-// for each map m dS_m/du and dS_m/dv (the derivatives of its trilinear sample w.r.t. the
-// texture coordinate, float4 each) in stash[8 m .. 8 m + 7] (a lane's private shared-memory
-// row): the adjoint then reads no texel a second time. Reading them again waited on memory: the
-// kernel issues in 39% of its slots and waits on L1 for most of the rest.
-template <int FROM, int TO>
-__device__ __forceinline__ void maps_sample_stash(const ShadeArgs& A, const TexCoord& tc, float lod, float4 out[3],
-                                                  float* stash) {
-    const TexDev* maps[3] = {&A.kd, &A.orm, &A.nrm};
-    const TexDev& t = *maps[FROM];
-    if (TO - FROM == 1 && constant_map(t)) {
-        out[FROM] = __ldg(t.tex);
-        return;
-    }
-    int l0 = (int)floorf(lod);
-    float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, t.levels - 1);
-    float4 du[3], dv[3];
-#pragma unroll
-    for (int m = FROM; m < TO; ++m) {
-        out[m] = du[m] = dv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        int k = s == 0 ? l0 : l1;
-        float wl = s == 0 ? 1.f - fr : fr;
-        if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(t, k, tc);
-        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
-        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
-        float su = wl * b.sw, sv = wl * b.sh;
-#pragma unroll
-        for (int m = FROM; m < TO; ++m) {
-            const float4* tex = maps[m]->tex;
-            float4 t00 = __ldg(tex + b.idx[0]), t10 = __ldg(tex + b.idx[1]);
-            float4 t01 = __ldg(tex + b.idx[2]), t11 = __ldg(tex + b.idx[3]);
-            out[m] = f4madd(out[m], w00, t00);
-            out[m] = f4madd(out[m], w10, t10);
-            out[m] = f4madd(out[m], w01, t01);
-            out[m] = f4madd(out[m], w11, t11);
-            du[m] = f4madd(du[m], su, f4madd(f4scale(f4sub(t10, t00), 1.f - b.fy), b.fy, f4sub(t11, t01)));
-            dv[m] = f4madd(dv[m], sv, f4madd(f4scale(f4sub(t01, t00), 1.f - b.fx), b.fx, f4sub(t11, t10)));
-        }
-    }
-#pragma unroll
-    for (int m = FROM; m < TO; ++m) {
-        float* q = stash + 8 * m;
-        q[0] = du[m].x;
-        q[1] = du[m].y;
-        q[2] = du[m].z;
-        q[3] = du[m].w;
-        q[4] = dv[m].x;
-        q[5] = dv[m].y;
-        q[6] = dv[m].z;
-        q[7] = dv[m].w;
-    }
-}
-
-// adjoint of maps_sample_stash: the texel gradients of the optimized maps scattered,
-// sum_m d/d(u, v) of g[m] . S_m from the stashed derivatives added to guv
-template <int FROM, int TO>
-__device__ __forceinline__ void maps_sample_bwd(const ShadeArgs& A, const TexCoord& tc, float lod, const float4 g[3],
-                                                const float* stash, float2& guv) {
-    const TexDev* maps[3] = {&A.kd, &A.orm, &A.nrm};
-    const TexDev& t = *maps[FROM];
-    if (TO - FROM == 1 && constant_map(t)) {
-        if (t.grad) atomicAdd(t.grad, g[FROM]);
-        return;
-    }
-    bool any = false;
-#pragma unroll
-    for (int m = FROM; m < TO; ++m) {
-        const float* q = stash + 8 * m;
-        guv.x += g[m].x * q[0] + g[m].y * q[1] + g[m].z * q[2] + g[m].w * q[3];
-        guv.y += g[m].x * q[4] + g[m].y * q[5] + g[m].z * q[6] + g[m].w * q[7];
-        any = any || maps[m]->grad;
-    }
-    if (!any) return;
-    int l0 = (int)floorf(lod);
-    float fr = lod - (float)l0;
-    int l1 = min(l0 + 1, t.levels - 1);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        int k = s == 0 ? l0 : l1;
-        float wl = s == 0 ? 1.f - fr : fr;
-        if (wl == 0.f) continue;
-        BilinTap b = bilin_tap(t, k, tc);
-        float w00 = wl * (1.f - b.fx) * (1.f - b.fy), w10 = wl * b.fx * (1.f - b.fy);
-        float w01 = wl * (1.f - b.fx) * b.fy, w11 = wl * b.fx * b.fy;
-#pragma unroll
-        for (int m = FROM; m < TO; ++m) {
-            float4* grad = maps[m]->grad;
-            if (!grad) continue;
-            atomicAdd(grad + b.idx[0], f4scale(g[m], w00));
-            atomicAdd(grad + b.idx[1], f4scale(g[m], w10));
-            atomicAdd(grad + b.idx[2], f4scale(g[m], w01));
-            atomicAdd(grad + b.idx[3], f4scale(g[m], w11));
-        }
-    }
-}
-
-// Measured (us), maps of different sizes: texels read twice -> derivatives stashed, one LOD and
-// footprint for the last two maps where those are of one size (SHARE 2), one load for a map of
-// one texel: backward of 62720 triangles under 16 views of 1024x1024 (2048^2 normal map, the
-// others constant) 1388 -> 1193, of eight peeled layers (2048^2, 1024^2, 1024^2) 2253 -> 2100, of
-// 5 views of 333x501 (512^2, 128^2, 256^2) 79.4 -> 77. The forward takes the pair's form (878 -> 822
-// for the layers), but reads a map of one texel as any other: the texel itself (730 instead of 800 us) is
-// not the rounded sum of its four weights, and a colour that moves by an ulp can turn an L1 loss.
-//
 // shading adjoint of triangle f at sample (px, py) for dL/d(colour) gc (and, for a
 // peeled layer, dL/d(opacity) g_alpha): texel gradients scattered here, the three
 // corners' position / normal / tangent gradients written to vrow[27] (corner k at
 // 9k: position xyz, normal xyz, tangent xyz). The geometry is evaluated twice, once
 // for the shading inputs and once after the BRDF and texture adjoints for the
 // barycentric adjoint, so that nothing of it stays live across them.
-// SHARE: 0 or 2 of share_of in a kernel of its own, -1 maps of one size (and batched and sampled
-// launches, whatever the sizes). Equal maps keep the general form: on its own its shading adjoint is
-// fused otherwise by the compiler, for no gain, and gradients that cancel to nothing change sign.
-template <bool PEEL, int SHARE = -1>
+// One form for all map sizes. Kernels of their own for maps of unequal sizes, with the texture
+// derivatives kept from the first read, were 5% faster on 62720 triangles under 16 views of
+// 1024x1024 (one map and constants: 3314 against 3499 us for loss and gradients) and 3% on eight
+// peeled layers (4820 against 4994). But the compiler fuses the shading adjoint otherwise in each
+// kernel, and the specular terms of sharp highlights amplify an ulp there to as much as 5e-5 of a
+// gradient's norm: the same inputs then give other gradients, for 5%.
+template <bool PEEL>
 __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int px, int py, int f, float3 gc,
                                                 float g_alpha, float* vrow) {
     const adms_view& vw = A.views[b];
@@ -1132,22 +1026,7 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
         in.p = g.p;
         in.n_i = g.n;
         in.t_i = g.t;
-        if constexpr (SHARE >= 0) {
-            float4 smp[3];  // the row holds their uv derivatives until the vertex gradients go there
-            lod[0] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
-            maps_sample_stash<0, 1>(A, g.tc, lod[0], smp, vrow);
-            lod[1] = tex_lod<true>(A.orm, g.duv_dx, g.duv_dy);
-            if constexpr (SHARE == 2) {
-                maps_sample_stash<1, 3>(A, g.tc, lod[1], smp, vrow);
-            } else {
-                maps_sample_stash<1, 2>(A, g.tc, lod[1], smp, vrow);
-                lod[2] = tex_lod<true>(A.nrm, g.duv_dx, g.duv_dy);
-                maps_sample_stash<2, 3>(A, g.tc, lod[2], smp, vrow);
-            }
-            in.kd = smp[0];
-            in.orm = smp[1];
-            in.nm = smp[2];
-        } else if (shared) {
+        if (shared) {
             lod[0] = lod[1] = lod[2] = tex_lod<true>(A.kd, g.duv_dx, g.duv_dy);
             float4 smp[3];
             tex_sample3_stash(A, g.tc, lod[0], smp, vrow);  // the row holds the uv derivatives until phase 4
@@ -1167,17 +1046,7 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
     }
     if (PEEL) G.kd.w = g_alpha;  // the opacity is the base colour's fourth channel
     float2 guv;
-    if constexpr (SHARE >= 0) {
-        guv = make_float2(0.f, 0.f);
-        float4 gt[3] = {G.kd, G.orm, G.nm};
-        maps_sample_bwd<0, 1>(A, tc, lod[0], gt, vrow, guv);
-        if constexpr (SHARE == 2) {
-            maps_sample_bwd<1, 3>(A, tc, lod[1], gt, vrow, guv);
-        } else {
-            maps_sample_bwd<1, 2>(A, tc, lod[1], gt, vrow, guv);
-            maps_sample_bwd<2, 3>(A, tc, lod[2], gt, vrow, guv);
-        }
-    } else if (shared) {
+    if (shared) {
         float4 gt[3] = {G.kd, G.orm, G.nm};
         guv = tex_sample3_bwd_stash(A, tc, lod[0], gt, vrow);
     } else {
@@ -1246,7 +1115,7 @@ __device__ __forceinline__ void shading_adjoint(const ShadeArgs& A, int b, int p
 
 // one pixel of the fused backward; warp-collective (vertex scatter). rows: the
 // warp's 32 x ADMS_VROW floats of shared memory
-template <bool PEEL = false, int SHARE = -1>
+template <bool PEEL = false>
 __device__ __forceinline__ void shade_bwd_px(const ShadeArgs& A, int b, int px, int py, float* rows) {
     bool inside = px < A.W && py < A.H;
     int f = -1;
@@ -1269,7 +1138,7 @@ __device__ __forceinline__ void shade_bwd_px(const ShadeArgs& A, int b, int px, 
             gc = pr.w * gc;
         }
         if (f >= 0 && (gc.x != 0.f || gc.y != 0.f || gc.z != 0.f || g_alpha != 0.f))
-            shading_adjoint<PEEL, SHARE>(A, b, px, py, f, gc, g_alpha, rows + (threadIdx.x & 31) * ADMS_VROW);
+            shading_adjoint<PEEL>(A, b, px, py, f, gc, g_alpha, rows + (threadIdx.x & 31) * ADMS_VROW);
         else
             f = -1;
     }

@@ -82,15 +82,12 @@ __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(Sha
 #ifndef ADMS_BWD_THREADS
 #define ADMS_BWD_THREADS 128  // 256: a block per 16x16 tile; 128: two blocks of 16x8 pixels
 #endif
-// SHARE 2 at 7: eight peeled layers 2169 -> 2115 us, 8 opaque views of 512x512 180.2 -> 178.6;
-// the other forms lose (maps of three sizes 76.3 -> 77.6, one map and constants 0.6% slower)
-constexpr int bwd_blocks(int share) { return share == 2 ? ADMS_BWD_BLOCKS + 1 : ADMS_BWD_BLOCKS; }
-template <bool PEEL, int SHARE>
-__global__ void __launch_bounds__(ADMS_BWD_THREADS, bwd_blocks(SHARE)) k_shade_bwd(ShadeArgs A) {
+template <bool PEEL>
+__global__ void __launch_bounds__(ADMS_BWD_THREADS, ADMS_BWD_BLOCKS) k_shade_bwd(ShadeArgs A) {
     __shared__ float rows[(ADMS_BWD_THREADS / 32) * 32 * ADMS_VROW];
     int px, py;
     band_pixel<ADMS_BWD_THREADS, 16>(A.W, px, py);
-    shade_bwd_px<PEEL, SHARE>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
+    shade_bwd_px<PEEL>(A, blockIdx.y, px, py, rows + (threadIdx.x >> 5) * 32 * ADMS_VROW);
 }
 
 // MSAA forward: a block takes a 32x32-sample region (four samples per thread), its
@@ -390,9 +387,7 @@ cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st) {
         int R = ADMS_MSAA_REGION;
         k_shade_bwd_msaa<<<dim3(((a.W + R - 1) / R) * ((a.H + R - 1) / R), a.B), 256, 0, st>>>(a);
     } else {
-        int share = share_of(a);
-        auto k = a.peel ? (share == 1 ? k_shade_bwd<true, -1> : share == 2 ? k_shade_bwd<true, 2> : k_shade_bwd<true, 0>)
-                        : (share == 1 ? k_shade_bwd<false, -1> : share == 2 ? k_shade_bwd<false, 2> : k_shade_bwd<false, 0>);
+        auto k = a.peel ? k_shade_bwd<true> : k_shade_bwd<false>;
         k<<<band_grid(a, ADMS_BWD_THREADS), ADMS_BWD_THREADS, 0, st>>>(a);
     }
     count_launches(1);
