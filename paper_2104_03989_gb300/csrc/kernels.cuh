@@ -172,6 +172,8 @@ cudaError_t shade_forward(const ShadeArgs& a, cudaStream_t st, int layers = 1);
 // finish_call_loss(finish, out); *finished tells whether it will
 cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st, struct JobState* finish = nullptr, float* out = nullptr,
                             bool* finished = nullptr);
+// the same of opaque colours that are a caller's, those of empty pixels too
+cudaError_t aa_loss_given(const ShadeArgs& a, cudaStream_t st);
 cudaError_t shade_backward(const ShadeArgs& a, cudaStream_t st);
 
 // per-pixel resolve of a supersampled render: pixel = mean of its s x s antialiased

@@ -695,13 +695,15 @@ __device__ __forceinline__ unsigned silhouette_pairs(const ShadeArgs& A, int b, 
 // AA, loss terms and dL/d(AA colour) of one pixel; its loss terms go to sum. Issue-bound (83%
 // of the slots at 742 instructions a warp): the four neighbours share one copy of the pair
 // code, which only pixels beside another triangle enter, told by the keys' low words (the
-// neighbours' at constant offsets), and empty pixels read no colour. 8 views of 512x512 53 ->
+// neighbours' at constant offsets), and empty pixels read no colour of the shading's. 8 views of 512x512 53 ->
 // 49 us, 16 of 1024x1024 (two passes) 703 -> 671, 16 passes over peeled layers 1023 -> 1005.
 // Strips of 2 or 4 rows per thread (ids reused downwards, a quarter of the block sums) lost
 // more in loads in flight than they saved (52 and 56 us), blocks of 256 threads too (51).
 // PEEL: A is a layer of a depth-peeled composite (A.peel set); a separate
 // instantiation keeps the opaque path's registers to its own needs
-template <bool PEEL>
+// GIVEN: the colours are the caller's (per-stage call), empty pixels' too; elsewhere the
+// shading has left those black
+template <bool PEEL, bool GIVEN = false>
 __device__ __forceinline__ void aa_pixel(const ShadeArgs& A, int b, int px, int py, LossSum& sum) {
     if (px >= A.W || py >= A.H) return;
     size_t pix = ((size_t)b * A.H + py) * A.W + px;
@@ -710,7 +712,7 @@ __device__ __forceinline__ void aa_pixel(const ShadeArgs& A, int b, int px, int 
     int id = __ldg(ids + 2 * pix);
     int up = py > 0 ? __ldg(ids + 2 * (pix - A.W)) : id, down = py + 1 < A.H ? __ldg(ids + 2 * (pix + A.W)) : id;
     int left = px > 0 ? __ldg(ids + 2 * pix - 2) : id, right = px + 1 < A.W ? __ldg(ids + 2 * pix + 2) : id;
-    float4 own = id >= 0 ? A.pre[pix] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 own = GIVEN || id >= 0 ? A.pre[pix] : make_float4(0.f, 0.f, 0.f, 0.f);
     float y0 = 0.f, y1 = 0.f, y2 = 0.f;
     if (A.ref) {
         const float* y = A.ref + pix * 3;

@@ -62,12 +62,12 @@ __global__ void __launch_bounds__(ADMS_FWD_THREADS, fwd_blocks(INLINE, SHARE)) k
 }
 
 // FINISH: the last block finishes the call's loss (a launch of its own otherwise)
-template <bool PEEL, bool FINISH>
+template <bool PEEL, bool FINISH, bool GIVEN = false>
 __global__ void __launch_bounds__(ADMS_AA_THREADS, ADMS_AA_BLOCKS) k_aa_loss(ShadeArgs A, JobState* fin, float* out) {
     __shared__ float red[ADMS_AA_THREADS / 16];
     int bx = (A.W + 31) / 32;  // a warp takes 32 columns of one row
     LossSum sum;
-    aa_pixel<PEEL>(A, blockIdx.y, (blockIdx.x % bx) * 32 + (threadIdx.x & 31),
+    aa_pixel<PEEL, GIVEN>(A, blockIdx.y, (blockIdx.x % bx) * 32 + (threadIdx.x & 31),
                    (blockIdx.x / bx) * (ADMS_AA_THREADS / 32) + (threadIdx.x >> 5), sum);
     add_block_loss(A, sum, red);
     if (FINISH && threadIdx.x == 0 && last_block(fin, TICKET_LOSS, gridDim.x * gridDim.y)) finish_job_loss(fin, out);
@@ -379,6 +379,13 @@ cudaError_t aa_loss_forward(const ShadeArgs& a, cudaStream_t st, JobState* finis
     if (finished) *finished = fin;
     auto k = a.peel ? k_aa_loss<true, false> : fin ? k_aa_loss<false, true> : k_aa_loss<false, false>;
     k<<<grid, ADMS_AA_THREADS, 0, st>>>(a, finish, out);
+    count_launches(1);
+    return cudaGetLastError();
+}
+cudaError_t aa_loss_given(const ShadeArgs& a, cudaStream_t st) {
+    int rows = ADMS_AA_THREADS / 32;
+    dim3 grid(((a.W + 31) / 32) * ((a.H + rows - 1) / rows), a.B);
+    k_aa_loss<false, false, true><<<grid, ADMS_AA_THREADS, 0, st>>>(a, nullptr, nullptr);
     count_launches(1);
     return cudaGetLastError();
 }

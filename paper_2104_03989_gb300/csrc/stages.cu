@@ -606,7 +606,7 @@ adms_status adms_aa_loss_fwd(const adms_stage_mesh* m, const adms_view* views, i
     a.loss_acc = ref ? loss : nullptr;
     a.gprime = reinterpret_cast<float4*>(gprime);
     a.out_img = img;
-    ADMS_STAGE_CHECK(aa_loss_forward(a, (cudaStream_t)cuda_stream));
+    ADMS_STAGE_CHECK(aa_loss_given(a, (cudaStream_t)cuda_stream));
     return ADMS_OK;
 }
 
