@@ -59,6 +59,20 @@ def _order(waiting, stream, tensors=()):
             t.record_stream(waiting)
 
 
+def _ordinary(g):
+    """Whether an incoming gradient is a plain tensor of values: no graph to keep (create_graph), no forward-mode
+    tangent, not batched or wrapped by a function transform (those have no data of their own)."""
+    if type(g) is not torch.Tensor or (torch.is_grad_enabled() and g.requires_grad):
+        return False
+    if torch.autograd.forward_ad._current_level >= 0:
+        return False
+    try:
+        g.data_ptr()
+    except RuntimeError:
+        return False
+    return True
+
+
 class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def forward(fctx, ctx, job, views, refs, names, *tensors):
@@ -75,15 +89,19 @@ class _RenderLoss(torch.autograd.Function):
     def backward(fctx, g):
         ctx, job = fctx.ctx, fctx.job
         here, there = torch.cuda.current_stream(), _context_stream(ctx)
-        scale = g.detach().to(torch.float32).contiguous()
         grads = [torch.empty(shape, dtype=torch.float32, device=g.device) for shape in fctx.shapes]
-        _order(there, here, (scale, *grads))
+        # an ordinary incoming gradient goes along as the scale of the one pass that hands the job's
+        # out; one that torch follows further (a graph, a batch, a tangent) multiplies them in torch
+        scale = g.detach().to(torch.float32).contiguous() if _ordinary(g) else None
+        _order(there, here, grads if scale is None else (scale, *grads))
         B.adms_job_zero_gradients(ctx.ctx, job)
         ctx.backward([job], recompute_raster=True)
-        # times the incoming gradient, folded over the mip chains, the job's buffers left at
-        # zero: one pass over each, and nothing for the host to wait for
+        # folded over the mip chains, the job's buffers left at zero: one pass over each, and
+        # nothing for the host to wait for
         B.adms_job_take_gradients(ctx.ctx, job, scale, **{_TAKE[n]: buf for n, buf in zip(fctx.names, grads)})
         _order(here, there)
+        if scale is None:
+            grads = [buf * g for buf in grads]
         return (None, None, None, None, None, *grads)
 
 
