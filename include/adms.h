@@ -262,6 +262,8 @@ adms_status adms_job_set_bones(adms_ctx* ctx, adms_job job, const float* bones);
  * (the job stays valid), ADMS_ERR_ARG for non-positive or > 16384 sizes. */
 adms_status adms_job_reserve(adms_ctx* ctx, adms_job job, int32_t n_views, int32_t H, int32_t W);
 adms_status adms_job_params(adms_ctx* ctx, adms_job job, adms_param_view* out);
+/* The sizes of a job's latents alone (pointers and t zero): touches no device. */
+adms_status adms_job_sizes(adms_ctx* ctx, adms_job job, adms_param_view* out);
 adms_status adms_job_stats(adms_ctx* ctx, adms_job job, adms_stats* out);
 /* The latched status of each job (0, or e.g. ADMS_ERR_NONFINITE) into out
  * (device, [n_jobs] int32), ordered on the context's stream like the step

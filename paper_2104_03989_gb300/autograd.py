@@ -18,6 +18,8 @@ frame are rebuilt.
 
 from __future__ import annotations
 
+import math
+
 import torch
 
 from . import binding as B
@@ -73,6 +75,16 @@ def _ordinary(g):
     return True
 
 
+def _gradient_shapes(ctx, job, names, shapes):
+    """The shapes of the buffers that the library fills whole: the job's own, whatever tensors the caller passed
+    (a texture's may come in another shape of as many texels; torch refuses a gradient that does not fit)."""
+    z = B.adms_job_sizes(ctx.ctx, job)
+    own = {"pos": (z.n_verts, 3), "disp": (z.disp_h, z.disp_w), "w": (z.n_verts, z.n_bones),
+           **{k: (getattr(z, k + "_h"), getattr(z, k + "_w"), 4) for k in TEXTURES}}
+    return [shape if n in TEXTURES and math.prod(shape) == math.prod(own[n]) else own[n]
+            for n, shape in zip(names, shapes)]
+
+
 class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def forward(fctx, ctx, job, views, refs, names, *tensors):
@@ -89,7 +101,8 @@ class _RenderLoss(torch.autograd.Function):
     def backward(fctx, g):
         ctx, job = fctx.ctx, fctx.job
         here, there = torch.cuda.current_stream(), _context_stream(ctx)
-        grads = [torch.empty(shape, dtype=torch.float32, device=g.device) for shape in fctx.shapes]
+        grads = [torch.empty(shape, dtype=torch.float32, device=g.device)
+                 for shape in _gradient_shapes(ctx, job, fctx.names, fctx.shapes)]
         # an ordinary incoming gradient goes along as the scale of the one pass that hands the job's
         # out; one that torch follows further (a graph, a batch, a tangent) multiplies them in torch
         scale = g.detach().to(torch.float32).contiguous() if _ordinary(g) else None

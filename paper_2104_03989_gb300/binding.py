@@ -107,6 +107,7 @@ SIGNATURES = {
     "adms_job_skinning": ([P, C.c_int32, P, C.c_int32, C.c_float], C.c_int),
     "adms_job_set_bones": ([P, C.c_int32, P], C.c_int),
     "adms_job_params": ([P, C.c_int32, C.POINTER(adms_param_view)], C.c_int),
+    "adms_job_sizes": ([P, C.c_int32, C.POINTER(adms_param_view)], C.c_int),
     "adms_job_stats": ([P, C.c_int32, C.POINTER(adms_stats)], C.c_int),
     "adms_jobs_status": ([P, P, C.c_int32, P], C.c_int),
     "adms_render_reference": ([P, C.c_int32, P, C.c_int32, C.c_int32, C.c_int32, P], C.c_int),
@@ -286,6 +287,12 @@ def adms_job_reserve(ctx, job, n_views, H, W):
 def adms_job_params(ctx, job):
     out = adms_param_view()
     _check(ctx, lib().adms_job_params(ctx, job, C.byref(out)))
+    return out
+
+
+def adms_job_sizes(ctx, job):
+    out = adms_param_view()
+    _check(ctx, lib().adms_job_sizes(ctx, job, C.byref(out)))
     return out
 
 

@@ -1502,11 +1502,37 @@ adms_status adms_job_reserve(adms_ctx* ctx, adms_job job, int32_t n_views, int32
     return ensure_scratch(ctx, *j, n_views, H, W);
 }
 
+// the sizes of a job's latents (the pointers left null)
+static void param_sizes(const Job& j, adms_param_view* out) {
+    memset(out, 0, sizeof(*out));
+    out->disp_h = j.dh;
+    out->disp_w = j.dw;
+    out->n_verts = j.LV;
+    out->n_tris_render = j.F;
+    out->kd_h = j.kd.h;
+    out->kd_w = j.kd.w;
+    out->orm_h = j.orm.h;
+    out->orm_w = j.orm.w;
+    out->nrm_h = j.nrm.h;
+    out->nrm_w = j.nrm.w;
+    out->kd_levels = j.kd.levels;
+    out->orm_levels = j.orm.levels;
+    out->nrm_levels = j.nrm.levels;
+    out->n_bones = j.SB;
+}
+
+adms_status adms_job_sizes(adms_ctx* ctx, adms_job job, adms_param_view* out) {
+    Job* j = get_job(ctx, job);
+    if (!j || !out) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
+    param_sizes(*j, out);
+    return ADMS_OK;
+}
+
 adms_status adms_job_params(adms_ctx* ctx, adms_job job, adms_param_view* out) {
     Job* j = get_job(ctx, job);
     if (!j || !out) return fail(ctx, ADMS_ERR_ARG, "invalid job handle");
     if (adms_status fs = flush_job(ctx, *j)) return fs;  // its deferred texture step first
-    memset(out, 0, sizeof(*out));
+    param_sizes(*j, out);
     out->pos = j->pos;
     out->kd = (float*)j->kd.data;
     out->orm = (float*)j->orm.data;
@@ -1517,26 +1543,12 @@ adms_status adms_job_params(adms_ctx* ctx, adms_job job, adms_param_view* out) {
     out->g_nrm = (float*)j->nrm.grad;
     out->disp = j->disp;
     out->g_disp = j->g_disp;
-    out->disp_h = j->dh;
-    out->disp_w = j->dw;
-    out->n_verts = j->LV;
-    out->n_tris_render = j->F;
-    out->kd_h = j->kd.h;
-    out->kd_w = j->kd.w;
-    out->orm_h = j->orm.h;
-    out->orm_w = j->orm.w;
-    out->nrm_h = j->nrm.h;
-    out->nrm_w = j->nrm.w;
-    out->kd_levels = j->kd.levels;
-    out->orm_levels = j->orm.levels;
-    out->nrm_levels = j->nrm.levels;
     JobState hs;
     CK(cudaMemcpyAsync(&hs, j->st, sizeof(hs), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     out->t = hs.t;
     out->skin_w = j->skin_w;
     out->g_skin_w = j->g_skin_w;
-    out->n_bones = j->SB;
     return ADMS_OK;
 }
 
