@@ -18,8 +18,6 @@ frame are rebuilt.
 
 from __future__ import annotations
 
-import math
-
 import torch
 
 from . import binding as B
@@ -44,18 +42,36 @@ def latents(ctx, job, names=None):
 
 
 def invalidate(ctx, job):
+    here, there = _streams(ctx)
+    _order(there, here)  # the caller's writes to the latents
     B.adms_job_invalidate(ctx.ctx, job)
+    _order(here, there)
 
 
-def _context_stream(ctx):
-    s = ctx.stream
-    return s if hasattr(s, "cuda_stream") else torch.cuda.ExternalStream(int(s))
+def _recording(stream):
+    """Whether a graph is being recorded from the stream (never from the default one)."""
+    if stream.cuda_stream == 0:
+        return False
+    with torch.cuda.stream(stream):
+        return torch.cuda.is_current_stream_capturing()
+
+
+def _streams(ctx):
+    """torch's current stream and the context's. Twice the same, so that nothing is ordered, while the context's
+    records a graph that torch's has no part in: what is recorded runs when the graph does."""
+    there = ctx.stream
+    if getattr(there, "cuda_stream", there) == torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()):
+        return there, there
+    if not hasattr(there, "cuda_stream"):
+        there = torch.cuda.ExternalStream(int(there))
+    here = torch.cuda.current_stream()
+    return (there, there) if _recording(there) and not _recording(here) else (here, there)
 
 
 def _order(waiting, stream, tensors=()):
     """Order a stream after another's work so far and keep the tensors' memory until the waiting one is through
     with them (nothing to do when both are one stream)."""
-    if waiting.cuda_stream != stream.cuda_stream:
+    if waiting is not stream:
         waiting.wait_stream(stream)
         for t in tensors:
             t.record_stream(waiting)
@@ -79,16 +95,20 @@ def _gradient_shapes(ctx, job, names, shapes):
     """The shapes of the buffers that the library fills whole: the job's own, whatever tensors the caller passed
     (a texture's may come in another shape of as many texels; torch refuses a gradient that does not fit)."""
     z = B.adms_job_sizes(ctx.ctx, job)
-    own = {"pos": (z.n_verts, 3), "disp": (z.disp_h, z.disp_w), "w": (z.n_verts, z.n_bones),
-           **{k: (getattr(z, k + "_h"), getattr(z, k + "_w"), 4) for k in TEXTURES}}
-    return [shape if n in TEXTURES and math.prod(shape) == math.prod(own[n]) else own[n]
-            for n, shape in zip(names, shapes)]
+    out = []
+    for n, shape in zip(names, shapes):
+        if n in TEXTURES:
+            own = (getattr(z, n + "_h"), getattr(z, n + "_w"), 4)
+            out.append(shape if shape.numel() == own[0] * own[1] * 4 else own)
+        else:
+            out.append((z.disp_h, z.disp_w) if n == "disp" else (z.n_verts, z.n_bones if n == "w" else 3))
+    return out
 
 
 class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def forward(fctx, ctx, job, views, refs, names, *tensors):
-        here, there = torch.cuda.current_stream(), _context_stream(ctx)
+        here, there = _streams(ctx)
         _order(there, here, (refs,))
         loss = torch.empty((), dtype=torch.float32, device="cuda")
         ctx.forward_loss([job], [views], [refs], out_loss=loss)
@@ -100,7 +120,7 @@ class _RenderLoss(torch.autograd.Function):
     @staticmethod
     def backward(fctx, g):
         ctx, job = fctx.ctx, fctx.job
-        here, there = torch.cuda.current_stream(), _context_stream(ctx)
+        here, there = _streams(ctx)
         grads = [torch.empty(shape, dtype=torch.float32, device=g.device)
                  for shape in _gradient_shapes(ctx, job, fctx.names, fctx.shapes)]
         # an ordinary incoming gradient goes along as the scale of the one pass that hands the job's
@@ -129,7 +149,10 @@ class _Laplacian(torch.autograd.Function):
     def forward(fctx, ctx, job, pos):
         out = torch.empty((), dtype=torch.float32, device=pos.device)
         grad = torch.empty_like(pos)
+        here, there = _streams(ctx)
+        _order(there, here, (out, grad))
         B.adms_laplacian(ctx.ctx, job, out, grad)
+        _order(here, there)
         fctx.save_for_backward(grad)
         return out
 

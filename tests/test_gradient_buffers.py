@@ -23,6 +23,8 @@ def test_buffers_are_of_the_jobs_sizes(monkeypatch, pos, kd, disp, w):
     stream = SimpleNamespace(cuda_stream=0)
     handed = {}
     monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: stream)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 0, raising=False)
     monkeypatch.setattr(AG, "B", SimpleNamespace(
         adms_job_zero_gradients=lambda *a: None,
         adms_job_sizes=lambda *a: SimpleNamespace(n_verts=V, kd_h=H, kd_w=W, orm_h=1, orm_w=1, nrm_h=1, nrm_w=1, disp_h=DH,
