@@ -100,6 +100,7 @@ struct Job {
     RasterScratch rs{};
     // latest forward
     bool have_fwd = false;
+    unsigned long long fwd_capture = 0;  // the stream capture that recorded it (0: none, it ran)
     int B = 0, H = 0, W = 0;  // views and the grid the kernels work on (the sample grid when S > 1)
     // supersampled rendering (Sec. 5.2): S x S samples per pixel; MSAA shades once per
     // pixel (at its centre), ssaa shades every sample; the resolve averages them
@@ -587,6 +588,16 @@ adms_status prep_job(adms_ctx* ctx, Job& j, bool clear_grads, bool clear_loss, P
     in.small_px = j.L > 0 ? 0 : j.opt.raster_direct_px > 0 ? j.opt.raster_direct_px : ADMS_SMALL_PX;
     in.zfilter = j.opt.raster_depth_filter;
     return ADMS_OK;
+}
+
+// The stream capture that the calls are being recorded into (0: none).
+unsigned long long capture_id(adms_ctx* ctx) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(ctx->stream, &cs, &id) == cudaSuccess)
+        return cs == cudaStreamCaptureStatusActive ? id : 0;
+    (void)cudaGetLastError();  // the query's own error
+    return 0;
 }
 
 // One job's views into its buffer: pageable host memory goes with the launch of its
@@ -1743,12 +1754,17 @@ adms_status adms_forward_loss(adms_ctx* ctx, const adms_job* jobs, int32_t n_job
     std::vector<JobState*> sts;
     for (Job* jp : js) sts.push_back(jp->st);
     if (!finished) CK(TIMED(ST_SMALL, finish_call_loss(sts.data(), n_jobs, out_loss, ctx->stream)));
-    for (Job* jp : js) jp->have_fwd = true;
+    unsigned long long capture = capture_id(ctx);
+    for (Job* jp : js) {
+        jp->have_fwd = true;
+        jp->fwd_capture = capture;
+    }
     return ADMS_OK;
 }
 
 adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, int32_t recompute_raster) {
     if (!ctx || !jobs || n_jobs <= 0) return fail(ctx, ADMS_ERR_ARG, "invalid backward arguments");
+    unsigned long long capture = capture_id(ctx);
     std::vector<Job*> js;
     for (int k = 0; k < n_jobs; ++k) {
         Job* jp = get_job(ctx, jobs[k]);
@@ -1776,7 +1792,14 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
                 CK(TIMED(ST_AA_LOSS, aa_loss_forward(r, ctx->stream)));
             }
         }
-        // (the forward, or the recomputation above, cleared g_nrm, g_tan and g_rpos: prep_job)
+        // The forward, or the recomputation above, cleared g_nrm, g_tan and g_rpos (prep_job); a
+        // backward recorded without its forward clears them itself, each replay starting afresh.
+        if (!recompute_raster && j.fwd_capture != capture) {
+            ClearList c;
+            c.add(j.g_nrm, sizeof(double) * 6 * j.V);
+            if (j.tess || j.skin) c.add(j.g_rpos, sizeof(float) * 3 * j.V);
+            CK(clear_buffers(c, ctx->stream));
+        }
         if (n_jobs == 1 && j.L > 0) {
             adms_status s = peel_backward(ctx, j);
             if (s) return s;
