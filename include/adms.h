@@ -310,7 +310,9 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
  * loss is NaN or infinite, when a vertex-stage gradient sum of the backward is,
  * or (from the next step on) when this step meets a non-finite gradient
  * element, which it leaves unapplied; no latent ever receives a NaN or an
- * infinity from an update. The other jobs of a batched call are unaffected. */
+ * infinity from an update. The other jobs of a batched call are unaffected.
+ * A job named more than once takes its entries' updates one after another, all
+ * with this call's t; t advances by their number. */
 adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs);
 
 /* Level-0 gradient of each optimized texture with the adjoint of the box-filter

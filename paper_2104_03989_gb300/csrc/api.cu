@@ -1836,6 +1836,44 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
     return ADMS_OK;
 }
 
+// The step of a list that names a job more than once: its entries share the job's state, moments
+// and counters, so each entry's launches follow the one before on the context's stream (rows of
+// one launch, as below, would update them at once). All schedules first, then the flat latents,
+// the textures and the counters.
+static adms_status step_in_turn(adms_ctx* ctx, const std::vector<Job*>& js) {
+    cudaStream_t st = ctx->stream;
+    for (Job* jp : js) {
+        Job& j = *jp;
+        if (j.opt.optimize_pos && !j.lap_valid) CK(TIMED(ST_LAPLACIAN, laplacian_forward(lap_args(j), st)));
+        SchedArgs sa{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV};
+        CK(TIMED(ST_SMALL, schedule_step(&sa, 1, st)));
+    }
+    for (Job* jp : js) {
+        Job& j = *jp;
+        if (j.opt.optimize_pos) {
+            CK(TIMED(ST_LAPLACIAN, laplacian_add(lap_args(j), st)));
+            CK(TIMED(ST_ADAM, adam_flat(j.pos, j.g_pos, j.m_pos, j.v_pos, (long long)j.LV * 3, j.st, st)));
+        } else {
+            CK(cudaMemsetAsync(j.g_pos, 0, sizeof(float) * 3 * j.LV, st));
+        }
+        if (j.g_skin_w)
+            CK(TIMED(ST_ADAM, adam_flat(j.skin_w, j.g_skin_w, j.m_skin_w, j.v_skin_w, (long long)j.LV * j.SB, j.st, st,
+                                        j.skin_lr_scale)));
+        if (j.tess && j.opt.optimize_disp)
+            CK(TIMED(ST_ADAM, adam_flat(j.disp, j.g_disp, j.m_disp, j.v_disp, (long long)j.dh * j.dw, j.st, st)));
+    }
+    for (Job* jp : js) {
+        jp->frame_valid = false;
+        jp->lap_valid = false;
+        jp->tex_pending = ctx->pipeline;
+    }
+    if (ctx->pipeline) return ADMS_OK;
+    for (Job* jp : js)
+        if (adms_status s = texture_adams(ctx, {jp}, st, nullptr)) return s;
+    for (Job* jp : js) CK(TIMED(ST_SMALL, advance_step(&jp->st, 1, st)));
+    return ADMS_OK;
+}
+
 adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs) {
     if (!ctx || !jobs || n_jobs <= 0) return fail(ctx, ADMS_ERR_ARG, "invalid optimizer_step arguments");
     std::vector<Job*> js;
@@ -1848,6 +1886,11 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
     for (Job* jp : js) {
         adms_status s = flush_job(ctx, *jp);  // a step not yet consumed by a forward_loss
         if (s) return s;
+    }
+    if (n_jobs > 1) {
+        std::vector<Job*> sorted(js);
+        std::sort(sorted.begin(), sorted.end());
+        if (std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end()) return step_in_turn(ctx, js);
     }
     // the schedules (after the Laplacian when no forward computed it for these positions), with
     // the positions' step where they are optimized; then skin weights and displacement, if

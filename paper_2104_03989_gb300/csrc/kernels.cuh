@@ -369,6 +369,8 @@ struct PrepJob {
 cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st);
 // *out = L_delta after laplacian_forward
 cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st);
+// a.g_pos += lambda_t dL_delta/dpos after laplacian_forward (a latched job's is left as it is)
+cudaError_t laplacian_add(const LapArgs& a, cudaStream_t st);
 // a.g_pos = scale * dL_delta/dpos (overwrites) after laplacian_forward
 cudaError_t laplacian_gradient(const LapArgs& a, float scale, cudaStream_t st);
 #define ADMS_MIP_TEX 3  // textures per fold or rebuild launch (a job's maps)

@@ -182,6 +182,24 @@ cudaError_t laplacian_value(const LapArgs& a, float* out, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// g_pos += lambda_t dL_delta/dpos
+__global__ void k_lap_add(LapArgs a) {
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= a.V || a.st->status) return;
+    float scale = 2.f * a.st->lam / (float)a.V;
+    float3 g = f3(a.delta[3 * k], a.delta[3 * k + 1], a.delta[3 * k + 2]);
+    ring_adjoint(a, k, g);
+    a.g_pos[3 * k] += scale * g.x;
+    a.g_pos[3 * k + 1] += scale * g.y;
+    a.g_pos[3 * k + 2] += scale * g.z;
+}
+
+cudaError_t laplacian_add(const LapArgs& a, cudaStream_t st) {
+    k_lap_add<<<(a.V + 127) / 128, 128, 0, st>>>(a);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 cudaError_t laplacian_gradient(const LapArgs& a, float scale, cudaStream_t st) {
     k_lap_grad_out<<<(a.V + 127) / 128, 128, 0, st>>>(a, scale);
     count_launches(1);
