@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cstring>
 #include <vector>
 
@@ -77,6 +78,13 @@ struct alignas(16) TriRec {
 };
 static_assert(sizeof(TriRec) == 48, "two records per triangle and view fill the 96-byte allocation");
 #define ADMS_REC_PAD 2
+
+// Entries that the tile lists of a raster pass may hold: the list buffer's and those of the second
+// half of its record buffer. Never more than INT_MAX: a tile's offset is an int that saturates
+// there (k_list_alloc), and a segment that ends beyond the room is the sign to scan every triangle.
+inline long long tile_list_room(long long capacity, long long records) {
+    return std::min(capacity + records * (long long)(sizeof(TriRec) / sizeof(int)), (long long)INT_MAX);
+}
 
 // triangles with at most this many samples in their pixel bbox skip binning (default)
 #define ADMS_SMALL_PX 16

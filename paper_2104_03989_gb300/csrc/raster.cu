@@ -804,8 +804,7 @@ __global__ void __launch_bounds__(256) k_raster_kbuf(const TileArgs A, unsigned 
 }
 
 static TileLists tile_lists(const TriRec* rec, const int* list, long long capacity, long long records) {
-    return TileLists{list, reinterpret_cast<const int*>(rec + records), capacity,
-                     capacity + records * (long long)(sizeof(TriRec) / sizeof(int))};
+    return TileLists{list, reinterpret_cast<const int*>(rec + records), capacity, tile_list_room(capacity, records)};
 }
 
 struct RasterBatch {
