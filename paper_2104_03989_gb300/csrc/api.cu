@@ -608,12 +608,17 @@ adms_status put_views(adms_ctx* ctx, Job& j, const adms_view* views, int B, cons
     if (B <= ADMS_PARAM_VIEWS && !ctx->capturing) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         cudaPointerAttributes pa;
-        bool free_stream = cudaStreamIsCapturing(ctx->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
-        if (free_stream && cudaPointerGetAttributes(&pa, views) == cudaSuccess && pa.type == cudaMemoryTypeUnregistered) {
-            *by_launch = views;
-            return ADMS_OK;
+        cudaError_t e = cudaStreamIsCapturing(ctx->stream, &cs);
+        if (!e && cs == cudaStreamCaptureStatusNone) {
+            e = cudaPointerGetAttributes(&pa, views);
+            if (!e && pa.type == cudaMemoryTypeUnregistered) {
+                *by_launch = views;
+                return ADMS_OK;
+            }
         }
-        (void)cudaGetLastError();  // a failed query is no error of this call: the copy below decides
+        // a failed query is no error of this call, the copy below decides; one that was pending
+        // before the call stays for the launches to report
+        if (e) (void)cudaGetLastError();
     }
     CK(cudaMemcpyAsync(j.views, views, sizeof(adms_view) * B, cudaMemcpyDefault, ctx->stream));
     return ADMS_OK;
