@@ -854,10 +854,22 @@ cudaError_t raster_tiles_batched(const RasterJob* args, const int* item_off, int
 
 // ---------------------------------------------------------------- host launchers
 cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
-    std::vector<BeginArgs> begin(n);
-    std::vector<SetupArgs> setup(n);
-    std::vector<AllocArgs> alloc(n);
-    std::vector<FillArgs> fill(n);
+    // a single job's arguments stay on the stack: the per-stage and no-allocation calls allocate
+    // nothing, and have nobody to catch what a failed allocation throws
+    struct Args {
+        BeginArgs begin{};
+        SetupArgs setup{};
+        AllocArgs alloc{};
+        FillArgs fill{};
+    } one;
+    std::vector<BeginArgs> begins(n > 1 ? n : 0);
+    std::vector<SetupArgs> setups(n > 1 ? n : 0);
+    std::vector<AllocArgs> allocs(n > 1 ? n : 0);
+    std::vector<FillArgs> fills(n > 1 ? n : 0);
+    BeginArgs* begin = n > 1 ? begins.data() : &one.begin;
+    SetupArgs* setup = n > 1 ? setups.data() : &one.setup;
+    AllocArgs* alloc = n > 1 ? allocs.data() : &one.alloc;
+    FillArgs* fill = n > 1 ? fills.data() : &one.fill;
     bool zf = false, frame = false;
     for (int k = 0; k < n; ++k) {
         const RasterIn& in = jobs[k].in;
@@ -930,7 +942,7 @@ cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
         count_launches(1);
         e = cudaGetLastError();
     } else {
-        e = launch_packed(begin.data(), n, 256, st, k_begin<1>, k_begin<M>,
+        e = launch_packed(begin, n, 256, st, k_begin<1>, k_begin<M>,
                           [](const BeginArgs& a) { return a.nb_vert + a.nb_fill; });
     }
     auto tri_blocks = [](const SetupArgs& a) { return (a.B * a.F + 255) / 256; };
@@ -953,16 +965,16 @@ cudaError_t raster_prepare(const PrepJob* jobs, int n, cudaStream_t st) {
             e = cudaGetLastError();
         }
     } else if (!e) {
-        e = zf ? launch_packed(setup.data(), n, 256, st, k_setup<true, 1>, k_setup<true, M>, tri_blocks)
-               : launch_packed(setup.data(), n, 256, st, k_setup<false, 1>, k_setup<false, M>, tri_blocks);
+        e = zf ? launch_packed(setup, n, 256, st, k_setup<true, 1>, k_setup<true, M>, tri_blocks)
+               : launch_packed(setup, n, 256, st, k_setup<false, 1>, k_setup<false, M>, tri_blocks);
     }
     if (!e)
-        e = launch_packed(alloc.data(), n, 256, st, k_list_alloc<1>, k_list_alloc<M>,
+        e = launch_packed(alloc, n, 256, st, k_list_alloc<1>, k_list_alloc<M>,
                           [](const AllocArgs& a) { return (a.n + 255) / 256; });
     auto fill_blocks = [](const FillArgs& a) { return a.nb_frame + a.nb_lap + a.nb_fill; };
     if (!e)
-        e = frame ? launch_packed(fill.data(), n, 256, st, k_bin_fill<true, 1>, k_bin_fill<true, M>, fill_blocks)
-                  : launch_packed(fill.data(), n, 256, st, k_bin_fill<false, 1>, k_bin_fill<false, M>, fill_blocks);
+        e = frame ? launch_packed(fill, n, 256, st, k_bin_fill<true, 1>, k_bin_fill<true, M>, fill_blocks)
+                  : launch_packed(fill, n, 256, st, k_bin_fill<false, 1>, k_bin_fill<false, M>, fill_blocks);
     return e;
 }
 
