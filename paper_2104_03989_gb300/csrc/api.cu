@@ -594,6 +594,7 @@ adms_status prep_job(adms_ctx* ctx, Job& j, bool clear_grads, bool clear_loss, P
 unsigned long long capture_id(adms_ctx* ctx) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
+    if (!ctx->stream) return 0;  // the legacy default stream is never captured
     if (cudaStreamGetCaptureInfo(ctx->stream, &cs, &id) == cudaSuccess)
         return cs == cudaStreamCaptureStatusActive ? id : 0;
     (void)cudaGetLastError();  // the query's own error
