@@ -308,7 +308,19 @@ __device__ __forceinline__ void near_pack(const Edges<int>& e, int Sx, int Sy, i
 // is below the stored one. The stored key only ever decreases, so a read that lags behind
 // other threads' updates can only let an unneeded atomicMin through. Without it (closed
 // surfaces, about two fragments per sample) the read would only add a round trip.
-#define ADMS_ROUNDS_MIN (1 << 18)
+//
+// From ADMS_ROUNDS_MIN triangles x views on, a single filtered job goes in four rounds of an eighth,
+// an eighth, a quarter and a half of the triangles, between them a pass over the tiles' stored
+// depths, by which the later rounds drop what is hidden. One pass against rounds, whole renders in
+// us (leaves of half-side 0.015 - 0.03, 120 fragments on a sample at 2^22 under 8 views of 512x512):
+//   triangles x views     2^18         2^20         2^21         2^22         2^23          2^24
+//   8 of 512x512       222 : 429    386 : 461    593 : 545    992 : 738   1795 : 1132   3374 : 1874
+//   4 of 1024x1024     512 : 746   1198 : 1259  2075 : 1831  3817 : 2675  7183 : 3912  14110 : 6120
+//   4 of 256x256        93 : 161    168 : 203    260 : 272    459 : 409    838 : 682    1591 : 1225
+// The line is where every size of image gains. (Leaves so small that five fragments land on a sample,
+// which is not what the filter is for, lose 11% at 2^22 and 4% at 2^24.) Jobs of a batched call take
+// one pass: their launches are shared, and a candidate is far smaller than a reference.
+#define ADMS_ROUNDS_MIN (1 << 22)
 // resident blocks per SM: 4 (5: 1% faster on the displaced mesh, 3% slower on 11k billboards),
 // 5 with the key read, whose latency the extra warps hide (the canopy's preparation 1.15 ->
 // 1.06 ms; 6: 1.07, 3: 1.29)

@@ -5,7 +5,7 @@ layers and views) against the same views one per call (refined where they are sh
 float32 arithmetic, which the compiler may fuse otherwise in the two kernels (1e-5; a pixel refined
 with another view's camera or another layer's triangle would be off by its whole colour).
 
-The depth-filtered direct raster in rounds (2^18 triangle-views and more), its tiles looked over by
+The depth-filtered direct raster in rounds (2^22 triangle-views and more), its tiles looked over by
 a small grid (4096 tiles and more), with a last group of the triangles' permutation that is not
 full, an odd image and views whose triangles begin inside a group: keys bit for bit."""
 
@@ -48,13 +48,13 @@ def test_peeled_layers_in_one_launch_equal_one_view_a_call(gpu_lib, W, H, layers
     ctx.close()
 
 
-@pytest.mark.parametrize("quads,W,H,n", [(32803, 533, 517, 4), (43693, 641, 531, 3)])
+@pytest.mark.parametrize("quads,W,H,n", [(265003, 533, 517, 8), (700011, 641, 531, 3)])
 def test_depth_filtered_rounds_with_remainders(gpu_lib, quads, W, H, n):
     from paper_2104_03989_gb300.engine import Context
 
-    scene = _cloud(quads, (0.01, 0.03), 32, 1.0)
+    scene = _cloud(quads, (0.005, 0.015), 32, 1.0)
     pos, tri = scene.mesh.pos, scene.mesh.tri_pos
-    assert len(tri) % 64 and n * len(tri) >= 1 << 18 and n * ((W + 15) // 16) * ((H + 15) // 16) >= 2 * 2048
+    assert len(tri) % 64 and n * len(tri) >= 1 << 22 and n * ((W + 15) // 16) * ((H + 15) // 16) >= 2 * 2048
     views = synth.sample_views(6, 0, n, W, H)
     want, _ = OV.raster_views(views, pos, tri, W, H)
     ctx = Context()
@@ -66,3 +66,26 @@ def test_depth_filtered_rounds_with_remainders(gpu_lib, quads, W, H, n):
     assert (want != OV.EMPTY_KEY).any()
     torch.cuda.synchronize()
     ctx.close()
+
+
+@pytest.mark.parametrize("quads,n,rounds", [(32768, 4, False), (262143, 8, False), (262144, 8, True)])
+def test_rounds_are_taken_by_large_clouds_only(gpu_lib, quads, n, rounds):
+    """Four rounds and three passes over the tiles' depths in place of one launch. At 2^18 triangle-views the
+    rounds took 429 us where one pass takes 222."""
+    from paper_2104_03989_gb300 import binding as B
+    from paper_2104_03989_gb300.engine import Context
+
+    W = H = 64
+    views = synth.sample_views(6, 0, n, W, H)
+    launches = []
+    for zfilter in (False, True):
+        ctx = Context()
+        job = ctx.create_job(dataclasses.replace(_cloud(quads, (0.005, 0.015), 32, 1.0), optimize={}), frozen=True,
+                             raster_direct_px=256, raster_depth_filter=zfilter)
+        ctx.render_reference(job, views, H, W)
+        before = B.lib().adms_launch_count()
+        ctx.render_reference(job, views, H, W)
+        launches.append(B.lib().adms_launch_count() - before)
+        torch.cuda.synchronize()
+        ctx.close()
+    assert launches[1] - launches[0] == (6 if rounds else 0)
