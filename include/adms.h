@@ -131,9 +131,10 @@ typedef struct {
                                 the L layers' keys, layer after layer. 0: opaque rendering, the
                                 fourth channel unused */
     int32_t raster_direct_px; /* raster tuning (no counterpart in the paper; results do not depend on
-                                it): triangles whose pixel bounding box holds at most this many
-                                samples are rasterized one thread per triangle with a 64-bit atomicMin
-                                per covered sample, larger ones binned into 16x16 tiles. 0 = 16.
+                                it): triangles of up to 96 pixels a side whose pixel bounding box
+                                holds at most this many samples are rasterized directly, a lane per
+                                sample of the box with a 64-bit atomicMin per covered one, larger ones
+                                binned into 16x16 tiles. 0 = 16.
                                 Dense clouds of small triangles (e.g. a 1.2M-triangle foliage
                                 reference) run faster with a few hundred. Ignored with layers > 0
                                 (every triangle is binned). In [0, 4096] */
@@ -170,7 +171,8 @@ typedef struct {
     int32_t t;            /* optimizer steps taken */
     int32_t status;       /* 0, or an adms_status latched on the device */
     int64_t tile_overflows; /* raster tiles that fell back to a full triangle scan */
-    double call_loss;     /* L_image of the latest forward_loss call, float64 accumulation */
+    double call_loss;     /* L_image of the latest forward_loss call: float32 terms, summed per block in
+                             compensated float32 (about 2^-46) and over the blocks in float64 */
 } adms_stats;
 
 /* ---- context ------------------------------------------------------------- */

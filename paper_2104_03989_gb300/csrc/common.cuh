@@ -77,8 +77,10 @@ __device__ __forceinline__ void comp_add(float& hi, float& lo, float bhi, float 
 // every thread calls it; red: 2 floats per warp of shared memory). Float64 runs at 1/64 of
 // the float32 rate here: the warp sums in float64 held the FP64 pipe 73% busy and were most
 // of the antialiasing kernel; the compensated sums cost 8 float32 operations a step instead
-// of a 16-cycle DADD. The terms are summed scaled by 2^-16 (exact), so that no block's sum
-// leaves float32's range unless one of its terms does.
+// of a 16-cycle DADD. The terms are summed scaled by 2^-16, so that no block's sum leaves
+// float32's range unless one of its terms does (exact for terms of 2^-110 and more; what a
+// smaller one has below 2^-133 is lost). A block's sum is good to about 2^-46 of the sum of its
+// terms' sizes, where each float32 term is good to 2^-24 of itself; blocks add up in float64.
 struct LossSum {
     float hi = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(float a, float b, float c) {

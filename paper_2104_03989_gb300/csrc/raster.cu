@@ -825,7 +825,7 @@ struct RasterBatch {
 };
 // persistent: block k takes items k, k + gridDim.x, ... (the items are equal
 // 16x16 tiles, so a static stride balances them without a shared counter); the
-// jobs' arguments are kernel parameters (up to 64 jobs per launch)
+// jobs' arguments are kernel parameters (up to ADMS_BATCH_JOBS per launch)
 __global__ void __launch_bounds__(256) k_raster_batch(const __grid_constant__ RasterBatch P,
                                                       const WorkItem* __restrict__ items, int n, int job0) {
     __shared__ TileSmem<1> sm;

@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(256) k_refine_batch(const ShadeBatch P) {
 
 // Two blocks of 128 threads take a tile, as in the single-job kernels: shorter tails and finer
 // register rounding (eight uneven jobs: backward 498 -> 484 us, shading 206 -> 190, AA + loss 143
-// -> 135 against blocks of 256). The grid and the tuned blocks per SM stay in tiles.
+// -> 135 against blocks of 256). The grid and the tuned blocks per SM stay in tiles. Shading at 10
+// blocks per SM: 190 us, at the single-job kernel's 8: 208.
 constexpr int batch_blocks(int kind) { return kind == 2 ? ADMS_BWD_BLOCKS : kind == 1 ? ADMS_AA_BLOCKS : 10; }
 template <int KIND>
 __global__ void __launch_bounds__(128, batch_blocks(KIND))

@@ -224,7 +224,7 @@ class AALoss(torch.autograd.Function):
             fctx.pre = fctx.gprime = None
         else:
             fctx.pre, fctx.gprime = pre.detach(), gprime
-        return loss[0]   # float64: the per-pixel terms are summed in float64
+        return loss[0]   # float64: float32 terms, compensated float32 sums per block, float64 over the blocks
 
     @staticmethod
     def backward(fctx, g_loss):
