@@ -594,8 +594,12 @@ __global__ void __launch_bounds__(ADMS_ADAM_THREADS, ADMS_ADAM_MIN_BLOCKS)
 // thread) the next is formed from shared memory: a level costs two block barriers instead of
 // a round trip to L2.
 // CLEAR: the levels' gradients, read by every tile of the optimizer step, are cleared.
-#define ADMS_MIP_TOP_THREADS 1024
-template <bool CLEAR>
+// THREADS: 256 where level 6 has no more texels in any texture of the launch (sides of up to 1024):
+// fewer warps to meet at the barriers, and a block that finds room beside others; 1024 above. Three
+// maps with Adam's clears, 256 against 1024 threads: 5.6 : 6.1 us (512x512), 6.8 : 7.6 (1024x1024),
+// 10.9 : 8.6 (2048x2048); rebuilds 3.9 : 4.5, 4.2 : 5.2 and 8.8 : 6.8.
+inline bool mip_top_small(const TexDev& t) { return t.levels <= 6 || max(t.w0 >> 6, 1) * max(t.h0 >> 6, 1) <= 256; }
+template <bool CLEAR, int THREADS>
 __device__ __forceinline__ void mip_top(const TexDev& t, float4* s) {
     float4* tex = const_cast<float4*>(t.tex);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -606,7 +610,7 @@ __device__ __forceinline__ void mip_top(const TexDev& t, float4* s) {
         int sx = ws > 1 ? 2 : 1, sy = hs > 1 ? 2 : 1;
         float inv = 1.f / (float)(sx * sy);
         const float4* src = held ? s : tex + t.off[lv - 1];
-        bool fits = wd * hd <= ADMS_MIP_TOP_THREADS;
+        bool fits = wd * hd <= THREADS;
         float4 v = zero;
         for (int i = threadIdx.x; i < wd * hd; i += blockDim.x) {
             int x = i % wd, y = i / wd;
@@ -627,11 +631,11 @@ __device__ __forceinline__ void mip_top(const TexDev& t, float4* s) {
 }
 
 // advance: the job whose step this launch ends (the last block advances it), or null
-__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_adam_mip_top(const __grid_constant__ TexAdamBatch P,
-                                                                       JobState* advance) {
-    __shared__ float4 s[ADMS_MIP_TOP_THREADS];
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_adam_mip_top(const __grid_constant__ TexAdamBatch P, JobState* advance) {
+    __shared__ float4 s[THREADS];
     const TexAdam& A = P.a[blockIdx.x];
-    if (!A.js->status) mip_top<true>(A.t, s);
+    if (!A.js->status) mip_top<true, THREADS>(A.t, s);
     if (!advance) return;
     __syncthreads();  // every thread has read the status
     if (threadIdx.x == 0 && last_block(advance, TICKET_TEX, gridDim.x)) advance_job(advance);
@@ -694,7 +698,10 @@ cudaError_t adam_textures_tiled(std::vector<TexAdam>& list, cudaStream_t st, uin
         P.extra_tx = extra_tx;
         int blocks = std::min(tiles, std::max(1, sms * ADMS_ADAM_GRID_PCT / 100));
         k_adam_tex_stream<<<blocks, ADMS_ADAM_THREADS, sizeof(AdamSmem), st>>>(P, tiles);
-        k_adam_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P, advance);
+        bool small = true;
+        for (int i = 0; i < P.n; ++i) small = small && mip_top_small(P.a[i].t);
+        if (small) k_adam_mip_top<256><<<P.n, 256, 0, st>>>(P, advance);
+        else k_adam_mip_top<1024><<<P.n, 1024, 0, st>>>(P, advance);
         count_launches(2);
         cudaError_t e = cudaGetLastError();
         if (e) return e;
@@ -902,9 +909,10 @@ __global__ void __launch_bounds__(256) k_mip_tiles(const __grid_constant__ MipBa
     if (tid == 0) tex[t.off[5] + by * (t.w0 >> 5) + bx] = quad_mean(l4, a1, a2, a3);
 }
 
-__global__ void __launch_bounds__(ADMS_MIP_TOP_THREADS) k_mip_top(const __grid_constant__ MipBatch P) {
-    __shared__ float4 s[ADMS_MIP_TOP_THREADS];
-    mip_top<false>(P.t[blockIdx.x], s);
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_mip_top(const __grid_constant__ MipBatch P) {
+    __shared__ float4 s[THREADS];
+    mip_top<false, THREADS>(P.t[blockIdx.x], s);
 }
 
 cudaError_t mip_build(const TexDev* ts, int n, cudaStream_t st) {
@@ -932,7 +940,10 @@ cudaError_t mip_build(const TexDev* ts, int n, cudaStream_t st) {
         k_mip_tiles<<<tiles, 256, 0, st>>>(P);
         count_launches(1);
         if (top > 0) {
-            k_mip_top<<<P.n, ADMS_MIP_TOP_THREADS, 0, st>>>(P);
+            bool small = true;
+            for (int i = 0; i < P.n; ++i) small = small && mip_top_small(P.t[i]);
+            if (small) k_mip_top<256><<<P.n, 256, 0, st>>>(P);
+            else k_mip_top<1024><<<P.n, 1024, 0, st>>>(P);
             count_launches(1);
         }
     }
