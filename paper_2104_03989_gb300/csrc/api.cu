@@ -1842,28 +1842,26 @@ adms_status adms_backward(adms_ctx* ctx, const adms_job* jobs, int32_t n_jobs, i
     return ADMS_OK;
 }
 
-// The step in launches of their own for schedules, positions and step counters, for two cases.
-// repeated: the list names a job more than once. Its entries share the job's state, moments and
-// counters, so each entry's launches follow the one before (rows of one launch, as below, would
-// update them at once): all schedules first, then the flat latents, the textures, the counters.
-// recorded: a graph is being recorded. Its launches cost the host nothing at replay, and the flat
-// latents' step, forked from the context's stream, runs beside the textures' instead of before it.
-// Three graphs of one view of 150x150 and 20000 triangles replayed in turn on streams of their own:
-// 55.1 us a step with maps of 512x512 (61.4 in the direct form below), 73.0 with three sizes (79.6);
-// of the plain step (8 views of 512x512), 389 us (394).
-static adms_status step_apart(adms_ctx* ctx, const std::vector<Job*>& js, bool repeated, bool recorded) {
+// The step in launches of their own for schedules, positions and step counters, entry by entry of
+// the list, for two cases.
+// A list that names a job more than once: its entries share the job's state, moments and counters,
+// so each entry's launches follow the one before (rows of one launch, as below, would update them
+// at once): all schedules first, then the flat latents, the textures, the counters.
+// A single job's graph being recorded (fork): its launches cost the host nothing at replay, and the
+// flat latents' step, forked from the context's stream, runs beside the textures' instead of before
+// it. Three graphs of one view of 150x150 and 20000 triangles replayed in turn on streams of their
+// own: 55.1 us a step with maps of 512x512 (61.4 in the direct form below), 73.0 with three sizes
+// (79.6); of the plain step (8 views of 512x512), 389 us (394). Several jobs share the direct form's
+// launches, recorded or not: 20 small jobs 172 us a step, 244 in this form.
+static adms_status step_apart(adms_ctx* ctx, const std::vector<Job*>& js, bool fork) {
     cudaStream_t st = ctx->stream, bs = st;
-    std::vector<SchedArgs> sched;
-    std::vector<JobState*> sts;
     for (Job* jp : js) {
         Job& j = *jp;
         if (j.opt.optimize_pos && !j.lap_valid) CK(TIMED(ST_LAPLACIAN, laplacian_forward(lap_args(j), st)));
-        sched.push_back(SchedArgs{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV});
-        sts.push_back(j.st);
+        SchedArgs sa{j.st, j.opt.lr0, j.opt.lambda0, j.opt.optimize_pos, j.LV};
+        CK(TIMED(ST_SMALL, schedule_step(&sa, 1, st)));
     }
-    const int n = (int)js.size(), at_once = repeated ? 1 : n;  // jobs a launch
-    for (int k = 0; k < n; k += at_once) CK(TIMED(ST_SMALL, schedule_step(sched.data() + k, at_once, st)));
-    if (recorded) {
+    if (fork) {
         cudaError_t fe;
         bs = fork_branch(ctx, fe);
         CK(fe);
@@ -1883,15 +1881,13 @@ static adms_status step_apart(adms_ctx* ctx, const std::vector<Job*>& js, bool r
             CK(TIMED(ST_ADAM, adam_flat(j.disp, j.g_disp, j.m_disp, j.v_disp, (long long)j.dh * j.dw, j.st, bs)));
         j.frame_valid = false;
         j.lap_valid = false;
+        j.tex_pending = ctx->pipeline;
     }
-    if (ctx->pipeline) {
-        for (Job* jp : js) jp->tex_pending = true;
-        return ADMS_OK;
-    }
-    for (int k = 0; k < n; k += at_once)
-        if (adms_status s = texture_adams(ctx, {js.begin() + k, js.begin() + k + at_once}, st, nullptr)) return s;
-    if (recorded) CK(join_branch(ctx));
-    for (int k = 0; k < n; k += at_once) CK(TIMED(ST_SMALL, advance_step(sts.data() + k, at_once, st)));
+    if (ctx->pipeline) return ADMS_OK;
+    for (Job* jp : js)
+        if (adms_status s = texture_adams(ctx, {jp}, st, nullptr)) return s;
+    if (fork) CK(join_branch(ctx));
+    for (Job* jp : js) CK(TIMED(ST_SMALL, advance_step(&jp->st, 1, st)));
     return ADMS_OK;
 }
 
@@ -1914,8 +1910,8 @@ adms_status adms_optimizer_step(adms_ctx* ctx, const adms_job* jobs, int32_t n_j
         std::sort(sorted.begin(), sorted.end());
         repeated = std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end();
     }
-    bool recorded = !ctx->pipeline && capture_id(ctx) != 0;
-    if (repeated || recorded) return step_apart(ctx, js, repeated, recorded);
+    bool recorded = n_jobs == 1 && !ctx->pipeline && capture_id(ctx) != 0;
+    if (repeated || recorded) return step_apart(ctx, js, recorded);
     // the schedules (after the Laplacian when no forward computed it for these positions), with
     // the positions' step where they are optimized; then skin weights and displacement, if
     // any, on a branch beside the textures; every job's tiled textures in one launch; then,
