@@ -1,6 +1,6 @@
-"""Maps of equal, partly equal, different and one-texel sizes: the combinations take different forms
-in the shading kernels (all taps shared, those of the last two maps shared, none) and in their
-adjoint (all taps shared or none). Noise maps against the float64 oracle; maps of
+"""Maps of equal, partly equal, different and one-texel sizes: each combination has a form of
+its own in the shading kernels and their adjoint (all taps shared, those of the last two maps
+shared, none, none for a map of one texel). Noise maps against the float64 oracle; maps of
 one value, whose size cannot matter, against each other, opaque and in peeled layers."""
 
 import dataclasses
